@@ -617,12 +617,15 @@ void fas_down64(mg_hierarchy* H, const Eq& e, int l) {
     const double* f[3] = {fptr(H, e, l, 0), fptr(H, e, l, 1), fptr(H, e, l, 2)};
     launch_residual_vec(v, L.u, f, L.r, (unsigned long long*)nullptr, 0, H->st);
   }
+  RestrictFields<double> rf{};
   for (int c = 0; c < e.ncomp; ++c) {
-    const double* a[4] = {L.u[c], L.r[c], nullptr, nullptr};
-    double* b[4] = {C.u[c], C.f[c], nullptr, nullptr};
-    double* cp[3] = {C.uh[c], nullptr, nullptr};
-    launch_restrict(v, vc, 2, a, b, cp, H->st);
+    rf.a[c] = L.u[c];
+    rf.b[c] = C.u[c];
+    rf.copy[c] = C.uh[c];
+    rf.a[e.ncomp + c] = L.r[c];
+    rf.b[e.ncomp + c] = C.f[c];
   }
+  launch_restrict(v, vc, 2 * e.ncomp, rf, H->st);
   if (e.kind != EQ_VEC) {
     launch_apply_scalar(vc, e.kind, C.u[0], s0ptr(H, e, l + 1), s1ptr(H, e, l + 1), C.f[0], 1, H->st);
   } else {
@@ -723,10 +726,12 @@ void restrict_sources(mg_hierarchy* H, const Eq& e) {
   for (int l = 1; l < H->nlev; ++l) {
     Level& F = H->L[l - 1];
     Level& C = H->L[l];
-    const double* a[4] = {e.kind == EQ_PSI ? F.s0 : F.s1, F.s1, nullptr, nullptr};
-    double* b[4] = {e.kind == EQ_PSI ? C.s0 : C.s1, C.s1, nullptr, nullptr};
-    double* cp[3] = {nullptr, nullptr, nullptr};
-    launch_restrict(F.v64, C.v64, nf, a, b, cp, H->st);
+    RestrictFields<double> rf{};
+    rf.a[0] = e.kind == EQ_PSI ? F.s0 : F.s1;
+    rf.b[0] = e.kind == EQ_PSI ? C.s0 : C.s1;
+    rf.a[1] = F.s1;
+    rf.b[1] = C.s1;
+    launch_restrict(F.v64, C.v64, nf, rf, H->st);
   }
 }
 
@@ -916,10 +921,10 @@ void restrict_k32(mg_hierarchy* H, int from) {
   for (int l = from; l < H->nlev; ++l) {
     Level& F = H->L[l - 1];
     Level& C = H->L[l];
-    const float* a[4] = {F.k32, nullptr, nullptr, nullptr};
-    float* b[4] = {C.k32, nullptr, nullptr, nullptr};
-    float* cp[3] = {nullptr, nullptr, nullptr};
-    launch_restrict<float>(F.v32, C.v32, 1, a, b, cp, H->st);
+    RestrictFields<float> rf{};
+    rf.a[0] = F.k32;
+    rf.b[0] = C.k32;
+    launch_restrict<float>(F.v32, C.v32, 1, rf, H->st);
   }
 }
 
@@ -936,10 +941,10 @@ void fmg32(mg_hierarchy* H, const Eq& e) {
     auto v = with_bc(L.v32, e.bc);
     auto vc = with_bc(C.v32, e.bc);
     for (int c = 0; c < e.ncomp; ++c) {
-      const float* a[4] = {L.f32[c], nullptr, nullptr, nullptr};
-      float* b[4] = {C.f32[c], nullptr, nullptr, nullptr};
-      float* cp[3] = {nullptr, nullptr, nullptr};
-      launch_restrict<float>(v, vc, 1, a, b, cp, H->st);
+      RestrictFields<float> rf{};
+      rf.a[0] = L.f32[c];
+      rf.b[0] = C.f32[c];
+      launch_restrict<float>(v, vc, 1, rf, H->st);
     }
   }
   for (int c = 0; c < e.ncomp; ++c) cudaMemsetAsync(H->L[lb].e[c], 0, sizeof(float) * H->L[lb].ng, H->st);
@@ -1203,7 +1208,11 @@ int ensure_ghost_push(mg_hierarchy* H) {
     if (ce != cudaSuccess) break;
     const int n0 = v.n0, n1 = v.n1, n2 = v.three ? v.n2 : 1;
     const long ncell = H->L[l].ng;  // cells of the level array, ghosts and padding included
-    const int nb = push_blocks(v);
+    GhostPush shape;
+    push_shape(v, H->d.precision != MG_MIXED, &shape);
+    for (int c = 0; c < 3; ++c)
+      for (int colour = 0; colour < 2; ++colour) H->L[l].push[c][colour] = shape;
+    const int nb = push_blocks(v, shape);
     auto interior = [&](int i, int j, int k) { return i >= 0 && i < n0 && j >= 0 && j < n1 && k >= 0 && k < n2; };
     for (int c = 0; c < 3; ++c) {
       const int* G = gc.data() + 8 * c * ng;
@@ -1217,9 +1226,9 @@ int ensure_ghost_push(mg_hierarchy* H) {
           ok = false;
           break;
         }
-        push_slot(v, o[3], o[4], o[5], &blk[g], &slot[g]);
+        push_slot(v, shape, o[3], o[4], o[5], &blk[g], &slot[g]);
         col[g] = (o[3] + o[4] + o[5]) & 1;
-        if (blk[g] < 0 || blk[g] >= nb || slot[g] < 0 || slot[g] >= 256 * vec_cells_per_thread(v)) ok = false;
+        if (blk[g] < 0 || blk[g] >= nb || slot[g] < 0 || slot[g] >= 256 * shape.nk) ok = false;
         // face neighbours of the ghost updated in the same pass as its source
         for (int d = 0; d < (v.three ? 3 : 2) && ok; ++d)
           for (int s = -1; s <= 1 && ok; s += 2) {
@@ -1227,7 +1236,7 @@ int ensure_ghost_push(mg_hierarchy* H) {
             if (!interior(r[0], r[1], r[2]) || ((r[0] + r[1] + r[2]) & 1) != col[g]) continue;
             if (r[0] == o[3] && r[1] == o[4] && r[2] == o[5]) continue;
             int rb, rt;
-            push_slot(v, r[0], r[1], r[2], &rb, &rt);
+            push_slot(v, shape, r[0], r[1], r[2], &rb, &rt);
             if (rb != blk[g]) ok = false;
           }
       }
@@ -2909,10 +2918,10 @@ int mg_restrict(mg_hierarchy* H, const double* fine, double* coarse) {
   Level& F = H->L[0];
   Level& C = H->L[1];
   copy_in(H, fine, F.r[0]);
-  const double* a[4] = {F.r[0], nullptr, nullptr, nullptr};
-  double* b[4] = {C.r[0], nullptr, nullptr, nullptr};
-  double* cp[3] = {nullptr, nullptr, nullptr};
-  launch_restrict(F.v64, C.v64, 1, a, b, cp, H->st);
+  RestrictFields<double> rf{};
+  rf.a[0] = F.r[0];
+  rf.b[0] = C.r[0];
+  launch_restrict(F.v64, C.v64, 1, rf, H->st);
   launch_copy_out<double, double>(C.v64, C.r[0], coarse, 0.0, H->st);
   CK(cudaStreamSynchronize(H->st));
   CK(cudaGetLastError());

@@ -147,20 +147,17 @@ inline bool fused_sweep_applies(const LevelView<T>& L) {
 struct GhostPush {
   const int* off = nullptr;
   const int2* ent = nullptr;
+  int threads = 256, nk = 1;  // threads per block, cells per thread of the pass the table was built for
 };
 template <typename T>
 void launch_smooth_vec(const LevelView<T>& L, T* V[3], const T* f, int comp, int colour, cudaStream_t st,
                        GhostPush gp = GhostPush{});
-// Block count of a pass with a ghost-push table, and the block of that pass
-// which updates cell (i, j, k) with the cell's slot in its new values.
-template <typename T>
-int push_blocks(const LevelView<T>& L);
-// Cells a thread of the vector colour pass updates when it pushes ghosts
-// (2 on 3D levels of 2^19 cells and more, whose pass then fits one wave).
-template <typename T>
-int vec_cells_per_thread(const LevelView<T>& L);
-template <typename T>
-void push_slot(const LevelView<T>& L, int i, int j, int k, int* block, int* slot);
+// Launch shape of a level's passes with a ghost-push table (FP64 or FP32
+// smoothing), its block count, and the block of that pass which updates cell
+// (i, j, k) with the cell's slot in its new values.
+void push_shape(const LevelView<double>& L, bool fp64, GhostPush* gp);
+int push_blocks(const LevelView<double>& L, const GhostPush& gp);
+void push_slot(const LevelView<double>& L, const GhostPush& gp, int i, int j, int k, int* block, int* slot);
 // Source of every ghost of vector component comp, in the enumeration of
 // the ghost fill: gc[8 g ..] = ghost i, j, k, source i, j, k, ghost index,
 // source index; fac[g] = the product of the boundary factors.
@@ -182,9 +179,17 @@ void launch_apply_scalar(const LevelView<T>& L, int kind, const T* u, const T* s
                          int add, cudaStream_t st);
 template <typename T>
 void launch_apply_vec(const LevelView<T>& L, T* const V[3], T* const out[3], int add, cudaStream_t st);
+// Fields of one restriction launch (nf = 1, 2 or 6): a[m] restricted into
+// b[m], a copy of b[0 .. 2] into copy[0 .. 2] when non-null.
 template <typename T>
-void launch_restrict(const LevelView<T>& F, const LevelView<T>& C, int nf, const T* const a[4],
-                     T* const b[4], T* const copy[3], cudaStream_t st);
+struct RestrictFields {
+  const T* a[6];
+  T* b[6];
+  T* copy[3];
+};
+template <typename T>
+void launch_restrict(const LevelView<T>& F, const LevelView<T>& C, int nf, const RestrictFields<T>& P,
+                     cudaStream_t st);
 template <typename T>
 void launch_prolong(const LevelView<T>& F, const LevelView<T>& C, T* u, const T* uH, const T* uhH, int comp,
                     cudaStream_t st);

@@ -19,6 +19,58 @@ unsigned long long launch_count() { return g_launches.load(std::memory_order_rel
 static inline dim3 block_for(int three) { return three ? dim3(32, 4, 2) : dim3(32, 8, 1); }
 static inline unsigned cdiv(long a, long b) { return (unsigned)((a + b - 1) / b); }
 
+static int g_sms = 0;  // multiprocessors of the device, set when a hierarchy is created
+static inline int sm_count() { return g_sms > 0 ? g_sms : 152; }
+
+// Threads per block of a pass with one thread per item over n items: the
+// smallest of lo .. 256 that needs at most 8 blocks per multiprocessor.  The
+// FP64 pipe takes ~16 cycles per warp instruction, so a level of a few
+// thousand cells in 256-thread blocks keeps a few SMs busy for microseconds
+// while the others idle: the FP64 vector colour pass took ~11 us on every
+// level of a 64x32x32 hierarchy, down to 128 cells, before the blocks were
+// made small enough to spread over the device.
+static inline unsigned spread_threads(long n, unsigned lo) {
+  unsigned t = lo;
+  while (t < 256 && n > 8L * sm_count() * t) t *= 2;
+  return t;
+}
+// Block of at most t threads (a power of two) that tiles nx x ny x nz items
+// (powers of two) without idle threads, z planes deep at least: the FP64
+// pipe spends a whole instruction slot on a warp with idle lanes too.
+static inline dim3 fit_block(int nx, int ny, int nz, unsigned t, unsigned z = 1) {
+  dim3 b(1, 1, z);
+  t = t > z ? t / z : 1;
+  b.x = std::min<unsigned>({(unsigned)nx, 32u, t});
+  t /= b.x;
+  b.y = std::min<unsigned>((unsigned)ny, t);
+  t /= b.y;
+  b.z *= std::max<unsigned>(1u, std::min<unsigned>((unsigned)nz / z, t));
+  return b;
+}
+template <typename T>
+static inline long ncells(const LevelView<T>& L) {
+  return (long)L.n0 * L.n1 * L.n2;
+}
+// Blocks of a pass over all cells, and of one over the cells of one colour.
+// FP32 passes are not bound by their pipe: larger blocks.
+template <typename T>
+static inline dim3 cells_block(const LevelView<T>& L) {
+  return fit_block(L.n0, L.n1, L.n2, spread_threads(ncells(L), sizeof(T) == 8 ? 32 : 128));
+}
+template <typename T>
+static inline dim3 colour_block(const LevelView<T>& L) {
+  return fit_block(L.n0 / 2, L.n1, L.n2, spread_threads(ncells(L) / 2, sizeof(T) == 8 ? 32 : 128));
+}
+// Passes that end in block maxima and atomics: at most 512 blocks until
+// they have 256 threads.
+template <typename T>
+static inline dim3 norm_block(const LevelView<T>& L, long per_thread, unsigned z = 1) {
+  const long n = ncells(L) / per_thread;
+  unsigned t = 32;
+  while (t < 256 && n > 512L * t) t *= 2;
+  return fit_block(L.n0, L.n1, std::max(1, (int)(L.n2 / per_thread)), t, z);
+}
+
 // ------------------------------------------------------------ smoothers
 
 // One colour of the red-black sweep: cells with (i + j + k) % 2 == colour.
@@ -54,6 +106,7 @@ __global__ void k_smooth_vec(LevelView<T> L, T* __restrict__ A, T* __restrict__ 
     vec_update<T, G>(L, A, B, C, f, comp, i, j, k);
     return;
   }
+  // nv slot of a thread's w-th cell: its number in the block + 256 w
   __shared__ T nv[NK * 256];
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nthr = blockDim.x * blockDim.y * blockDim.z;
@@ -67,7 +120,6 @@ __global__ void k_smooth_vec(LevelView<T> L, T* __restrict__ A, T* __restrict__ 
   const int k0 = L.three ? (int)blockIdx.z + (int)threadIdx.z * (L.n2 >> 1) : 0;
   T* V = comp == 0 ? A : (comp == 1 ? B : C);
   if (2 * t < L.n0 && j < L.n1 && k0 < L.n2) {
-    // nv slot of the w-th cell: tid + 256 w
 #pragma unroll
     for (int w = 0; w < NK; ++w) {
       const int k = k0 + w * (L.n2 >> 2);
@@ -670,13 +722,16 @@ __global__ void k_fill_ghosts3(LevelView<T> L, T* __restrict__ u0, T* __restrict
 // max |r| (slot 0) and, when weighted, max |w r| (slot 1), max |w S| (slot 2).
 // A thread walks RES_KZ planes (k strided by blockDim.z) so that the block
 // reduction of the norms is paid once per RES_KZ cells.
+// On levels below RES_KZ_CELLS a thread takes one cell: 64x32x32 in four
+// planes per thread is 64 blocks, less than half of the SMs (19 us instead
+// of 9 for eq. psi in FP64).
 constexpr int RES_KZ = 4;
+constexpr long RES_KZ_CELLS = 1L << 21;
 // The vector residual carries three components' worth of FP64 work per
 // cell: one plane per thread and at most 128 registers (two blocks per SM)
 // spread it over more blocks.
-constexpr int RES_KZ_VEC = 1;
 
-template <typename T, int G, int KIND>
+template <typename T, int G, int KIND, int KZ>
 __global__ void k_residual_scalar(LevelView<T> L, const T* __restrict__ u, const T* __restrict__ f,
                                   const T* __restrict__ s0, const T* __restrict__ s1, T* __restrict__ r,
                                   float* __restrict__ r32, float* __restrict__ k32, unsigned long long* red,
@@ -688,8 +743,8 @@ __global__ void k_residual_scalar(LevelView<T> L, const T* __restrict__ u, const
   if (i < L.n0 && j < L.n1) {
     const double w = weighted ? (double)norm_weight(L, i, j) : 1.0;
 #pragma unroll
-    for (int it = 0; it < RES_KZ; ++it) {
-      const int k = (blockIdx.z * RES_KZ + it) * blockDim.z + threadIdx.z;
+    for (int it = 0; it < KZ; ++it) {
+      const int k = (blockIdx.z * KZ + it) * blockDim.z + threadIdx.z;
       if (k >= L.n2) continue;
       const long p = L.idx(i, j, k);
       T Sv, kp;
@@ -725,10 +780,8 @@ __global__ void __launch_bounds__(256, 2) k_residual_vec(LevelView<T> L, const T
     const T* fs[3] = {f0, f1, f2};
     T* rs[3] = {r0, r1, r2};
     float* qs[3] = {q0, q1, q2};
-#pragma unroll 1
-    for (int it = 0; it < RES_KZ_VEC; ++it) {
-      const int k = (blockIdx.z * RES_KZ_VEC + it) * blockDim.z + threadIdx.z;
-      if (k >= L.n2) continue;
+    const int k = blockIdx.z * blockDim.z + threadIdx.z;
+    if (k < L.n2) {
       const long p = L.idx(i, j, k);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -850,22 +903,24 @@ __global__ void k_apply_vec(LevelView<T> L, const T* __restrict__ A, const T* __
 
 // Piecewise-constant restriction (Sec. 2.7.3): coarse = volume-weighted mean
 // of the 2^d children (Cartesian: the equal-weight 1/4, 1/8 stencil).
-// Restricts up to 4 fields; copy (if non-null) receives a second copy of
-// field 0 (the FAS u_H kept for the correction).
-template <typename T>
-__global__ void k_restrict(LevelView<T> F, LevelView<T> Cv, int nf, const T* __restrict__ a0,
-                           const T* __restrict__ a1, const T* __restrict__ a2, const T* __restrict__ a3,
-                           T* __restrict__ b0, T* __restrict__ b1, T* __restrict__ b2, T* __restrict__ b3,
-                           T* __restrict__ copy0, T* __restrict__ copy1, T* __restrict__ copy2) {
+// Restricts NF fields in one launch; copies of the first three (if
+// non-null) keep the FAS u_H for the correction.
+template <typename T, int NF>
+__global__ void k_restrict(LevelView<T> F, LevelView<T> Cv, const __grid_constant__ RestrictFields<T> P) {
   pdl_entry();
   const int I = blockIdx.x * blockDim.x + threadIdx.x;
   const int J = blockIdx.y * blockDim.y + threadIdx.y;
   const int K = blockIdx.z * blockDim.z + threadIdx.z;
   if (I >= Cv.n0 || J >= Cv.n1 || K >= Cv.n2) return;
-  const T* as[4] = {a0, a1, a2, a3};
-  T* bs[4] = {b0, b1, b2, b3};
-  T* cs[3] = {copy0, copy1, copy2};
-  restrict_cell(F, Cv, nf, as, bs, cs, I, J, K);
+  const T* as[NF];
+  T* bs[NF];
+#pragma unroll
+  for (int m = 0; m < NF; ++m) {
+    as[m] = P.a[m];
+    bs[m] = P.b[m];
+  }
+  T* const cs[3] = {P.copy[0], P.copy[1], P.copy[2]};
+  restrict_cell<T, NF>(F, Cv, NF, as, bs, cs, I, J, K);
 }
 
 // Kwak prolongation (Sec. 2.7.3, Fig. kwak) of e = uH - uhH, added into u.
@@ -1208,7 +1263,7 @@ template <typename T>
 void launch_smooth_scalar(const LevelView<T>& L, int kind, T* u, const T* f, const T* s0, const T* s1,
                           int colour, cudaStream_t st) {
   count_launch();
-  dim3 b = block_for(L.three), g = grid_colour(L, b);
+  const dim3 b = colour_block(L), g = grid_colour(L, b);
   GMG_GEOM_DISPATCH(L.geom, if (kind == EQ_PSI) launch_k(k_smooth_scalar<T, GG, EQ_PSI>, g, b, 0, st, L, u, f, s0, s1, colour);
                     else launch_k(k_smooth_scalar<T, GG, EQ_LIN>, g, b, 0, st, L, u, f, s0, s1, colour));
 }
@@ -1227,8 +1282,6 @@ int fused_sweep_tx(const LevelView<T>& L) {
 
 // Blocks of k_sweep_rb resident on the whole device, [geometry][TX == 128]
 // [with c], set when a hierarchy is created (outside any stream capture).
-static int g_fused_sms = 0;
-
 template <typename T>
 struct FusedCapacity {
   static int blocks[3][2][2];
@@ -1263,7 +1316,7 @@ void init_fused_sweep_attributes() {
   int d = 0, sms = 0;
   cudaGetDevice(&d);
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess || sms < 1) sms = 1;
-  g_fused_sms = sms;
+  g_sms = sms;
   set_fused_capacity_g<T, CART>(sms);
   set_fused_capacity_g<T, CYL>(sms);
   set_fused_capacity_g<T, SPH>(sms);
@@ -1280,7 +1333,7 @@ template <typename T>
 int fused_sweep_chunk(const LevelView<T>& L, int tx, bool with_c) {
   const long cols = (long)cdiv(L.n0, tx) * cdiv(L.n1, tx == 128 ? RbShape<128>::TY : RbShape<64>::TY);
   const long cap = FusedCapacity<T>::blocks[L.geom][tx == 128][with_c];
-  const long sms = g_fused_sms > 0 ? g_fused_sms : 1;
+  const long sms = sm_count();
   int best = 8;
   long best_cost = -1;
   for (int zc = 4; zc <= 64; ++zc) {
@@ -1380,12 +1433,23 @@ void launch_fill_ghosts(const LevelView<T>& L, T* u, int comp, cudaStream_t st) 
   launch_k(k_fill_ghosts<T>, grid_flat(n, 256), 256, 0, st, L, u, comp);
 }
 
+// Block of a colour pass with a ghost-push table: in 3D two threads deep
+// (planes n2 / 2 apart).
+template <typename T>
+static dim3 push_block(const LevelView<T>& L, int threads) {
+  if (!L.three) return fit_block(L.n0 / 2, L.n1, 1, threads);
+  dim3 b = fit_block(L.n0 / 2, L.n1, 1, std::max(threads / 2, 1));
+  b.z = 2;
+  return b;
+}
+
 template <typename T>
 void launch_smooth_vec(const LevelView<T>& L, T* V[3], const T* f, int comp, int colour, cudaStream_t st,
                        GhostPush gp) {
   count_launch();
-  dim3 b = block_for(L.three), g = grid_colour(L, b);
-  const int nk = gp.off ? vec_cells_per_thread(L) : 1;
+  const int nk = gp.off ? gp.nk : 1;
+  const dim3 b = gp.off ? push_block(L, gp.threads) : colour_block(L);
+  dim3 g = grid_colour(L, b);
   if (gp.off && L.three) g.z = (unsigned)(L.n2 / (2 * nk));  // b.z = 2: planes k and k + n2 / 2 (and n2 / 4 up)
   if (nk == 2) {
     GMG_GEOM_DISPATCH(L.geom,
@@ -1396,25 +1460,26 @@ void launch_smooth_vec(const LevelView<T>& L, T* V[3], const T* f, int comp, int
   }
 }
 
-template <typename T>
-int vec_cells_per_thread(const LevelView<T>& L) {
-  return (L.three && L.n2 % 4 == 0 && (long)L.n0 * L.n1 * L.n2 >= (1L << 19)) ? 2 : 1;
+// Launch shape of a level's colour passes with a ghost-push table: FP64
+// passes spread over the device (spread_threads), FP32 ones (mixed) take 256
+// threads and, from 2^19 cells on, two cells per thread.
+void push_shape(const LevelView<double>& L, bool fp64, GhostPush* gp) {
+  gp->nk = (!fp64 && L.three && L.n2 % 4 == 0 && ncells(L) >= (1L << 19)) ? 2 : 1;
+  gp->threads = fp64 ? (int)spread_threads(ncells(L) / 2, 32) : 256;
 }
 
-template <typename T>
-int push_blocks(const LevelView<T>& L) {
-  const dim3 b = block_for(L.three), g = grid_colour(L, b);
-  return (int)(g.x * g.y * (L.three ? L.n2 / (2 * vec_cells_per_thread(L)) : 1));
+int push_blocks(const LevelView<double>& L, const GhostPush& gp) {
+  const dim3 b = push_block(L, gp.threads), g = grid_colour(L, b);
+  return (int)(g.x * g.y * (L.three ? L.n2 / (2 * gp.nk) : 1));
 }
 
 // The block of a pass with a ghost-push table that updates cell (i, j, k),
 // and the cell's slot in the block's shared new values: with NK cells per
 // thread, plane k = bz + (2 tz + w) q (q = n2 / (2 NK)) is thread z = tz's
 // w-th cell, slot = thread + 256 w.
-template <typename T>
-void push_slot(const LevelView<T>& L, int i, int j, int k, int* block, int* slot) {
-  const dim3 b = block_for(L.three), g = grid_colour(L, b);
-  const int t = i >> 1, nk = vec_cells_per_thread(L);
+void push_slot(const LevelView<double>& L, const GhostPush& gp, int i, int j, int k, int* block, int* slot) {
+  const dim3 b = push_block(L, gp.threads), g = grid_colour(L, b);
+  const int t = i >> 1, nk = gp.nk;
   const int q = L.three ? L.n2 / (2 * nk) : 1;
   const int bz = L.three ? k % q : 0, r = L.three ? k / q : 0;  // r = nk tz + w
   const int tz = r / nk, w = r % nk;
@@ -1454,25 +1519,30 @@ void launch_residual_scalar(const LevelView<T>& L, int kind, const T* u, const T
                             const T* s1, T* r, unsigned long long* red, int weighted, cudaStream_t st, float* r32,
                             float* k32) {
   count_launch();
-  dim3 b = block_for(L.three), g = grid_cells(L, b);
-  g.z = cdiv(L.n2, (long)b.z * RES_KZ);
-  GMG_GEOM_DISPATCH(L.geom, if (kind == EQ_PSI) launch_k(k_residual_scalar<T, GG, EQ_PSI>, g, b, 0, st, L, u, f, s0, s1, r, r32, k32, red, weighted);
-                    else launch_k(k_residual_scalar<T, GG, EQ_LIN>, g, b, 0, st, L, u, f, s0, s1, r, r32, nullptr, red, weighted));
+  if (L.three && ncells(L) >= RES_KZ_CELLS) {
+    dim3 b = block_for(L.three), g = grid_cells(L, b);
+    g.z = cdiv(L.n2, (long)b.z * RES_KZ);
+    GMG_GEOM_DISPATCH(L.geom, if (kind == EQ_PSI) launch_k(k_residual_scalar<T, GG, EQ_PSI, RES_KZ>, g, b, 0, st, L, u, f, s0, s1, r, r32, k32, red, weighted);
+                      else launch_k(k_residual_scalar<T, GG, EQ_LIN, RES_KZ>, g, b, 0, st, L, u, f, s0, s1, r, r32, nullptr, red, weighted));
+    return;
+  }
+  const dim3 b = red ? norm_block(L, 1) : cells_block(L), g = grid_cells(L, b);
+  GMG_GEOM_DISPATCH(L.geom, if (kind == EQ_PSI) launch_k(k_residual_scalar<T, GG, EQ_PSI, 1>, g, b, 0, st, L, u, f, s0, s1, r, r32, k32, red, weighted);
+                    else launch_k(k_residual_scalar<T, GG, EQ_LIN, 1>, g, b, 0, st, L, u, f, s0, s1, r, r32, nullptr, red, weighted));
 }
 
 template <typename T>
 void launch_residual_vec(const LevelView<T>& L, T* const V[3], const T* const f[3], T* const r[3],
                          unsigned long long* red, int weighted, cudaStream_t st, float* const r32[3]) {
   count_launch();
-  dim3 b = block_for(L.three), g = grid_cells(L, b);
-  g.z = cdiv(L.n2, (long)b.z * RES_KZ_VEC);
+  const dim3 b = red ? norm_block(L, 1) : cells_block(L), g = grid_cells(L, b);
   float* q[3] = {nullptr, nullptr, nullptr};
   if (r32)
     for (int c = 0; c < 3; ++c) q[c] = r32[c];
   if constexpr (sizeof(T) == 8) {
     if (L.geom == SPH && L.vc && L.mixed == 0) {
-      const dim3 bs(32, L.three ? 2 : 8, L.three ? 4 : 1);
-      const dim3 gs(cdiv(L.n0, 32), cdiv(L.n1, bs.y), cdiv(L.n2, bs.z));
+      const dim3 bs = norm_block(L, 1, L.three && L.n2 >= 4 ? 4 : 1);
+      const dim3 gs(cdiv(L.n0, bs.x), cdiv(L.n1, bs.y), cdiv(L.n2, bs.z));
       launch_k(k_residual_vec_sph, gs, bs, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], r[0], r[1], r[2], q[0],
                q[1], q[2], red, weighted);
       return;
@@ -1485,7 +1555,7 @@ template <typename T>
 void launch_apply_scalar(const LevelView<T>& L, int kind, const T* u, const T* s0, const T* s1, T* out, int add,
                          cudaStream_t st) {
   count_launch();
-  dim3 b = block_for(L.three), g = grid_cells(L, b);
+  const dim3 b = cells_block(L), g = grid_cells(L, b);
   GMG_GEOM_DISPATCH(L.geom, if (kind == EQ_PSI) launch_k(k_apply_scalar<T, GG, EQ_PSI>, g, b, 0, st, L, u, s0, s1, out, add);
                     else launch_k(k_apply_scalar<T, GG, EQ_LIN>, g, b, 0, st, L, u, s0, s1, out, add));
 }
@@ -1493,17 +1563,21 @@ void launch_apply_scalar(const LevelView<T>& L, int kind, const T* u, const T* s
 template <typename T>
 void launch_apply_vec(const LevelView<T>& L, T* const V[3], T* const out[3], int add, cudaStream_t st) {
   count_launch();
-  dim3 b = block_for(L.three), g = grid_cells(L, b);
+  const dim3 b = cells_block(L), g = grid_cells(L, b);
   GMG_GEOM_DISPATCH(L.geom, launch_k(k_apply_vec<T, GG>, g, b, 0, st, L, V[0], V[1], V[2], out[0], out[1], out[2], add));
 }
 
 template <typename T>
-void launch_restrict(const LevelView<T>& F, const LevelView<T>& C, int nf, const T* const a[4], T* const b[4],
-                     T* const copy[3], cudaStream_t st) {
+void launch_restrict(const LevelView<T>& F, const LevelView<T>& C, int nf, const RestrictFields<T>& P,
+                     cudaStream_t st) {
   count_launch();
-  dim3 bl = block_for(C.three), g = grid_cells(C, bl);
-  launch_k(k_restrict<T>, g, bl, 0, st, F, C, nf, a[0], a[1], a[2], a[3], b[0], b[1], b[2], b[3], copy[0], copy[1],
-                                   copy[2]);
+  const dim3 b = cells_block(C), g = grid_cells(C, b);
+  if (nf == 1)
+    launch_k(k_restrict<T, 1>, g, b, 0, st, F, C, P);
+  else if (nf == 2)
+    launch_k(k_restrict<T, 2>, g, b, 0, st, F, C, P);
+  else
+    launch_k(k_restrict<T, 6>, g, b, 0, st, F, C, P);
 }
 
 template <typename T>
@@ -1518,7 +1592,8 @@ template <typename T>
 void launch_prolong3(const LevelView<T>& F, const LevelView<T>& C, T* const u[3], const T* const uH[3],
                      const T* const uhH[3], int ncomp, int vec, cudaStream_t st) {
   count_launch();
-  dim3 b = block_for(F.three), g = grid_cells(F, b);
+  const dim3 b = sizeof(T) == 8 ? cells_block(F) : block_for(F.three);
+  const dim3 g = grid_cells(F, b);
   CPtr3<T> hh{};
   if (uhH) hh = CPtr3<T>::of(uhH, ncomp);
   if (ncomp == 1)
@@ -1634,9 +1709,6 @@ void launch_add_correction(const LevelView<double>& L, int ncomp, double* const 
   template void launch_prolong3<T>(const LevelView<T>&, const LevelView<T>&, T* const[3], const T* const[3],  \
                                    const T* const[3], int, int, cudaStream_t);                                 \
   template void launch_smooth_vec<T>(const LevelView<T>&, T* [3], const T*, int, int, cudaStream_t, GhostPush); \
-  template int push_blocks<T>(const LevelView<T>&);                                                            \
-  template int vec_cells_per_thread<T>(const LevelView<T>&);                                                   \
-  template void push_slot<T>(const LevelView<T>&, int, int, int, int*, int*);                                  \
   template void launch_residual_scalar<T>(const LevelView<T>&, int, const T*, const T*, const T*, const T*, T*, \
                                           unsigned long long*, int, cudaStream_t, float*, float*);              \
   template void launch_residual_vec<T>(const LevelView<T>&, T* const[3], const T* const[3], T* const[3],       \
@@ -1644,8 +1716,8 @@ void launch_add_correction(const LevelView<double>& L, int ncomp, double* const 
   template void launch_apply_scalar<T>(const LevelView<T>&, int, const T*, const T*, const T*, T*, int,        \
                                        cudaStream_t);                                                           \
   template void launch_apply_vec<T>(const LevelView<T>&, T* const[3], T* const[3], int, cudaStream_t);         \
-  template void launch_restrict<T>(const LevelView<T>&, const LevelView<T>&, int, const T* const[4],           \
-                                   T* const[4], T* const[3], cudaStream_t);                                     \
+  template void launch_restrict<T>(const LevelView<T>&, const LevelView<T>&, int, const RestrictFields<T>&,      \
+                                   cudaStream_t);                                                               \
   template void launch_prolong<T>(const LevelView<T>&, const LevelView<T>&, T*, const T*, const T*, int,       \
                                   cudaStream_t);                                                                \
   template void launch_coarse_scalar<T>(const LevelView<T>&, int, T*, const T*, const T*, const T*, int,       \

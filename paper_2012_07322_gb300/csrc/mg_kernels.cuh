@@ -231,9 +231,9 @@ __device__ __forceinline__ T vec_residual_cell(const LevelView<T>& L, const T* _
 // Volume-weighted piecewise-constant restriction (Sec. 2.7.3, weights
 // Delta V of the fine cells) of nf fields a[m] into b[m] at coarse cell
 // (I, J, K); copies into cs[m] too when non-null.
-template <typename T>
+template <typename T, int NF = 4>
 __device__ __forceinline__ void restrict_cell(const LevelView<T>& F, const LevelView<T>& Cv, int nf,
-                                              const T* const (&as)[4], T* const (&bs)[4], T* const (&cs)[3],
+                                              const T* const* as, T* const* bs, T* const* cs,
                                               int I, int J, int K) {
   T wi[2], wj[2];
   wi[0] = F.TI(TI_VW, 2 * I);
@@ -248,7 +248,7 @@ __device__ __forceinline__ void restrict_cell(const LevelView<T>& F, const Level
   const T inv = T(1) / wsum;
   const long q = Cv.idx(I, J, K);
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < NF; ++m) {
     if (m >= nf) break;
     T s = T(0);
     for (int dk = 0; dk < nk; ++dk)
