@@ -93,6 +93,10 @@ struct mg_hierarchy {
   int cinv_state[3] = {0, 0, 0};
   double* cmat[3] = {};  // scalar equations: the coarsest operator per boundary rule (same states)
   int cmat_state[3] = {0, 0, 0};
+  // FP64 vector equations: dense rows of the coarsest operator and its
+  // inverted Newton diagonal per boundary rule (same states)
+  double* crow[3] = {};
+  int crow_state[3] = {0, 0, 0};
   double* d_aa_part = nullptr;  // AA_SCRATCH_DOUBLES of device scratch
   // ghost-push tables of the vector colour passes: state 0 not built, 1
   // built, -1 unavailable; one device buffer holds every level's tables
@@ -594,10 +598,18 @@ void coarse64(mg_hierarchy* H, const Eq& e, int l) {
   Level& L = H->L[l];
   auto v = with_bc(L.v64, e.bc);
   if (e.kind != EQ_VEC) {
-    launch_coarse_scalar(v, e.kind, L.u[0], fptr(H, e, l, 0), s0ptr(H, e, l), s1ptr(H, e, l), COARSE_SWEEPS, H->st);
+    if (!launch_coarse_scalar_small(v, e.kind, L.u[0], fptr(H, e, l, 0), s0ptr(H, e, l), s1ptr(H, e, l),
+                                    COARSE_SWEEPS, H->st))
+      launch_coarse_scalar(v, e.kind, L.u[0], fptr(H, e, l, 0), s0ptr(H, e, l), s1ptr(H, e, l), COARSE_SWEEPS,
+                           H->st);
   } else {
     const double* f[3] = {fptr(H, e, l, 0), fptr(H, e, l, 1), fptr(H, e, l, 2)};
-    launch_coarse_vec(v, L.u, f, COARSE_SWEEPS, H->st);
+    const int n = (int)(3 * L.cells());
+    if (H->crow_state[e.bc] == 1)
+      launch_coarse_vec_dense(v, L.u, f, H->crow[e.bc], H->crow[e.bc] + (size_t)(n + 3) * n, n, COARSE_SWEEPS,
+                              H->st);
+    else
+      launch_coarse_vec(v, L.u, f, COARSE_SWEEPS, H->st);
   }
 }
 
@@ -1134,6 +1146,35 @@ int ensure_coarse_inverse(mg_hierarchy* H, int bc) {
   return MG_OK;
 }
 
+// FP64 vector equations: dense rows of the coarsest operator, built once per
+// boundary rule before the first cycle (outside graph capture).  Coarsest
+// levels of more than CV_N unknowns keep the stencil sweeps.
+int ensure_coarse_rows(mg_hierarchy* H, int bc) {
+  if (H->crow_state[bc] != 0) return MG_OK;
+  H->crow_state[bc] = -1;
+  Level& Lc = H->L[H->nlev - 1];
+  const int n = (int)(3 * Lc.cells());
+  if (n > CV_N) return MG_OK;
+  double *scratch = nullptr, *d = nullptr;
+  if (cudaMalloc(&scratch, sizeof(double) * 3 * (size_t)(n + 3) * Lc.ng) != cudaSuccess ||
+      cudaMalloc(&d, sizeof(double) * (size_t)(n + 4) * n) != cudaSuccess) {
+    cudaFree(scratch);
+    cudaFree(d);
+    cudaGetLastError();
+    return MG_OK;
+  }
+  launch_coarse_rows_vec(with_bc(Lc.v64, bc), scratch, d, d + (size_t)(n + 3) * n, n, H->st);
+  const cudaError_t ce = cudaStreamSynchronize(H->st);
+  cudaFree(scratch);
+  if (ce != cudaSuccess) {
+    cudaFree(d);
+    return fail(MG_ERR_CUDA, cudaGetErrorString(ce));
+  }
+  H->crow[bc] = d;
+  H->crow_state[bc] = 1;
+  return MG_OK;
+}
+
 // Mixed precision, scalar equations: the coarsest operator as dense rows
 // (its boundary rule folded in), assembled once per boundary rule before the
 // first cycle (outside graph capture), for the one-block cycle's coarsest
@@ -1482,6 +1523,8 @@ int run_solve_body(mg_hierarchy* H, const Eq& e, mg_solve_report* rep) {
     if (int est = ensure_coarse_inverse(H, e.bc)) return est;
   if (mixed && e.kind != EQ_VEC)
     if (int est = ensure_coarse_matrix(H, e.bc)) return est;
+  if (!mixed && e.kind == EQ_VEC)
+    if (int est = ensure_coarse_rows(H, e.bc)) return est;
   if (e.kind == EQ_VEC && e.bc == MG_BC_DIRICHLET)
     if (int est = ensure_ghost_push(H)) return est;
   if (e.kind == EQ_VEC) fill_all64(H, e, 0);
@@ -2218,6 +2261,8 @@ int mg_destroy_hierarchy(mg_hierarchy* H) {
   for (double* p : H->cinv)
     if (p) cudaFree(p);
   for (double* p : H->cmat)
+    if (p) cudaFree(p);
+  for (double* p : H->crow)
     if (p) cudaFree(p);
   if (H->d_aa_part) cudaFree(H->d_aa_part);
   if (H->batch_mem) cudaFree(H->batch_mem);

@@ -205,6 +205,18 @@ void launch_resid_restrict32(const LevelView<float>& F, const LevelView<float>& 
 template <typename T>
 void launch_coarse_scalar(const LevelView<T>& L, int kind, T* u, const T* f, const T* s0, const T* s1,
                           int max_sweeps, cudaStream_t st);
+// The same FP64 solves on coarsest levels of a few dozen cells (mg_coarse.cu):
+// scalar equations in two warps (false when the level is larger); vector
+// equations from dense rows of the operator (A: n + 3 columns of n, n = 3 x
+// cells at most CV_N, and the inverted Newton diagonal), built once per
+// hierarchy and boundary rule; scratch holds 3 (n + 3) ghosted fields.
+constexpr int CV_N = 192;
+bool launch_coarse_scalar_small(const LevelView<double>& L, int kind, double* u, const double* f, const double* s0,
+                                const double* s1, int max_sweeps, cudaStream_t st);
+void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double* A, double* invD, int n,
+                            cudaStream_t st);
+void launch_coarse_vec_dense(const LevelView<double>& L, double* const V[3], const double* const f[3],
+                             const double* A, const double* invD, int n, int max_sweeps, cudaStream_t st);
 template <typename T>
 void launch_coarse_vec(const LevelView<T>& L, T* V[3], const T* const f[3], int max_sweeps, cudaStream_t st);
 // u -= mean(u) over the interior (the Neumann gauge); the nparts block sums
