@@ -223,12 +223,18 @@ __device__ void bt_restrict_k_all(const Team& T, const BatchItem& I) {
     bt_restrict_k(T, I.bc.lv[q - 1].v, I.bc.lv[q - 1].k32, I.bc.lv[q].v, const_cast<float*>(I.bc.lv[q].k32));
 }
 
+// The one-block cycle, out of line (its registers are not the callers').
+template <int G, bool VEC>
+__device__ __noinline__ void bt_block(const BlockCycle32& P) {
+  bc_run<G, VEC, true>(P);
+}
+
 // One V-cycle of the FP32 correction equation from e = 0 at level 0 (lv[0].e
 // zeroed by the caller): pre-smoothing and residual restriction down to
 // level nl, the one-block cycle from there (rank 0 of a team runs it alone),
 // prolongation and post-smoothing back up.
 template <int G>
-__device__ void bt_vcycle(const Team& T, const BatchItem& I, bool fold, float* sm, double* smd) {
+__device__ void bt_vcycle(const Team& T, const BatchItem& I, bool fold) {
   for (int l = 0; l < I.nl; ++l) {
     bt_smooth<G>(T, I.lv[l], I.nu1);
     bt_resid_restrict<G>(T, I.lv[l], I.lv[l + 1], fold);
@@ -236,7 +242,7 @@ __device__ void bt_vcycle(const Team& T, const BatchItem& I, bool fold, float* s
   if (fold)
     for (int q = 1; q < I.bc.nl; ++q)
       bt_restrict_k(T, I.bc.lv[q - 1].v, I.bc.lv[q - 1].k32, I.bc.lv[q].v, const_cast<float*>(I.bc.lv[q].k32));
-  if (T.rank == 0) bc_run<G, false, true>(I.bc, sm, smd);
+  if (T.rank == 0) bt_block<G, false>(I.bc);
   T.sync();
   for (int l = I.nl - 1; l >= 0; --l) {
     const BatchLevel& F = I.lv[l];
@@ -560,14 +566,13 @@ __device__ void bt_resid_restrict_vec(const Team& T, const BatchLevel& F, const 
 
 // One FP32 correction V-cycle of the vector equation from e = 0 at level 0.
 template <int G>
-__device__ __noinline__ void bt_vcycle_vec(const Team& T, const BatchItem& I, unsigned char* smem_raw) {
+__device__ __noinline__ void bt_vcycle_vec(const Team& T, const BatchItem& I) {
   for (int l = 0; l < I.nlv; ++l) {
     bt_smooth_vec<G>(T, I.lv[l], I.nu1);
     bt_resid_restrict_vec<G>(T, I.lv[l], I.lv[l + 1]);
   }
   if (T.rank == 0)
-    bc_run<G, true, true>(I.bcv, reinterpret_cast<float*>(smem_raw),
-                    reinterpret_cast<double*>(smem_raw + I.bcv.fp64_at));
+    bt_block<G, true>(I.bcv);
   T.sync();
   for (int l = I.nlv - 1; l >= 0; --l) {
     const BatchLevel& F = I.lv[l];
@@ -605,7 +610,7 @@ __device__ void bt_fill_u3(const Team& T, const BatchItem& I) {
 // rank 0's shared memory after a barrier.  Returns the status.
 template <int G, int KIND>
 __device__ __noinline__ int bt_solve(const Team& T, const BatchItem& I, const double* f, const double* s0, const double* s1,
-                        BatchOut& O, int eq, double* hist, float* sm, double* smd, BtShared& S) {
+                        BatchOut& O, int eq, double* hist, BtShared& S) {
   const LevelView<double>& L = I.v64;
   const long n = bt_cells(L), ng = bt_ghosted(L);
   if (KIND == EQ_LIN) {
@@ -646,7 +651,7 @@ __device__ __noinline__ int bt_solve(const Team& T, const BatchItem& I, const do
       for (long q = T.start(); q < ng; q += T.stride()) I.aa[q] = I.u[q];
     for (long q = T.start(); q < ng; q += T.stride()) I.lv[0].e[q] = 0.0f;
     T.sync();
-    bt_vcycle<G>(T, I, KIND == EQ_PSI, sm, smd);
+    bt_vcycle<G>(T, I, KIND == EQ_PSI);
     bt_add_correction(T, I);
     bool mixstep = false;
     int mst = 0;
@@ -706,7 +711,7 @@ __device__ bool bt_momentum_free(const Team& T, const BatchItem& I, BtShared& S)
 // caller.  Returns the status.
 template <int G>
 __device__ __noinline__ int bt_solve_vec(const Team& T, const BatchItem& I, BatchOut& O, int eq, double* hist,
-                            unsigned char* smem_raw, BtShared& S) {
+                            BtShared& S) {
   const LevelView<double>& L = I.v64;
   const long n = bt_cells(L), ng = bt_ghosted(L);
   bt_fill_u3(T, I);
@@ -739,7 +744,7 @@ __device__ __noinline__ int bt_solve_vec(const Team& T, const BatchItem& I, Batc
       for (long q = T.start(); q < ng; q += T.stride()) I.lv[0].e3[c][q] = 0.0f;
     }
     T.sync();
-    bt_vcycle_vec<G>(T, I, smem_raw);
+    bt_vcycle_vec<G>(T, I);
     // u += e, then the FP64 ghosts
     for (long q = T.start(); q < n; q += T.stride()) {
       int i, j, k;
@@ -804,10 +809,7 @@ __device__ void bt_trivial(const Team& T, BatchOut& O, int eq, double* hist) {
 // the four equations' histories.  Problems with momentum on a hierarchy
 // whose vector levels do not fit are marked BATCH_GENERAL.
 template <int G>
-__device__ void bt_problem(const Team& T, const BatchItem& I, BatchOut& O, double* hist, unsigned char* smem_raw,
-                           BtShared& S) {
-  float* sm = reinterpret_cast<float*>(smem_raw);
-  double* smd = reinterpret_cast<double*>(smem_raw + I.bc.fp64_at);
+__device__ void bt_problem(const Team& T, const BatchItem& I, BatchOut& O, double* hist,                            BtShared& S) {
   const LevelView<double>& L = I.v64;
   const long n = bt_cells(L), ng = bt_ghosted(L);
   bool mf = true;  // momentum-free: X = beta = 0 exactly
@@ -832,7 +834,7 @@ __device__ void bt_problem(const Team& T, const BatchItem& I, BatchOut& O, doubl
         }
       }
       T.sync();
-      const int sx = bt_solve_vec<G>(T, I, O, 0, hist, smem_raw, S);
+      const int sx = bt_solve_vec<G>(T, I, O, 0, hist, S);
       for (long q = T.start(); q < ng; q += T.stride())
 #pragma unroll
         for (int c = 0; c < 3; ++c) I.Xg[c][q] = I.u3[c][q];
@@ -870,7 +872,7 @@ __device__ void bt_problem(const Team& T, const BatchItem& I, BatchOut& O, doubl
     I.s1[p] = a2;
   }
   T.sync();
-  const int st = bt_solve<G, EQ_PSI>(T, I, nullptr, I.s0, I.s1, O, 1, hist + BATCH_HIST, sm, smd, S);
+  const int st = bt_solve<G, EQ_PSI>(T, I, nullptr, I.s0, I.s1, O, 1, hist + BATCH_HIST, S);
   if (T.rank == 0 && threadIdx.x == 0) O.ran |= 1 << 1;
   for (long q = T.start(); q < n; q += T.stride()) {
     int i, j, k;
@@ -897,7 +899,7 @@ __device__ void bt_problem(const Team& T, const BatchItem& I, BatchOut& O, doubl
     I.u[p] = I.alpha[q] * (1.0 + I.dpsi[p]) - 1.0;
   }
   T.sync();
-  const int sa = bt_solve<G, EQ_LIN>(T, I, I.f, nullptr, I.s1, O, 2, hist + 2 * BATCH_HIST, sm, smd, S);
+  const int sa = bt_solve<G, EQ_LIN>(T, I, I.f, nullptr, I.s1, O, 2, hist + 2 * BATCH_HIST, S);
   if (T.rank == 0 && threadIdx.x == 0) O.ran |= 1 << 2;
   for (long q = T.start(); q < ng; q += T.stride()) I.dap[q] = I.u[q];
   for (long q = T.start(); q < n; q += T.stride()) {
@@ -938,7 +940,7 @@ __device__ void bt_problem(const Team& T, const BatchItem& I, BatchOut& O, doubl
     }
   }
   T.sync();
-  bt_solve_vec<G>(T, I, O, 3, hist + 3 * BATCH_HIST, smem_raw, S);
+  bt_solve_vec<G>(T, I, O, 3, hist + 3 * BATCH_HIST, S);
   for (long q = T.start(); q < n; q += T.stride()) {
     int i, j, k;
     L.cell(q, i, j, k);
@@ -951,7 +953,7 @@ __device__ void bt_problem(const Team& T, const BatchItem& I, BatchOut& O, doubl
 
 // Problem idx by team T (each block holds its own copy of the descriptor).
 __device__ void bt_run(const Team& T, const BatchItem* items, BatchOut* outs, double* hist, int idx,
-                       unsigned char* smem_raw, BatchItem& I, BtShared& S) {
+                       BatchItem& I, BtShared& S) {
   {
     const int* src = reinterpret_cast<const int*>(items + idx);
     int* dst = reinterpret_cast<int*>(&I);
@@ -970,11 +972,11 @@ __device__ void bt_run(const Team& T, const BatchItem* items, BatchOut* outs, do
   __syncthreads();
   double* h = hist + (long)idx * 4 * BATCH_HIST;
   if (I.geom == CART)
-    bt_problem<CART>(T, I, O, h, smem_raw, S);
+    bt_problem<CART>(T, I, O, h, S);
   else if (I.geom == CYL)
-    bt_problem<CYL>(T, I, O, h, smem_raw, S);
+    bt_problem<CYL>(T, I, O, h, S);
   else
-    bt_problem<SPH>(T, I, O, h, smem_raw, S);
+    bt_problem<SPH>(T, I, O, h, S);
   T.sync();
   if (T.rank == 0 && threadIdx.x == 0) O.t_end = global_ns();
 }
@@ -1006,7 +1008,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 1)
         if (T.rank == 0) first = it;
         break;
       }
-      bt_run(T, items, outs, hist, idx, smem_raw, I, S);
+      bt_run(T, items, outs, hist, idx, I, S);
     }
   }
   const Team T{0, 1};
@@ -1020,7 +1022,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 1)
       __syncthreads();
     }
     if (it >= count) return;
-    bt_run(T, items, outs, hist, order[it], smem_raw, I, S);
+    bt_run(T, items, outs, hist, order[it], I, S);
   }
 }
 

@@ -14,12 +14,10 @@
 namespace gmg {
 
 template <int G, bool VEC>
-__global__ void __launch_bounds__(BC_THREADS) k_block_vcycle32(const __grid_constant__ BlockCycle32 P) {
+__global__ void __launch_bounds__(BC_THREADS, 1) k_block_vcycle32(const __grid_constant__ BlockCycle32 P) {
+  bc_stage_tables(P);  // fixed for the hierarchy: fetched before waiting for the preceding launch
   pdl_entry();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* sm = reinterpret_cast<float*>(smem_raw);
-  double* smd = reinterpret_cast<double*>(smem_raw + P.fp64_at);
-  bc_run<G, VEC>(P, sm, smd);
+  bc_run<G, VEC, false, true>(P);
 }
 
 // Column col of the coarsest vector operator (lap V + 1/3 grad div V with

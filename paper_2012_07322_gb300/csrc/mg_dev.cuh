@@ -316,26 +316,26 @@ __device__ __forceinline__ T lap_scalar(const LevelView<T>& L, const T* __restri
 // Fields with materialised ghosts (edges included).  Components are the
 // orthonormal ones: (x, y, z), (R, z, phi), (r, theta, phi).
 
-template <typename T>
+template <typename T, typename LV = LevelView<T>, typename P = long>
 struct Stencil {
-  const LevelView<T>& L;
-  long p;
+  const LV& L;
+  P p;
   __device__ __forceinline__ T d1(const T* F, int d) const {
     if (d == 0) return (F[p + 1] - F[p - 1]) * L.hc0;
     if (d == 1) return (F[p + L.sx] - F[p - L.sx]) * L.hc1;
     if (!L.three) return T(0);
     return (F[p + L.sy] - F[p - L.sy]) * L.hc2;
   }
-  __device__ __forceinline__ long step(int d) const { return d == 0 ? 1 : (d == 1 ? L.sx : L.sy); }
+  __device__ __forceinline__ P step(int d) const { return d == 0 ? P(1) : (d == 1 ? P(L.sx) : P(L.sy)); }
   __device__ __forceinline__ T hs(int d) const { return d == 0 ? L.ih0s : (d == 1 ? L.ih1s : L.ih2s); }
   __device__ __forceinline__ T d2(const T* F, int d) const {
     if (d == 2 && !L.three) return T(0);
-    long s = step(d);
+    const P s = step(d);
     return (F[p + s] - T(2) * F[p] + F[p - s]) * hs(d);
   }
   __device__ __forceinline__ T mix(const T* F, int a, int b) const {
     if (b == 2 && !L.three) return T(0);
-    long sa = step(a), sb = step(b);
+    const P sa = step(a), sb = step(b);
     const T w = (a == 0 && b == 1) ? L.m01 : (a == 0 ? L.m02 : L.m12);
     if (L.mixed == 0) return (F[p + sa + sb] - F[p + sa - sb] - F[p - sa + sb] + F[p - sa - sb]) * w;
     return (-F[p + sa - sb] - F[p - sa + sb] + F[p + sa] + F[p - sa] + F[p + sb] + F[p - sb] - T(2) * F[p]) * w;
@@ -343,9 +343,8 @@ struct Stencil {
 };
 
 // Flux-form Laplacian of a component with materialised ghosts.
-template <typename T, int G>
-__device__ __forceinline__ T lap_ghosted(const LevelView<T>& L, const T* __restrict__ F, int i, int j, long p,
-                                         T& D) {
+template <typename T, int G, typename LV, typename P>
+__device__ __forceinline__ T lap_ghosted(const LV& L, const T* __restrict__ F, int i, int j, P p, T& D) {
   const T c = F[p];
   const T cE = L.TI(TI_CE, i), cW = L.TI(TI_CW, i);
   T Lu = cE * (F[p + 1] - c) - cW * (c - F[p - 1]);
@@ -406,17 +405,18 @@ __device__ __forceinline__ T vec_op_vc(const LevelView<T>& L, const T* __restric
 
 // Component c of lap V + 1/3 grad div V and its own-value derivative.  VC
 // false compiles the flux form only (the one-block cycle: its register
-// budget of 128 would spill with both forms).
-template <typename T, int G, bool VC = true>
-__device__ __forceinline__ T vec_op(const LevelView<T>& L, const T* __restrict__ A, const T* __restrict__ B,
-                                    const T* __restrict__ C, int c, int i, int j, long p, T& diag) {
+// budget of 128 would spill with both forms, and its levels carry no vc).
+// LV: LevelView, or the one-block cycle's view with 32-bit strides.
+template <typename T, int G, bool VC = true, typename LV, typename P>
+__device__ __forceinline__ T vec_op(const LV& L, const T* __restrict__ A, const T* __restrict__ B,
+                                    const T* __restrict__ C, int c, int i, int j, P p, T& diag) {
   if constexpr (VC && G == SPH && sizeof(T) == 4) {
     // FP32 (smoother and correction residual of mixed precision): the
     // coefficient form when the level carries the table
     if (L.vc && L.mixed == 0) return vec_op_vc<T>(L, A, B, C, c, i, j, p, diag);
   }
   const T third = T(1) / T(3);
-  Stencil<T> s{L, p};
+  const Stencil<T, LV, P> s{L, p};
   T LD;
   if (G == CART) {
     const T* V = (c == 0) ? A : (c == 1 ? B : C);

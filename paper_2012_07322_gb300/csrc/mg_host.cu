@@ -831,20 +831,30 @@ BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0) {
     BlockLevel32& B = P.lv[q];
     B.v = with_bc(L.v32, e.bc);
     for (int c = 0; c < 3; ++c) {
-      if (c < nc) {
-        B.e[c] = take(L.ng);
-        B.f32[c] = take(L.ng);
-        B.r32[c] = take(L.ng);
-      } else {
-        B.e[c] = B.e[0];
-        B.f32[c] = B.f32[0];
-        B.r32[c] = B.r32[0];
-      }
+      B.e[c] = c < nc ? take(L.ng) : B.e[0];
+      B.f32[c] = c < nc ? take(L.ng) : B.f32[0];
     }
     B.k32 = hasK ? L.k32 : nullptr;
     B.ti_at = take((long)NTI * (L.n[0] + 2));
     B.tj_at = take((long)NTJ * (L.n[1] + 2));
     B.k_at = hasK ? take(L.ng) : -1;
+    B.gc = e.bc == MG_BC_DIRICHLET ? -1.0f : (e.bc == MG_BC_NEUMANN ? 1.0f : L.v32.robin0);
+    B.gf_at = -1;
+    if (P.vec) {
+      B.ng = (int)ghost_count_host(L.v32);
+      B.gt_at = take(2 * (long)B.ng);
+      if (e.bc == MG_BC_ROBIN) B.gf_at = take(B.ng);
+      if (L.ng > 0xffff) return P;  // offsets of 16 bits; P.smem = 0
+    } else if (e.bc == MG_BC_ROBIN && H->d.geom != MG_SPH) {
+      const int f0 = L.n[1] * L.n[2], f1 = L.n[0] * L.n[2], f2 = L.n[0] * L.n[1];
+      const int size[6] = {f0, f0, f1, f1, f2, f2};
+      int at = 0;
+      for (int m = 0; m < 6; ++m) {
+        B.g_face[m] = at;
+        at += size[m];
+      }
+      B.gf_at = take(at);
+    }
   }
   Level& Lc = H->L[H->nlev - 1];
   P.c64 = with_bc(Lc.v64, e.bc);
@@ -888,13 +898,11 @@ int block_cycle_level(mg_hierarchy* H, const Eq& e) {
   return H->nlev;
 }
 
-void restrict_k32(mg_hierarchy* H, int from);
-
 // vcycle32 from level l0 down, in one block.
 void block_vcycle32(mg_hierarchy* H, const Eq& e, int l0) {
-  // K of eq. psi reached level l0 with the down leg; on to the block's levels
-  if (H->fold_k32) restrict_k32(H, l0 + 1);
-  const BlockCycle32 P = block_cycle_params(H, e, l0);
+  // K of eq. psi reached level l0 with the down leg; the block restricts it further
+  BlockCycle32 P = block_cycle_params(H, e, l0);
+  P.fold_k = H->fold_k32;
   for (int l = l0; l + 1 < H->nlev; ++l) H->updates += (int64_t)(H->d.nu1 + H->d.nu2) * H->L[l].cells() * e.ncomp;
   long tok = prof_begin(H, l0, MG_PROF_BLOCK_CYCLE32, H->L[l0].cells());
   launch_block_vcycle32(P, H->d.geom, H->st);

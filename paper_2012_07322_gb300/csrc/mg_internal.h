@@ -372,12 +372,19 @@ constexpr long BLOCK_CYCLE_CELLS = 4096;       // levels this small run in the b
 constexpr size_t BC_SMEM_MAX = 200 * 1024;     // dynamic shared memory of the block cycle
 struct BlockLevel32 {
   LevelView<float> v;        // boundary rule applied
-  int e[3], f32[3], r32[3];  // offsets (floats) of correction, right-hand side, residual in shared memory
+  int e[3], f32[3];          // offsets (floats) of correction and right-hand side in shared memory
   const float* k32;          // c of (L - c) e = f in HBM, null without
   int ti_at, tj_at, k_at;    // offsets (floats) of the level's coefficient tables and of c in shared memory
+  // Ghost rules, evaluated once per cycle.  Scalar: outer factors per face
+  // (low, high per dimension, offsets in gf_at; gf_at < 0: gc on every face).
+  // Vector: ng ghosts' sources and signs at gt_at (8 bytes each), and with
+  // the Robin rule their factors at gf_at.
+  int gf_at, g_face[6], gt_at, ng;
+  float gc;
 };
 struct BlockCycle32 {
   int nl, vec, nu1, nu2, coarse_sweeps;
+  int fold_k;  // restrict c from level l0 on the way down (else every level's is read from HBM)
   BlockLevel32 lv[BC_MAX];
   LevelView<double> c64;  // the coarsest level, boundary rule applied
   int cu[3], cf[3], ck;   // offsets (doubles, from fp64_at) of the FP64 coarsest solve; ck < 0: no c

@@ -98,10 +98,9 @@ __device__ __forceinline__ void scalar_update_lin_inv(const LevelView<T>& L, T* 
 
 // New value of vector component c at a cell after one Newton-Gauss-Seidel
 // update (ghosts current).
-template <typename T, int G, bool VC = true>
-__device__ __forceinline__ T vec_new_value(const LevelView<T>& L, T* __restrict__ A, T* __restrict__ B,
-                                           T* __restrict__ C, const T* __restrict__ f, int c, int i, int j,
-                                           long p) {
+template <typename T, int G, bool VC = true, typename LV, typename P>
+__device__ __forceinline__ T vec_new_value(const LV& L, T* __restrict__ A, T* __restrict__ B, T* __restrict__ C,
+                                           const T* __restrict__ f, int c, int i, int j, P p) {
   T D;
   T Lu = vec_op<T, G, VC>(L, A, B, C, c, i, j, p, D);
   const T* V = (c == 0) ? A : (c == 1 ? B : C);
@@ -218,10 +217,10 @@ __device__ __forceinline__ T scalar_residual_cell(const LevelView<T>& L, const T
 
 // Residual f_c - (lap V + 1/3 grad div V)_c of a vector equation (ghosts
 // current).
-template <typename T, int G, bool VC = true>
-__device__ __forceinline__ T vec_residual_cell(const LevelView<T>& L, const T* __restrict__ A,
-                                               const T* __restrict__ B, const T* __restrict__ C,
-                                               const T* __restrict__ f, int c, int i, int j, long p) {
+template <typename T, int G, bool VC = true, typename LV, typename P>
+__device__ __forceinline__ T vec_residual_cell(const LV& L, const T* __restrict__ A, const T* __restrict__ B,
+                                               const T* __restrict__ C, const T* __restrict__ f, int c, int i, int j,
+                                               P p) {
   T D;
   const T Lu = vec_op<T, G, VC>(L, A, B, C, c, i, j, p, D);
   const T fv = f ? f[p] : T(0);
