@@ -35,8 +35,13 @@ enum { TJ_S = 0, TJ_C, TJ_IS, TJ_IS2, TJ_COT, TJ_TN, TJ_TS, TJ_PF, TJ_VW, NTJ };
 // Per-(i, j) stencil coefficients of the vector operator on spherical
 // levels with four-point mixed derivatives (FP64 residual), stored
 // coefficient-major: vc[(q * n1 + j) * n0 + i].  Slots 0-11 component r,
-// 12-21 theta, 22-31 phi (k_residual_vec_sph), 32 the norm weight.
-constexpr int VC_N = 34;
+// 12-21 theta, 22-31 phi (k_residual_vec_sph), 32 the norm weight, 33-35 the
+// zero-order coefficient and 36-38 the inverted Newton diagonal of each
+// component (vec_op_dc).
+constexpr int VC_N = 40;
+// The FP64 coefficients of vec_op_dc on cylindrical levels (per i, slot-major
+// vc[q * n0 + i]) and on Cartesian ones (vc[q]).
+constexpr int VY_N = 20, VX_N = 12;
 
 template <typename T>
 struct LevelView {
@@ -401,6 +406,90 @@ __device__ __forceinline__ T vec_op_vc(const LevelView<T>& L, const T* __restric
             cf(30) * (B[p + sy] - B[p - sy]) + cf(31) * mix4(B, sx, sy);
   }
   return Lu;
+}
+
+// Component c of lap V + 1/3 grad div V in FP64 from the level's coefficient
+// table (four-point mixed derivatives), iD its inverted Newton diagonal:
+// neighbours are subtracted from the cell's own value before they are
+// multiplied, as in the flux form below, and the metric factors, the 1/3 and
+// the difference scales of a term are one coefficient.  ~30 FP64 operations
+// per component instead of ~100 and a division: the FP64 pipe bounds the
+// FP64 vector passes (64x32x32 colour pass 11 us with the flux form).
+template <int G>
+__device__ __forceinline__ double vec_op_dc(const LevelView<double>& L, const double* __restrict__ A,
+                                            const double* __restrict__ B, const double* __restrict__ C, int c, int i,
+                                            int j, long p, double& iD) {
+  const long sx = L.sx, sy = L.sy;
+  auto mix4 = [&](const double* F, long a, long b) {
+    return ((F[p + a + b] - F[p + a - b]) - F[p - a + b]) + F[p - a - b];
+  };
+  const double* F = c == 0 ? A : (c == 1 ? B : C);
+  const double v = F[p];
+  // own component: six neighbours (coefficients e, w, n, s, z) in two chains
+  auto own = [&](double e, double w, double n, double s, double z) {
+    double a = e * (F[p + 1] - v) + w * (F[p - 1] - v);
+    double b = n * (F[p + sx] - v) + s * (F[p - sx] - v);
+    if (L.three) a += z * ((F[p + sy] - v) + (F[p - sy] - v));
+    return a + b;
+  };
+  if (G == SPH) {
+    const long qs = (long)L.n0 * L.n1;
+    const double* __restrict__ V = L.vc + (long)j * L.n0 + i;
+    auto cf = [&](int q) { return V[q * qs]; };
+    iD = cf(36 + c);
+    if (c == 0) {
+      double x = cf(33) * v + cf(6) * (B[p + sx] - B[p - sx]) + cf(7) * B[p] + cf(8) * (B[p + 1] - B[p - 1]) +
+                 cf(9) * mix4(B, 1, sx);
+      if (L.three) x += cf(10) * (C[p + sy] - C[p - sy]) + cf(11) * mix4(C, 1, sy);
+      return own(cf(0), cf(1), cf(2), cf(3), cf(4)) + x;
+    } else if (c == 1) {
+      double x = cf(34) * v + cf(18) * (A[p + sx] - A[p - sx]) + cf(19) * mix4(A, 1, sx);
+      if (L.three) x += cf(20) * (C[p + sy] - C[p - sy]) + cf(21) * mix4(C, sx, sy);
+      return own(cf(12), cf(13), cf(14), cf(15), cf(16)) + x;
+    }
+    double x = cf(35) * v;
+    if (L.three)
+      x += cf(28) * (A[p + sy] - A[p - sy]) + cf(29) * mix4(A, 1, sy) + cf(30) * (B[p + sy] - B[p - sy]) +
+           cf(31) * mix4(B, sx, sy);
+    return own(cf(22), cf(23), cf(24), cf(25), cf(26)) + x;
+  }
+  if (G == CYL) {
+    const double* __restrict__ V = L.vc + i;
+    const int n0 = L.n0;
+    auto cf = [&](int q) { return V[q * n0]; };
+    if (c == 0) {
+      iD = cf(7);
+      double x = cf(3) * v + cf(4) * mix4(B, 1, sx);
+      if (L.three) x += cf(5) * (C[p + sy] - C[p - sy]) + cf(6) * mix4(C, 1, sy);
+      const double n = L.ih1s;
+      return own(cf(0), cf(1), n, n, cf(2)) + x;
+    } else if (c == 1) {
+      iD = cf(14);
+      double x = cf(4) * mix4(A, 1, sx) + cf(12) * (A[p + sx] - A[p - sx]);
+      if (L.three) x += cf(13) * mix4(C, sx, sy);
+      const double n = cf(10);
+      return own(cf(8), cf(9), n, n, cf(11)) + x;
+    }
+    iD = cf(19);
+    double x = cf(17) * v;
+    if (L.three) x += cf(18) * (A[p + sy] - A[p - sy]) + cf(6) * mix4(A, 1, sy) + cf(13) * mix4(B, sx, sy);
+    const double n = cf(15);
+    return own(cf(8), cf(9), n, n, cf(16)) + x;
+  }
+  const double* __restrict__ V = L.vc;
+  iD = V[9 + c];
+  const double e = V[c == 0 ? 3 : 0], n = V[c == 1 ? 4 : 1], z = V[c == 2 ? 5 : 2];
+  double x = 0.0;
+  if (c == 0) {
+    x = V[6] * mix4(B, 1, sx);
+    if (L.three) x += V[7] * mix4(C, 1, sy);
+  } else if (c == 1) {
+    x = V[6] * mix4(A, 1, sx);
+    if (L.three) x += V[8] * mix4(C, sx, sy);
+  } else if (L.three) {
+    x = V[7] * mix4(A, 1, sy) + V[8] * mix4(B, sx, sy);
+  }
+  return own(e, e, n, n, z) + x;
 }
 
 // Component c of lap V + 1/3 grad div V and its own-value derivative.  VC

@@ -39,7 +39,8 @@ struct Level {
   LevelView<float> v32;
   double* ti64 = nullptr;
   double* tj64 = nullptr;
-  double* vc64 = nullptr;  // spherical, four-point mixed derivatives: VC_N x n0 x n1
+  // four-point mixed derivatives: spherical VC_N x n0 x n1, cylindrical VY_N x n0, Cartesian VX_N
+  double* vc64 = nullptr;
   float* vc32 = nullptr;   // the same in FP32 (FP32 vector smoother and residual)
   float* ti32 = nullptr;
   float* tj32 = nullptr;
@@ -323,6 +324,8 @@ size_t layout(mg_hierarchy* H, const mg_grid_desc* d, char* base) {
     t64(L ? &L->ti64 : &dummy64, sizeof(double) * NTI * (n[l][0] + 2));
     t64(L ? &L->tj64 : &dummy64, sizeof(double) * NTJ * (n[l][1] + 2));
     t32(L ? &L->ti32 : &dummy32, sizeof(float) * NTI * (n[l][0] + 2));
+    if (d->geom != MG_SPH && d->mixed_deriv == MG_MIXED_4PT)
+      t64(L ? &L->vc64 : &dummy64, sizeof(double) * (d->geom == MG_CYL ? VY_N * n[l][0] : VX_N));
     if (d->geom == MG_SPH && d->mixed_deriv == MG_MIXED_4PT) {
       t64(L ? &L->vc64 : &dummy64, sizeof(double) * VC_N * n[l][0] * n[l][1]);
       if (mixed) t32(L ? &L->vc32 : &dummy32, sizeof(float) * VC_N * n[l][0] * n[l][1]);
@@ -483,8 +486,71 @@ void make_vec_coeffs(const mg_grid_desc* d, const Level& L, const std::vector<do
       c[30] = three ? 7.0 * t3 * ct * ir2 * ist2 * hc2 : 0.0;
       c[31] = three ? t3 * ir2 * ist * m12 : 0.0;
       c[32] = x * x * s;  // norm weight r^2 sin(theta)
+      c[33] = -8.0 * t3 * ir2;
+      c[34] = -4.0 * t3 * ir2 * ist2;
+      c[35] = -ir2 * ist2;
+      c[36] = 1.0 / c[5];
+      c[37] = 1.0 / c[17];
+      c[38] = 1.0 / c[27];
       for (int q = 0; q < VC_N; ++q) vc[((size_t)q * n1 + j) * n0 + i] = c[q];
     }
+}
+
+// The coefficients of vec_op_dc on a cylindrical level (slots per i) or a
+// Cartesian one: those of vec_op, multiplied out.
+void make_vec_coeffs_dc(const mg_grid_desc* d, const Level& L, const std::vector<double>& ti, std::vector<double>& vc) {
+  const int n0 = L.n[0];
+  const bool three = d->ndim == 3;
+  const double ih0s = 1.0 / (L.h[0] * L.h[0]), ih1s = 1.0 / (L.h[1] * L.h[1]);
+  const double ih2s = three ? 1.0 / (L.h[2] * L.h[2]) : 0.0;
+  const double hc0 = 0.5 / L.h[0], hc1 = 0.5 / L.h[1], hc2 = 0.5 / L.h[2];
+  const double m01 = 1.0 / (4.0 * L.h[0] * L.h[1]), m02 = 1.0 / (4.0 * L.h[0] * L.h[2]);
+  const double m12 = 1.0 / (4.0 * L.h[1] * L.h[2]), t3 = 1.0 / 3.0;
+  if (d->geom == MG_CART) {
+    vc.assign(VX_N, 0.0);
+    const double ihs[3] = {ih0s, ih1s, ih2s}, lap = -2.0 * (ih0s + ih1s + ih2s);
+    for (int c = 0; c < 3; ++c) {
+      vc[c] = ihs[c];
+      vc[3 + c] = ihs[c] + t3 * ihs[c];
+      vc[9 + c] = 1.0 / (lap - 2.0 * t3 * ihs[c]);
+    }
+    vc[6] = t3 * m01;
+    vc[7] = t3 * m02;
+    vc[8] = t3 * m12;
+    return;
+  }
+  vc.assign((size_t)VY_N * n0, 0.0);
+  for (int i = 0; i < n0; ++i) {
+    auto I = [&](int s) { return ti[(size_t)s * (n0 + 2) + i + 1]; };
+    auto S = [&](int q) -> double& { return vc[(size_t)q * n0 + i]; };
+    const double iR = I(TI_IX), iR2 = I(TI_IX2), cE = I(TI_CE), cW = I(TI_CW), pf = three ? I(TI_PHI) : 0.0;
+    const double lap = -(cE + cW) - 2.0 * ih1s - 2.0 * pf;
+    // R: lap V_R + 1/3 d_RR V_R + 1/3 R^-1 d_R V_R - 4/3 R^-2 V_R + 1/3 d_R d_z V_z
+    //    - 7/3 R^-2 d_phi V_phi + 1/3 R^-1 d_R d_phi V_phi
+    S(0) = cE + t3 * (ih0s + iR * hc0);
+    S(1) = cW + t3 * (ih0s - iR * hc0);
+    S(2) = pf;
+    S(3) = -4.0 * t3 * iR2;
+    S(4) = t3 * m01;
+    S(5) = three ? -7.0 * t3 * iR2 * hc2 : 0.0;
+    S(6) = three ? t3 * iR * m02 : 0.0;
+    S(7) = 1.0 / (lap - iR2 + t3 * (-2.0 * ih0s - iR2));
+    // z: lap V_z + 1/3 d_zz V_z + 1/3 d_R d_z V_R + 1/3 R^-1 d_z V_R + 1/3 R^-1 d_z d_phi V_phi
+    S(8) = cE;
+    S(9) = cW;
+    S(10) = ih1s + t3 * ih1s;
+    S(11) = pf;
+    S(12) = t3 * iR * hc1;
+    S(13) = three ? t3 * iR * m12 : 0.0;
+    S(14) = 1.0 / (lap - 2.0 * t3 * ih1s);
+    // phi: lap V_phi + 1/3 R^-2 d_phiphi V_phi - R^-2 V_phi + 7/3 R^-2 d_phi V_R
+    //    + 1/3 R^-1 d_R d_phi V_R + 1/3 R^-1 d_z d_phi V_z
+    S(15) = ih1s;
+    S(16) = pf + (three ? t3 * iR2 * ih2s : 0.0);
+    S(17) = -iR2;
+    S(18) = three ? 7.0 * t3 * iR2 * hc2 : 0.0;
+    S(19) = 1.0 / (lap - iR2 - (three ? 2.0 * t3 * iR2 * ih2s : 0.0));
+  }
 }
 
 template <typename T>
@@ -2180,7 +2246,10 @@ int mg_create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, mg_hierarch
     std::vector<double> vc;
     std::vector<float> vc32;
     if (L.vc64) {
-      make_vec_coeffs(&H->d, L, ti, tj, vc);
+      if (H->d.geom == MG_SPH)
+        make_vec_coeffs(&H->d, L, ti, tj, vc);
+      else
+        make_vec_coeffs_dc(&H->d, L, ti, vc);
       if (ce == cudaSuccess)
         ce = cudaMemcpyAsync(L.vc64, vc.data(), sizeof(double) * vc.size(), cudaMemcpyHostToDevice, H->st);
       if (L.vc32) {

@@ -893,8 +893,7 @@ __global__ void k_apply_vec(LevelView<T> L, const T* __restrict__ A, const T* __
   T* os[3] = {o0, o1, o2};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    T D;
-    const T Lu = vec_op<T, G>(L, A, B, C, c, i, j, p, D);
+    const T Lu = vec_apply_cell<T, G>(L, A, B, C, c, i, j, p);
     os[c][p] = add ? os[c][p] + Lu : Lu;
   }
 }

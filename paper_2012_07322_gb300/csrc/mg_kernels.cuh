@@ -101,10 +101,16 @@ __device__ __forceinline__ void scalar_update_lin_inv(const LevelView<T>& L, T* 
 template <typename T, int G, bool VC = true, typename LV, typename P>
 __device__ __forceinline__ T vec_new_value(const LV& L, T* __restrict__ A, T* __restrict__ B, T* __restrict__ C,
                                            const T* __restrict__ f, int c, int i, int j, P p) {
-  T D;
-  T Lu = vec_op<T, G, VC>(L, A, B, C, c, i, j, p, D);
   const T* V = (c == 0) ? A : (c == 1 ? B : C);
   const T fv = f ? f[p] : T(0);
+  T D;
+  if constexpr (VC && sizeof(T) == 8) {
+    if (L.vc && L.mixed == 0) {
+      const T Lv = vec_op_dc<G>(L, A, B, C, c, i, j, p, D);
+      return V[p] - (Lv - fv) * D;
+    }
+  }
+  T Lu = vec_op<T, G, VC>(L, A, B, C, c, i, j, p, D);
   return V[p] - (Lu - fv) / D;
 }
 
@@ -215,16 +221,25 @@ __device__ __forceinline__ T scalar_residual_cell(const LevelView<T>& L, const T
   return fv - Lu;
 }
 
+// (lap V + 1/3 grad div V)_c at a cell (ghosts current).
+template <typename T, int G, bool VC = true, typename LV, typename P>
+__device__ __forceinline__ T vec_apply_cell(const LV& L, const T* __restrict__ A, const T* __restrict__ B,
+                                            const T* __restrict__ C, int c, int i, int j, P p) {
+  T D;
+  if constexpr (VC && sizeof(T) == 8) {
+    if (L.vc && L.mixed == 0) return vec_op_dc<G>(L, A, B, C, c, i, j, p, D);
+  }
+  return vec_op<T, G, VC>(L, A, B, C, c, i, j, p, D);
+}
+
 // Residual f_c - (lap V + 1/3 grad div V)_c of a vector equation (ghosts
 // current).
 template <typename T, int G, bool VC = true, typename LV, typename P>
 __device__ __forceinline__ T vec_residual_cell(const LV& L, const T* __restrict__ A, const T* __restrict__ B,
                                                const T* __restrict__ C, const T* __restrict__ f, int c, int i, int j,
                                                P p) {
-  T D;
-  const T Lu = vec_op<T, G, VC>(L, A, B, C, c, i, j, p, D);
   const T fv = f ? f[p] : T(0);
-  return fv - Lu;
+  return fv - vec_apply_cell<T, G, VC>(L, A, B, C, c, i, j, p);
 }
 
 // Volume-weighted piecewise-constant restriction (Sec. 2.7.3, weights
