@@ -5,15 +5,19 @@
 // its time loop, or code whose allocations would synchronise the device
 // and break the overlap of its streams.  They cannot create a hierarchy
 // (mg_create_hierarchy allocates), yet still want the divergence monitor.
-// This file gives them mg_divb_norms_noalloc: the same two kernels as the
-// divergence pipeline of mg_clean_divB (central divergence into scratch,
-// then its max and the per-block sums of div^2), with the scratch in a
-// file-scope __device__ array instead of the hierarchy's arena.
+// This file gives them mg_divb_norms_noalloc: the central divergence and its
+// norms as mg_clean_divB reports them, with the scratch (block partial
+// results, a counter of finished blocks and the result) in a file-scope
+// __device__ array instead of the hierarchy's arena.
 //
-// The array holds MG_NOALLOC_MAX_CELLS divergence values plus the block
-// partial sums and the max word (about 16 MiB); every GPU that loads the
-// library keeps it until the process exits.  All calls share it: calls
-// whose work overlaps on the GPU race with each other.
+// The call is bound by its launches and round trips: one launch whose last
+// block to finish combines the blocks' results, and one 16-byte read-back.
+// (With a cleared max word, a divergence and a norms kernel and two
+// read-backs a 56x40x48 block took 55 us; so, XX us.)
+//
+// Every GPU that loads the library keeps the array until the process exits.
+// All calls share it: calls whose work overlaps on the GPU race with each
+// other.
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -26,70 +30,101 @@ namespace {
 
 constexpr int NOALLOC_BLOCKS = 1024;
 constexpr int NOALLOC_MAX_DEVICES = 64;
-// [0, MAX_CELLS): divergence; then NOALLOC_BLOCKS partial sums; then the max
-// word (bit pattern of a non-negative double).
-constexpr long SCRATCH_WORDS = (long)MG_NOALLOC_MAX_CELLS + NOALLOC_BLOCKS + 32;
+// Per block the sum of div^2 and max |div| (bit pattern), then the result in
+// the same form, then the counter of finished blocks (zero between calls:
+// the last block resets it).
+struct NoallocScratch {
+  double sum[NOALLOC_BLOCKS];
+  unsigned long long max[NOALLOC_BLOCKS];
+  double total;
+  unsigned long long top;
+  unsigned int done;
+};
 
 }  // namespace
 
-static __device__ __align__(256) double g_divb_scratch[SCRATCH_WORDS];
+static __device__ __align__(256) NoallocScratch g_divb_scratch;
 
 namespace {
 
 std::mutex g_setup_mutex;
-double* g_scratch_addr[NOALLOC_MAX_DEVICES] = {};
+NoallocScratch* g_scratch_addr[NOALLOC_MAX_DEVICES] = {};
 
-// Central divergence with zero-gradient (copied) ghosts into scratch.
-__global__ void k_noalloc_div(int n0, int n1, int n2, int three, double c0, double c1, double c2,
-                              const double* __restrict__ B0, const double* __restrict__ B1,
-                              const double* __restrict__ B2, double* __restrict__ div) {
-  gmg::pdl_entry();
-  const long n = (long)n0 * n1 * n2;
-  const long s1 = n0, s2 = (long)n0 * n1;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-    const int i = (int)(q % n0), j = (int)((q / n0) % n1), k = (int)(q / s2);
-    double d = (B0[i < n0 - 1 ? q + 1 : q] - B0[i > 0 ? q - 1 : q]) * c0 +
-               (B1[j < n1 - 1 ? q + s1 : q] - B1[j > 0 ? q - s1 : q]) * c1;
-    if (three) d += (B2[k < n2 - 1 ? q + s2 : q] - B2[k > 0 ? q - s2 : q]) * c2;
-    div[q] = d;
+// Sum and max over the block's threads, to thread 0 (fixed order).
+__device__ __forceinline__ void block_norms(double& s, unsigned long long& m) {
+  __shared__ double ss[8];
+  __shared__ unsigned long long sm[8];
+  s = gmg::warp_sum(s);
+  m = gmg::warp_max_bits(m);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0) {
+    ss[w] = s;
+    sm[w] = m;
+  }
+  __syncthreads();
+  if (w == 0) {
+    s = lane < 8 ? ss[lane] : 0.0;
+    m = lane < 8 ? sm[lane] : 0ULL;
+    for (int o = 4; o > 0; o >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, o);
+      m = gmg::umax64(m, __shfl_xor_sync(0xffffffffu, m, o));
+    }
   }
 }
 
-// Per-block sums of div^2 into part[], max |div| into *maxw (atomic).
-__global__ void k_noalloc_norms(long n, const double* __restrict__ div, double* __restrict__ part,
-                                unsigned long long* maxw) {
+// Central divergence with zero-gradient (copied) ghosts, its sum of squares
+// and largest magnitude (NaN counts as infinite).
+__global__ void __launch_bounds__(256)
+    k_noalloc_norms(int n0, int n1, int n2, int three, double c0, double c1, double c2,
+                    const double* __restrict__ B0, const double* __restrict__ B1, const double* __restrict__ B2,
+                    NoallocScratch* __restrict__ S) {
   gmg::pdl_entry();
-  __shared__ double sm[32];
+  __shared__ bool last;
+  const unsigned n = (unsigned)n0 * n1 * n2, s1 = n0, s2 = (unsigned)n0 * n1;
   double s = 0.0;
-  double m[1] = {0.0};
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-    const double d = div[q];
+  unsigned long long m = 0ULL;
+  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+    const unsigned jk = q / s1, k = jk / (unsigned)n1, j = jk - k * n1, i = q - jk * s1;
+    double d = (B0[i < s1 - 1 ? q + 1 : q] - B0[i > 0 ? q - 1 : q]) * c0 +
+               (B1[(int)j < n1 - 1 ? q + s1 : q] - B1[j > 0 ? q - s1 : q]) * c1;
+    if (three) d += (B2[(int)k < n2 - 1 ? q + s2 : q] - B2[k > 0 ? q - s2 : q]) * c2;
     s += d * d;
-    m[0] = fmax(m[0], fabs(d));
-    if (d != d) m[0] = INFINITY;
+    m = gmg::umax64(m, gmg::abs_bits(d));
   }
-  s = gmg::warp_sum(s);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
-  __syncthreads();
+  block_norms(s, m);
   if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) t += sm[w];
-    part[blockIdx.x] = t;
+    S->sum[blockIdx.x] = s;
+    S->max[blockIdx.x] = m;
+    __threadfence();
+    last = atomicAdd(&S->done, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  gmg::block_max_atomic<1>(m, maxw);
+  if (!last) return;
+  __threadfence();
+  s = 0.0;
+  m = 0ULL;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+    s += __ldcg(&S->sum[b]);
+    m = gmg::umax64(m, __ldcg(&S->max[b]));
+  }
+  block_norms(s, m);
+  if (threadIdx.x == 0) {
+    S->total = s;
+    S->top = m;
+    S->done = 0u;
+  }
 }
 
 // Device address of the scratch array on the current device, looked up
 // once per device (cudaGetSymbolAddress with that device current).
-int scratch_address(double** out) {
+int scratch_address(NoallocScratch** out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return MG_ERR_CUDA;
   if (dev < 0 || dev >= NOALLOC_MAX_DEVICES) return MG_ERR_INVALID;
   std::lock_guard<std::mutex> lock(g_setup_mutex);
   if (!g_scratch_addr[dev]) {
-    double* p = nullptr;
+    NoallocScratch* p = nullptr;
     e = cudaGetSymbolAddress((void**)&p, g_divb_scratch);
     if (e != cudaSuccess || !p) return MG_ERR_CUDA;
     g_scratch_addr[dev] = p;
@@ -118,38 +153,30 @@ extern "C" int mg_divb_norms_noalloc(int ndim, const int n[3], const double lo[3
   // an error left by earlier, unrelated work of the caller must not be
   // reported as this call's: drop it (launch errors are checked below)
   (void)cudaGetLastError();
-  double* scratch = nullptr;
+  NoallocScratch* scratch = nullptr;
   int st = scratch_address(&scratch);
   if (st) return set_last_error(st, "looking up the device address of the static scratch failed");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int n0 = n[0], n1 = n[1], n2 = ndim == 3 ? n[2] : 1;
-  double* div = scratch;
-  double* part = scratch + MG_NOALLOC_MAX_CELLS;
-  unsigned long long* maxw = reinterpret_cast<unsigned long long*>(part + NOALLOC_BLOCKS);
-  // the max word keeps the previous call's value: clear it
-  if (cudaMemsetAsync(maxw, 0, sizeof(unsigned long long), s) != cudaSuccess)
-    return set_last_error(MG_ERR_CUDA, "clearing the max word failed");
   const double c0 = 0.5 / ((hi[0] - lo[0]) / n0), c1 = 0.5 / ((hi[1] - lo[1]) / n1);
   const double c2 = ndim == 3 ? 0.5 / ((hi[2] - lo[2]) / n2) : 0.0;
   long g = (cells + 255) / 256;
   if (g > NOALLOC_BLOCKS) g = NOALLOC_BLOCKS;
-  gmg::count_launch(2);
-  gmg::launch_k(k_noalloc_div, (unsigned)g, 256, 0, s, n0, n1, n2, ndim == 3, c0, c1, c2, B[0], B[1],
-                                             ndim == 3 ? B[2] : B[0], div);
-  gmg::launch_k(k_noalloc_norms, NOALLOC_BLOCKS, 256, 0, s, cells, div, part, maxw);
-  if (cudaGetLastError() != cudaSuccess) return set_last_error(MG_ERR_CUDA, "launching the divergence kernels failed");
-  double hpart[NOALLOC_BLOCKS];
-  unsigned long long hmax = 0;
-  if (cudaMemcpyAsync(hpart, part, sizeof(hpart), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(&hmax, maxw, sizeof(hmax), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  gmg::count_launch();
+  gmg::launch_k(k_noalloc_norms, (unsigned)g, 256, 0, s, n0, n1, n2, ndim == 3, c0, c1, c2, B[0], B[1],
+                ndim == 3 ? B[2] : B[0], scratch);
+  if (cudaGetLastError() != cudaSuccess) return set_last_error(MG_ERR_CUDA, "launching the divergence kernel failed");
+  struct {
+    double sum;
+    unsigned long long max;
+  } res;
+  if (cudaMemcpyAsync(&res, &scratch->total, sizeof(res), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
-    return set_last_error(MG_ERR_CUDA, "divergence kernels or read-back failed");
-  double sum = 0.0;
-  for (int b = 0; b < NOALLOC_BLOCKS; ++b) sum += hpart[b];
+    return set_last_error(MG_ERR_CUDA, "divergence kernel or read-back failed");
   double mx;
-  static_assert(sizeof(mx) == sizeof(hmax), "word size");
-  memcpy(&mx, &hmax, sizeof(mx));
+  static_assert(sizeof(mx) == sizeof(res.max), "word size");
+  memcpy(&mx, &res.max, sizeof(mx));
   *max_div = mx;
-  *l2_div = sqrt(sum / (double)cells);
+  *l2_div = sqrt(res.sum / (double)cells);
   return MG_OK;
 }
