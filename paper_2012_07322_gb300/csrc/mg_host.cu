@@ -83,6 +83,7 @@ struct mg_hierarchy {
   // staging buffers for MG_HOST_POINTERS (allocated on first use)
   std::vector<double*> stage;
   int64_t updates = 0;
+  int cycles_done = 0;  // cycles of the solve in progress
   // optional event timing of finest-level kernels (mg_profile_enable)
   // Anderson mixing storage (allocated on first use): x, fprev, gprev, then
   // m columns of dF and m of dG, each ncomp arrays of L0.ng doubles
@@ -364,7 +365,7 @@ size_t layout(mg_hierarchy* H, const mg_grid_desc* d, char* base) {
   }
   char* p = take(sizeof(unsigned long long) * 8);
   if (H) H->d_red = (unsigned long long*)p;
-  p = take(sizeof(double) * NPARTS);
+  p = take(sizeof(double) * 2 * NPARTS);  // two sets of block sums
   if (H) H->d_part = (double*)p;
   return (off + 255) & ~size_t(255);
 }
@@ -1050,10 +1051,20 @@ void fmg32(mg_hierarchy* H, const Eq& e) {
 
 // ---------------------------------------------------------- cycle control
 
+// Whether the Neumann gauge can be fixed once, after the last cycle: the
+// operator, its residual and the corrections do not see a constant added to
+// u (a linear equation without c under Neumann rules), so removing the mean
+// after every cycle (two passes over u: 100 us of a 1.4 ms cycle at 256^3)
+// changes nothing but the constant.  The mixing does see it.
+bool gauge_at_end(const mg_hierarchy* H, const Eq& e) {
+  return e.zero_mean && e.kind == EQ_LIN && !e.has_c && e.bc == MG_BC_NEUMANN && H->d.accel_depth == 0;
+}
+
 // One application of the iteration map: a V-cycle (FP64 FAS, or the FP32
 // correction cycle of the defect-correction loop) and the Neumann gauge.
 int cycle_map(mg_hierarchy* H, const Eq& e) {
   Level& L0 = H->L[0];
+  const bool per_cycle_mean = e.zero_mean && !gauge_at_end(H, e);
   const bool fmg = H->d.cycle == MG_CYCLE_FMG;
   if (H->d.precision != MG_MIXED) {
     if (fmg)
@@ -1074,9 +1085,9 @@ int cycle_map(mg_hierarchy* H, const Eq& e) {
       vcycle32(H, e, 0);
     H->fold_k32 = false;
     const float* ee[3] = {L0.e[0], L0.e[1], L0.e[2]};
-    launch_add_correction<float>(v, e.ncomp, L0.u, ee, H->st, e.zero_mean ? H->d_part : nullptr, NPARTS);
+    launch_add_correction<float>(v, e.ncomp, L0.u, ee, H->st, per_cycle_mean ? H->d_part : nullptr, NPARTS);
   }
-  if (e.zero_mean) launch_sub_mean(L0.v64, L0.u[0], H->d_part, NPARTS, H->st, H->d.precision == MG_MIXED);
+  if (per_cycle_mean) launch_sub_mean(L0.v64, L0.u[0], H->d_part, NPARTS, H->st, H->d.precision == MG_MIXED);
   if (e.kind == EQ_VEC) fill_all64(H, e, 0);
   return MG_OK;
 }
@@ -1553,6 +1564,7 @@ int run_loop_graph(mg_hierarchy* H, const Eq& e, double* ax, double* afp, double
   CK(cudaStreamSynchronize(H->st));
   const LoopState& S = *H->h_loop;
   const int cyc = S.cyc;
+  H->cycles_done = cyc;
   H->updates += (int64_t)cyc * g->updates;
   count_launch((int)(g->launches_pre + (uint64_t)cyc * g->launches));
   auto t1 = std::chrono::steady_clock::now();
@@ -1573,7 +1585,9 @@ int run_solve_body(mg_hierarchy* H, const Eq& e, mg_solve_report* rep);
 // A solve, then the timeout flag of the tensor-map staged sweeps (set when a
 // block gave up waiting for a staged plane and stopped early).
 int run_solve(mg_hierarchy* H, const Eq& e, mg_solve_report* rep) {
+  H->cycles_done = 0;
   const int st = run_solve_body(H, e, rep);
+  if (H->cycles_done > 0 && gauge_at_end(H, e)) launch_sub_mean(H->L[0].v64, H->L[0].u[0], H->d_part, NPARTS, H->st);
   if (H->maps_on) {
     unsigned long long flag = 0;
     CK(cudaMemcpyAsync(&flag, H->d_red + 7, sizeof(flag), cudaMemcpyDeviceToHost, H->st));
@@ -1659,6 +1673,7 @@ int run_solve_body(mg_hierarchy* H, const Eq& e, mg_solve_report* rep) {
         CK(cudaMemcpyAsync(ax + (long)c * stride, L0.u[c], sizeof(double) * L0.ng, cudaMemcpyDeviceToDevice,
                            H->st));
     if ((st = run_cycle_map(H, e))) return st;
+    ++H->cycles_done;
     bool mixed_step = false;
     if (m > 0) {
       // dF, dG of this cycle go to ring slot head (none on the first cycle)
@@ -2817,25 +2832,29 @@ int mg_clean_divB(mg_hierarchy* H, double* B[3], double* phi_out, int flags, mg_
   Level& L0 = H->L[0];
   const LevelView<double>& v = L0.v64;
   const double N = (double)L0.cells();
-  auto norms = [&](double* mx, double* l2) -> int {
-    CK(cudaMemsetAsync(H->d_red, 0, sizeof(unsigned long long), H->st));
-    launch_div_norms(v, L0.r[0], H->d_part, NPARTS, H->d_red, H->st);
-    std::vector<double> part(NPARTS);
-    CK(cudaMemcpyAsync(H->h_red, H->d_red, sizeof(unsigned long long), cudaMemcpyDeviceToHost, H->st));
-    CK(cudaMemcpyAsync(part.data(), H->d_part, sizeof(double) * NPARTS, cudaMemcpyDeviceToHost, H->st));
+  // divergence norms: max |div| in slot 4 (before the cleaning) or 6 (after)
+  // of d_red, the sum of squares in slot 5 or 0, read together at the end
+  double* const psq = H->d_part + NPARTS;
+  auto norms = [&](int after) {
+    if (curv) launch_div_norms(v, L0.r[0], psq, NPARTS, H->d_red + (after ? 6 : 4), H->st);
+    launch_total(psq, NPARTS, reinterpret_cast<double*>(H->d_red + (after ? 0 : 5)), H->st);
+  };
+  auto read_norms = [&](double* mb, double* lb, double* ma, double* la) -> int {
+    CK(cudaMemcpyAsync(H->h_red, H->d_red, sizeof(unsigned long long) * 7, cudaMemcpyDeviceToHost, H->st));
     CK(cudaStreamSynchronize(H->st));
-    double s = 0.0;
-    for (double x : part) s += x;
-    *mx = bits_to_double(H->h_red[0]);
-    *l2 = std::sqrt(s / N);
+    *mb = bits_to_double(H->h_red[4]);
+    *lb = std::sqrt(bits_to_double(H->h_red[5]) / N);
+    *ma = bits_to_double(H->h_red[6]);
+    *la = std::sqrt(bits_to_double(H->h_red[0]) / N);
     return MG_OK;
   };
+  CK(cudaMemsetAsync(H->d_red + 4, 0, sizeof(unsigned long long) * 3, H->st));
   // curvilinear grids: B into ghosted copies with the vector rules (outer
   // copies, origin / axis parities), then the divergence of Sec. 2.2
   auto vn = with_bc(v, MG_BC_NEUMANN);
-  auto div_into_r = [&]() {
+  auto div_into_r = [&](int after) {
     if (!curv) {
-      launch_div_central(v, Bd, L0.r[0], H->d_part, NPARTS, H->st);
+      launch_div_central(v, Bd, L0.r[0], H->d_part, NPARTS, H->st, psq, H->d_red + (after ? 6 : 4));
       return;
     }
     for (int c = 0; c < nd; ++c) {
@@ -2863,9 +2882,9 @@ int mg_clean_divB(mg_hierarchy* H, double* B[3], double* phi_out, int flags, mg_
     // class-major in r[2]), B -= grad Phi with mirrored Phi ghosts
     const int ncl = nd == 3 ? 8 : 4;
     const long M = (long)L0.cells() / ncl;
-    div_into_r();
+    div_into_r(0);
+    norms(0);
     launch_class_gather(v, L0.r[0], H->d_part, NPARTS / 8, L0.r[1], H->st);
-    if ((st = norms(&mb, &lb))) return st;
     CK(cudaMemsetAsync(L0.r[2], 0, sizeof(double) * L0.cells(), H->st));
     mg_solve_report agg{};
     for (int q = 0; q < ncl; ++q) {
@@ -2892,8 +2911,9 @@ int mg_clean_divB(mg_hierarchy* H, double* B[3], double* phi_out, int flags, mg_
       if (host && (s2 = stage_get(H, 3, &pd))) return s2;
     }
     launch_grad_update_exact(v, L0.r[2], Bd, pd, H->st);
-    div_into_r();
-    if ((s2 = norms(&ma, &la))) return s2;
+    div_into_r(1);
+    norms(1);
+    if ((s2 = read_norms(&mb, &lb, &ma, &la))) return s2;
     if (phi_out && host && (s2 = stage_out(H, pd, phi_out))) return s2;
     if (host)
       for (int c = 0; c < nd; ++c)
@@ -2907,12 +2927,12 @@ int mg_clean_divB(mg_hierarchy* H, double* B[3], double* phi_out, int flags, mg_
     }
     return st;
   }
-  div_into_r();
+  div_into_r(0);
   if (curv)
     launch_sub_wmean_into(v, L0.r[0], H->d_part, NPARTS, wsum, L0.f[0], H->st);
   else
     launch_sub_mean_into(v, L0.r[0], H->d_part, NPARTS, L0.f[0], H->st);
-  if ((st = norms(&mb, &lb))) return st;
+  norms(0);
   CK(cudaMemsetAsync(L0.u[0], 0, sizeof(double) * L0.ng, H->st));
   Eq e{MG_EQ_LIN, MG_BC_NEUMANN, 1, 1, false};
   st = run_solve(H, e, rep ? &rep->solve : nullptr);
@@ -2922,8 +2942,9 @@ int mg_clean_divB(mg_hierarchy* H, double* B[3], double* phi_out, int flags, mg_
   } else {
     launch_grad_update(v, L0.u[0], Bd, H->st);
   }
-  div_into_r();
-  int s2 = norms(&ma, &la);
+  div_into_r(1);
+  norms(1);
+  int s2 = read_norms(&mb, &lb, &ma, &la);
   if (s2) return s2;
   if (phi_out) {
     double* pd = phi_out;

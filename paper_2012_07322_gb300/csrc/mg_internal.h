@@ -197,6 +197,20 @@ void launch_prolong(const LevelView<T>& F, const LevelView<T>& C, T* u, const T*
 template <typename T>
 void launch_prolong3(const LevelView<T>& F, const LevelView<T>& C, T* const u[3], const T* const uH[3],
                      const T* const uhH[3], int ncomp, int vec, cudaStream_t st);
+// Streaming forms on 3D Cartesian levels (mg_cart.cu): the FP64 residual of
+// a linear equation without c on equal spacings, the FP32 residual-restriction
+// without c, the prolongation of one field.
+bool resid_cart_applies(const LevelView<double>& L);
+void launch_resid_cart(const LevelView<double>& L, const double* u, const double* f, double* r,
+                       unsigned long long* red, int weighted, cudaStream_t st, float* r32);
+template <typename T>
+bool transfer_cart_applies(const LevelView<T>& F);
+void launch_resid_restrict_cart(const LevelView<float>& F, const LevelView<float>& C, const float* e, const float* f,
+                                float* fc, float* ec, cudaStream_t st);
+void launch_prolong_cart(const LevelView<float>& F, const LevelView<float>& C, float* u, const float* uH,
+                         const float* uhH, cudaStream_t st);
+void launch_prolong_cart(const LevelView<double>& F, const LevelView<double>& C, double* u, const double* uH,
+                         const double* uhH, cudaStream_t st);
 // Down leg of the FP32 correction cycle: residual of (L - K) e = f (or the
 // vector operator) restricted into fc, K into Kc (if non-null), ec zeroed.
 void launch_resid_restrict32(const LevelView<float>& F, const LevelView<float>& C, int vec, float* const e[3],
@@ -245,7 +259,9 @@ void launch_xcfc_beta_rhs(const LevelView<double>& L, double* const X[3], const 
                           cudaStream_t st);
 void launch_scale_into(const LevelView<double>& L, const double* src, double a, double* dst, cudaStream_t st);
 void launch_div_central(const LevelView<double>& L, double* const B[3], double* div, double* part, int nparts,
-                        cudaStream_t st);
+                        cudaStream_t st, double* sq = nullptr, unsigned long long* mx = nullptr);
+// *out = the sum of nparts block sums.
+void launch_total(const double* part, int nparts, double* out, cudaStream_t st);
 void launch_div_norms(const LevelView<double>& L, const double* div, double* part, int nparts,
                       unsigned long long* red, cudaStream_t st);
 // Curvilinear divergence cleaning: divergence from ghosted B with weighted

@@ -7,6 +7,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "mg_cart.cuh"
 #include "mg_internal.h"
 #include "mg_kernels.cuh"
 
@@ -295,12 +296,28 @@ __device__ __forceinline__ RbCoef<T> rb_coef(const LevelView<T>& L, int i, int j
   return c;
 }
 
+// The FP64 update on equal spacings: uc + (f - c S) / D with the sum of the
+// stencil on the integer units (mg_cart.cuh): four FP64 operations instead of
+// thirteen (128^3 sweep: 103 us with the flux form).
+__device__ __forceinline__ double rb_uniform_value(double c, double iD0, double uc, double ue, double uw, double un,
+                                                   double us, double uu, double ud, double fv) {
+  double res;
+  if (!fix_residual(fix_decode(uc), fix_decode(ue), fix_decode(uw), fix_decode(un), fix_decode(us), fix_decode(uu),
+                    fix_decode(ud), c, fv, res)) {
+    double Lu = c * (ue - uc) - c * (uc - uw);
+    Lu += c * (un - 2.0 * uc + us);
+    Lu += c * (uu - 2.0 * uc + ud);
+    res = fv - Lu;
+  }
+  return uc + res * iD0;
+}
+
 // Newton-Gauss-Seidel update of cell (i0 + x, j0 + y, s): the arithmetic of
 // lap_scalar and scalar_update<EQ_LIN>.  The outer ghosts a boundary cell
 // needs sit in the staged planes already (rb_fix_ghosts; across the origin
 // or the axis, and at the poles, the flux coefficient is zero), so every
 // cell takes the same path; RING cells outside the domain are skipped.
-template <typename T, int G, int TX, bool HAS_C, bool RING>
+template <typename T, int G, int TX, bool HAS_C, bool RING, bool UNI = false>
 __device__ __forceinline__ void rb_relax(const LevelView<T>& L, const RbPlanes<T>& R, int i0, int j0, int x, int y,
                                          const RbCoef<T>& k, T iD0) {
   constexpr int BX = RbShape<TX>::BX;
@@ -310,6 +327,10 @@ __device__ __forceinline__ void rb_relax(const LevelView<T>& L, const RbPlanes<T
   }
   const int q = (x + RB_HX) + (y + RB_HY) * BX;
   const T uc = R.P[q];
+  if constexpr (UNI) {
+    R.P[q] = rb_uniform_value(k.cE, iD0, uc, R.P[q + 1], R.P[q - 1], R.P[q + BX], R.P[q - BX], R.Pu[q], R.Pd[q], R.F[q]);
+    return;
+  }
   T Lu = k.cE * (R.P[q + 1] - uc) - k.cW * (uc - R.P[q - 1]);
   if (G == SPH)
     Lu += k.cN * (R.P[q + BX] - uc) - k.cS * (uc - R.P[q - BX]);
@@ -343,9 +364,10 @@ __device__ __forceinline__ RbCoef<T> rb_pick(int q, const RbCoef<T>& a, const Rb
 
 // The same update from operand values: centre uc, neighbours e, w, n, s (in
 // i and j), up and down (in k), right-hand side fv and coefficient cv.
-template <typename T, int G, bool HAS_C>
+template <typename T, int G, bool HAS_C, bool UNI = false>
 __device__ __forceinline__ T rb_new_value(const RbCoef<T>& k, T iD0, T uc, T ue, T uw, T un, T us, T uu, T ud, T fv,
                                           T cv) {
+  if constexpr (UNI) return rb_uniform_value(k.cE, iD0, uc, ue, uw, un, us, uu, ud, fv);
   T Lu = k.cE * (ue - uc) - k.cW * (uc - uw);
   if (G == SPH)
     Lu += k.cN * (un - uc) - k.cS * (uc - us);
@@ -418,7 +440,7 @@ struct RbLaneCoef {
 // Red cells of plane s on the ring around the column (the lane cells are
 // relaxed from registers in k_sweep_rb).  On a Cartesian level every cell
 // has the lane cells' coefficients.
-template <typename T, int G, int TX, bool HAS_C>
+template <typename T, int G, int TX, bool HAS_C, bool UNI = false>
 __device__ __forceinline__ void rb_red_ring(const LevelView<T>& L, const RbPlanes<T>& R, int i0, int j0, int s,
                                             const RbLaneCoef<T, TX>& lc, T iD0) {
   // threads 64 .. 64 + RING - 1 (from warp 2 on: warps 0 and 1 fix the
@@ -442,7 +464,7 @@ __device__ __forceinline__ void rb_red_ring(const LevelView<T>& L, const RbPlane
       y = 2 * (t - 2 * HR - HC) + par;
     }
     if (G == CART) {
-      rb_relax<T, G, TX, HAS_C, true>(L, R, i0, j0, x, y, lc.k[0][0], iD0);
+      rb_relax<T, G, TX, HAS_C, true, UNI>(L, R, i0, j0, x, y, lc.k[0][0], iD0);
     } else {
       const int ic = min(max(i0 + x, 0), L.n0 - 1), jc = min(max(j0 + y, 0), L.n1 - 1);
       rb_relax<T, G, TX, HAS_C, true>(L, R, i0, j0, x, y, rb_coef<T, G>(L, ic, jc), iD0);
@@ -460,7 +482,7 @@ __host__ __device__ constexpr bool rb_tma() {
   return sizeof(T) == 4 && G == CART && TX == 128;
 }
 
-template <typename T, int G, int TX, bool HAS_C>
+template <typename T, int G, int TX, bool HAS_C, bool UNI = false>
 __global__ void __launch_bounds__(RbShape<TX>::THREADS, TX == 128 ? (G == CART ? 2 : 1) : (sizeof(T) == 4 ? 4 : 2))
     k_sweep_rb(LevelView<T> L, const T* __restrict__ uin, T* __restrict__ uout, const T* __restrict__ f,
                const T* __restrict__ c, int zc, const __grid_constant__ SweepMaps M) {
@@ -619,7 +641,7 @@ __global__ void __launch_bounds__(RbShape<TX>::THREADS, TX == 128 ? (G == CART ?
           const int o = po + 64 * h + Q;
           const T uc = Q ? r0[h].y : r0[h].x, other = Q ? r0[h].x : r0[h].y;
           const T ue = Q ? P[o + 1] : other, uw = Q ? other : P[o - 1];
-          const T v = rb_new_value<T, G, HAS_C>(G == CART ? lc.k[0][0] : lc.k[h][Q], iD0, uc, ue, uw, P[o + BX],
+          const T v = rb_new_value<T, G, HAS_C, UNI>(G == CART ? lc.k[0][0] : lc.k[h][Q], iD0, uc, ue, uw, P[o + BX],
                                                 P[o - BX], Q ? rp1[h].y : rp1[h].x, Q ? rm1[h].y : rm1[h].x, F[o],
                                                 HAS_C ? Cc[o] : T(0));
           P[o] = v;
@@ -634,7 +656,7 @@ __global__ void __launch_bounds__(RbShape<TX>::THREADS, TX == 128 ? (G == CART ?
       else
         red(std::integral_constant<int, 0>{});
       const RbPlanes<T> R{su + bd * BP, P, su + bu * BP, F, Cc};
-      rb_red_ring<T, G, TX, HAS_C>(L, R, i0, j0, s, lc, iD0);
+      rb_red_ring<T, G, TX, HAS_C, UNI>(L, R, i0, j0, s, lc, iD0);
     }
     const int sb = s - 1;
     if (sb >= z0) {
@@ -653,7 +675,7 @@ __global__ void __launch_bounds__(RbShape<TX>::THREADS, TX == 128 ? (G == CART ?
           const int o = po + 64 * h + Q;
           const T uc = Q ? rm1[h].y : rm1[h].x, other = Q ? rm1[h].x : rm1[h].y;
           const T ue = Q ? P[o + 1] : other, uw = Q ? other : P[o - 1];
-          const T v = rb_new_value<T, G, HAS_C>(G == CART ? lc.k[0][0] : lc.k[h][Q], iD0, uc, ue, uw, P[o + BX],
+          const T v = rb_new_value<T, G, HAS_C, UNI>(G == CART ? lc.k[0][0] : lc.k[h][Q], iD0, uc, ue, uw, P[o + BX],
                                                 P[o - BX], Q ? r0[h].y : r0[h].x, Q ? rm2[h].y : rm2[h].x, F[o],
                                                 HAS_C ? Cc[o] : T(0));
           if (Q)
@@ -1292,6 +1314,8 @@ template <typename T, int G, int TX, bool HAS_C>
 static void set_fused_capacity(int sms) {
   const size_t smem = fused_sweep_smem<T, TX>(HAS_C);
   cudaFuncSetAttribute(k_sweep_rb<T, G, TX, HAS_C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if constexpr (sizeof(T) == 8 && G == CART && !HAS_C)
+    cudaFuncSetAttribute(k_sweep_rb<T, G, TX, HAS_C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sweep_rb<T, G, TX, HAS_C>, RbShape<TX>::THREADS, smem) !=
           cudaSuccess ||
@@ -1357,6 +1381,13 @@ static void launch_rb(const LevelView<T>& L, const T* uin, T* uout, const T* f, 
   SweepMaps none;
   std::memset(&none, 0, sizeof(none));
   const SweepMaps& M = (rb_tma<T, G, TX>() && maps) ? *maps : none;
+  if constexpr (sizeof(T) == 8 && G == CART) {
+    if (!c && L.ih0s == L.ih1s && L.ih1s == L.ih2s) {
+      launch_k(k_sweep_rb<T, G, TX, false, true>, g, NT, fused_sweep_smem<T, TX>(false), st, L, uin, uout, f,
+               nullptr, zc, M);
+      return;
+    }
+  }
   if (c)
     launch_k(k_sweep_rb<T, G, TX, true>, g, NT, fused_sweep_smem<T, TX>(true), st, L, uin, uout, f, c, zc, M);
   else
@@ -1517,6 +1548,12 @@ template <typename T>
 void launch_residual_scalar(const LevelView<T>& L, int kind, const T* u, const T* f, const T* s0,
                             const T* s1, T* r, unsigned long long* red, int weighted, cudaStream_t st, float* r32,
                             float* k32) {
+  if constexpr (sizeof(T) == 8) {
+    if (kind == EQ_LIN && !s1 && resid_cart_applies(L)) {
+      launch_resid_cart(L, u, f, r, red, weighted, st, r32);
+      return;
+    }
+  }
   count_launch();
   if (L.three && ncells(L) >= RES_KZ_CELLS) {
     dim3 b = block_for(L.three), g = grid_cells(L, b);
@@ -1590,6 +1627,10 @@ void launch_fill_ghosts3(const LevelView<T>& L, T* const u[3], int ncomp, int ve
 template <typename T>
 void launch_prolong3(const LevelView<T>& F, const LevelView<T>& C, T* const u[3], const T* const uH[3],
                      const T* const uhH[3], int ncomp, int vec, cudaStream_t st) {
+  if (ncomp == 1 && !vec && transfer_cart_applies(F)) {
+    launch_prolong_cart(F, C, u[0], uH[0], uhH ? uhH[0] : nullptr, st);
+    return;
+  }
   count_launch();
   const dim3 b = sizeof(T) == 8 ? cells_block(F) : block_for(F.three);
   const dim3 g = grid_cells(F, b);
@@ -1604,6 +1645,10 @@ void launch_prolong3(const LevelView<T>& F, const LevelView<T>& C, T* const u[3]
 void launch_resid_restrict32(const LevelView<float>& F, const LevelView<float>& C, int vec, float* const e[3],
                              float* const f[3], const float* K, float* const fc[3], float* const ec[3], float* Kc,
                              cudaStream_t st) {
+  if (!vec && !K && transfer_cart_applies(F)) {
+    launch_resid_restrict_cart(F, C, e[0], f[0], fc[0], ec[0], st);
+    return;
+  }
   count_launch();
   const int nc = vec ? 3 : 1;
   dim3 b = block_for(F.three), g = grid_cells(F, b);

@@ -103,32 +103,61 @@ __global__ void k_scale_into(LevelView<double> L, const double* __restrict__ src
 // B is in the caller's ghost-free layout; its ghosts are copies of the
 // boundary cells (zero normal gradient).
 
-__global__ void k_div_central(LevelView<double> L, const double* __restrict__ B0,
-                              const double* __restrict__ B1, const double* __restrict__ B2,
-                              double* __restrict__ div, double* __restrict__ part) {
+// Sum of nparts partial sums, to every thread of a 256-thread block (fixed
+// order).
+__device__ __forceinline__ double block_total(const double* __restrict__ part, int nparts) {
+  __shared__ double tot[33];
+  double s = 0.0;
+  for (int q = threadIdx.x; q < nparts; q += blockDim.x) s += part[q];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) tot[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double t = warp_sum(threadIdx.x < (blockDim.x >> 5) ? tot[threadIdx.x] : 0.0);
+    if (threadIdx.x == 0) tot[32] = t;
+  }
+  __syncthreads();
+  return tot[32];
+}
+
+// Central divergence; part gets the block sums of div, and with sq non-null
+// sq those of div^2 and mx (atomically) max |div|: the norms cost no pass of
+// their own (256^3: 282 us and 104 us for the norms before).
+__global__ void __launch_bounds__(256)
+    k_div_central(LevelView<double> L, const double* __restrict__ B0, const double* __restrict__ B1,
+                  const double* __restrict__ B2, double* __restrict__ div, double* __restrict__ part,
+                  double* __restrict__ sq, unsigned long long* __restrict__ mx) {
   pdl_entry();
-  __shared__ double sm[32];
-  const long n = (long)L.n0 * L.n1 * L.n2;
-  const long s1 = L.n0, s2 = (long)L.n0 * L.n1;
+  const unsigned n = (unsigned)L.n0 * L.n1 * L.n2, s1 = L.n0, s2 = L.n0 * L.n1;
   const double c0 = 0.5 / L.h0, c1 = 0.5 / L.h1, c2 = 0.5 / L.h2;
-  double acc = 0.0;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-    int i, j, k;
-    L.cell(q, i, j, k);
+  double acc = 0.0, ss = 0.0;
+  unsigned long long m[1] = {0ULL};
+#pragma unroll 4
+  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+    const int i = q & (L.n0 - 1), jk = q >> L.ln0, j = jk & (L.n1 - 1), k = jk >> L.ln1;
     double d = (B0[i < L.n0 - 1 ? q + 1 : q] - B0[i > 0 ? q - 1 : q]) * c0 +
                (B1[j < L.n1 - 1 ? q + s1 : q] - B1[j > 0 ? q - s1 : q]) * c1;
     if (L.three) d += (B2[k < L.n2 - 1 ? q + s2 : q] - B2[k > 0 ? q - s2 : q]) * c2;
     div[L.idx(i, j, k)] = d;
     acc += d;
+    if (sq) {
+      ss += d * d;
+      m[0] = umax64(m[0], abs_bits(d));
+    }
   }
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
+  block_sum_to(acc, part);
+  if (!sq) return;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) t += sm[w];
-    part[blockIdx.x] = t;
-  }
+  block_sum_to(ss, sq);
+  __syncthreads();
+  block_max_bits<1>(m, mx);
+}
+
+// *out = the sum of nparts partial sums (one block).
+__global__ void k_total(const double* __restrict__ part, int nparts, double* __restrict__ out) {
+  pdl_entry();
+  const double t = block_total(part, nparts);
+  if (threadIdx.x == 0) *out = t;
 }
 
 // max |div| -> red[0] (atomic), sum div^2 -> part (per block).
@@ -162,13 +191,9 @@ __global__ void k_div_norms(LevelView<double> L, const double* __restrict__ div,
 __global__ void k_sub_mean_into(LevelView<double> L, const double* __restrict__ div,
                                 const double* __restrict__ part, int nparts, double* __restrict__ b) {
   pdl_entry();
-  __shared__ double mean;
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int q = 0; q < nparts; ++q) s += part[q];
-    mean = s / ((double)L.n0 * L.n1 * L.n2);
-  }
-  __syncthreads();
+  // the partial sums by a block tree (one thread adding 1024 of them in turn
+  // took 34 us of dependent FP64 additions)
+  const double mean = block_total(part, nparts) / ((double)L.n0 * L.n1 * L.n2);
   const long n = (long)L.n0 * L.n1 * L.n2;
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
     int i, j, k;
@@ -182,11 +207,11 @@ __global__ void k_sub_mean_into(LevelView<double> L, const double* __restrict__ 
 __global__ void k_grad_update(LevelView<double> L, const double* __restrict__ phi, double* __restrict__ B0,
                               double* __restrict__ B1, double* __restrict__ B2) {
   pdl_entry();
-  const long n = (long)L.n0 * L.n1 * L.n2;
+  const unsigned n = (unsigned)L.n0 * L.n1 * L.n2;
   const double c0 = 0.5 / L.h0, c1 = 0.5 / L.h1, c2 = 0.5 / L.h2;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-    int i, j, k;
-    L.cell(q, i, j, k);
+#pragma unroll 4
+  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+    const int i = q & (L.n0 - 1), jk = q >> L.ln0, j = jk & (L.n1 - 1), k = jk >> L.ln1;
     const long p = L.idx(i, j, k);
     const double pc = phi[p];
     B0[q] -= ((i < L.n0 - 1 ? phi[p + 1] : pc) - (i > 0 ? phi[p - 1] : pc)) * c0;
@@ -240,13 +265,7 @@ __global__ void k_sub_wmean_into(LevelView<double> L, const double* __restrict__
                                  const double* __restrict__ part, int nparts, double wsum,
                                  double* __restrict__ b) {
   pdl_entry();
-  __shared__ double mean;
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int q = 0; q < nparts; ++q) s += part[q];
-    mean = s / wsum;
-  }
-  __syncthreads();
+  const double mean = block_total(part, nparts) / wsum;
   const long n = (long)L.n0 * L.n1 * L.n2;
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
     int i, j, k;
@@ -347,9 +366,14 @@ void launch_scale_into(const LevelView<double>& L, const double* src, double a, 
 }
 
 void launch_div_central(const LevelView<double>& L, double* const B[3], double* div, double* part, int nparts,
-                        cudaStream_t st) {
+                        cudaStream_t st, double* sq, unsigned long long* mx) {
   count_launch();
-  launch_k(k_div_central, nparts, 256, 0, st, L, B[0], B[1], B[2], div, part);
+  launch_k(k_div_central, nparts, 256, 0, st, L, B[0], B[1], B[2], div, part, sq, mx);
+}
+
+void launch_total(const double* part, int nparts, double* out, cudaStream_t st) {
+  count_launch();
+  launch_k(k_total, 1, 256, 0, st, part, nparts, out);
 }
 
 void launch_div_norms(const LevelView<double>& L, const double* div, double* part, int nparts,
@@ -432,14 +456,8 @@ __global__ void k_class_sums(LevelView<double> L, ClassGrid G, const double* __r
 __global__ void k_class_gather(LevelView<double> L, ClassGrid G, const double* __restrict__ div,
                                const double* __restrict__ part, int nparts, double* __restrict__ dst) {
   pdl_entry();
-  __shared__ double mean;
   const int s = blockIdx.y;
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int q = 0; q < nparts; ++q) t += part[s * nparts + q];
-    mean = t / (double)G.M;
-  }
-  __syncthreads();
+  const double mean = block_total(part + (long)s * nparts, nparts) / (double)G.M;
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < G.M; r += (long)gridDim.x * blockDim.x) {
     int i, j, k;
     G.fine(s, r, L.three, i, j, k);
