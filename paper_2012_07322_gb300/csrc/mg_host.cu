@@ -725,7 +725,46 @@ void fas_up64(mg_hierarchy* H, const Eq& e, int l) {
   if (e.kind == EQ_VEC) fill_all64(H, e, l);
 }
 
+// First level of the cluster-launched part of a scalar FP64 cycle (mg_fas.cu): at
+// most FAS_CLUSTER_CELLS cells, at least two levels, a coarsest level its
+// solves take; nlev when there is none.
+int fas_cluster_level(const mg_hierarchy* H, const Eq& e) {
+  if (e.kind == EQ_VEC || !fas_cycle_available() || H->L[H->nlev - 1].cells() > CS_CELLS) return H->nlev;
+  for (int l = std::max(0, H->nlev - FAS_MAX); l + 1 < H->nlev; ++l)
+    if (H->L[l].cells() <= FAS_CLUSTER_CELLS) return l;
+  return H->nlev;
+}
+
+// vcycle64 from level l0 down in one launch.
+void cluster_vcycle64(mg_hierarchy* H, const Eq& e, int l0) {
+  FasCycle P{};
+  P.nl = H->nlev - l0;
+  P.nu1 = H->d.nu1;
+  P.nu2 = H->d.nu2;
+  P.coarse_sweeps = COARSE_SWEEPS;
+  P.solo_from = P.nl - 1;
+  for (int q = P.nl - 1; q >= 0; --q) {
+    const int l = l0 + q;
+    Level& L = H->L[l];
+    FasLevel& F = P.lv[q];
+    F.v = with_bc(L.v64, e.bc);
+    F.u = L.u[0];
+    F.uh = L.uh[0];
+    F.f = const_cast<double*>(fptr(H, e, l, 0));
+    F.r = L.r[0];
+    F.s0 = s0ptr(H, e, l);
+    F.s1 = s1ptr(H, e, l);
+    if (L.cells() <= FAS_SOLO_CELLS) P.solo_from = q;
+    if (q + 1 < P.nl) H->updates += (int64_t)(H->d.nu1 + H->d.nu2) * L.cells();
+  }
+  launch_fas_cycle(P, H->d.geom, e.kind, H->st);
+}
+
 void vcycle64(mg_hierarchy* H, const Eq& e, int l) {
+  if (l >= fas_cluster_level(H, e)) {
+    cluster_vcycle64(H, e, l);
+    return;
+  }
   if (l == H->nlev - 1) {
     coarse64(H, e, l);
     return;
@@ -2236,6 +2275,7 @@ int mg_create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, mg_hierarch
   init_fused_sweep_attributes<double>();
   init_fused_sweep_attributes<float>();
   init_block_cycle_attributes();
+  init_fas_attributes();
   const int three = H->d.ndim == 3;
   for (int l = 0; l < H->nlev; ++l) {
     Level& L = H->L[l];

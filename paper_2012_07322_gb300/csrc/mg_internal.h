@@ -231,6 +231,26 @@ void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double*
                             cudaStream_t st);
 void launch_coarse_vec_dense(const LevelView<double>& L, double* const V[3], const double* const f[3],
                              const double* A, const double* invD, int n, int max_sweeps, cudaStream_t st);
+
+// The FP64 FAS V-cycle of a scalar equation on small levels in one cluster launch (mg_fas.cu):
+// levels lv[0 .. nl - 1], the last the coarsest; from solo_from on (at most
+// nl - 1) block 0 alone works.
+constexpr int FAS_MAX = 8;
+constexpr long FAS_CLUSTER_CELLS = 4096;  // the cycle runs from the first level this small
+constexpr long FAS_SOLO_CELLS = 128;
+struct FasLevel {
+  LevelView<double> v;  // boundary rule applied
+  double *u, *uh, *f, *r;
+  const double *s0, *s1;
+};
+struct FasCycle {
+  int nl, solo_from, nu1, nu2, coarse_sweeps;
+  FasLevel lv[FAS_MAX];
+};
+void init_fas_attributes();   // once a device is current, before any capture
+bool fas_cycle_available();
+void launch_fas_cycle(const FasCycle& P, int geom, int kind, cudaStream_t st);
+constexpr int CS_CELLS = 64;  // scalar coarsest levels the cycle solves
 template <typename T>
 void launch_coarse_vec(const LevelView<T>& L, T* V[3], const T* const f[3], int max_sweeps, cudaStream_t st);
 // u -= mean(u) over the interior (the Neumann gauge); the nparts block sums
