@@ -29,7 +29,7 @@ __device__ __forceinline__ double amr_volume(const LevelView<double>& L, int i, 
   if (L.geom == CYL) v *= L.xc0(i);
   if (L.geom == SPH) {
     const double r = L.xc0(i);
-    v *= r * r * sin(L.xc1(j));
+    v *= r * r * L.TJ(TJ_S, j);
   }
   return v;
 }
@@ -44,7 +44,7 @@ __device__ __forceinline__ double amr_area(const LevelView<double>& L, int d, in
   }
   if (d == 0) {
     const double rf = L.lo0 + (sd > 0 ? i + 1 : i) * L.h0;
-    return rf * rf * sin(L.xc1(j)) * L.h1 * h2;
+    return rf * rf * L.TJ(TJ_S, j) * L.h1 * h2;
   }
   if (d == 1) {
     // sin at the face, exactly zero on the poles
@@ -52,7 +52,7 @@ __device__ __forceinline__ double amr_area(const LevelView<double>& L, int d, in
     const double s = (jf == 0 || jf == L.n1) && L.lo1 == 0.0 ? 0.0 : sin(L.lo1 + jf * L.h1);
     return s * L.h0 * h2;
   }
-  return L.h0 * L.h1 / sin(L.xc1(j));
+  return L.h0 * L.h1 / L.TJ(TJ_S, j);
 }
 
 // ------------------------------------------------------ coarse-fine ghosts
@@ -122,11 +122,13 @@ __device__ __forceinline__ bool amr_face(long& g, int nd, long f0, long f1, long
   return false;
 }
 
-// One thread per coarse-fine ghost of the patch, faces enumerated as in
-// amr_face, the cells of a face dimension-0 fastest over the patch's
-// tangential extent.
-__global__ void k_amr_cf_ghosts(LevelView<double> Pv, LevelView<double> B, AmrBox box, double* __restrict__ up,
-                                const double* __restrict__ ub) {
+// The base's share (8/15 u~) of every coarse-fine ghost of the patch into
+// the ghost's place in gt: it stays while the base does; the patch's share is
+// added where a cell reads its ghost (amr_cf_ghost).  One thread per ghost,
+// faces enumerated as in amr_face, the cells of a face dimension-0 fastest
+// over the patch's tangential extent.
+__global__ void k_amr_cf_base(LevelView<double> Pv, LevelView<double> B, AmrBox box, double* __restrict__ gt,
+                              const double* __restrict__ ub) {
   pdl_entry();
   const int nd = Pv.three ? 3 : 2;
   const long n0 = Pv.n0, n1 = Pv.n1, n2 = Pv.three ? Pv.n2 : 1;
@@ -163,40 +165,118 @@ __global__ void k_amr_cf_ghosts(LevelView<double> Pv, LevelView<double> B, AmrBo
   }
   if (!Pv.three) t2 = 0.0;
   const double ut = amr_tangential(B, ub, d, I, J, K, t0, t1, t2);
-  // the ghost, the first and the second patch cell inward along d
-  const long pg = Pv.idx(i + (d == 0) * s, j + (d == 1) * s, k + (d == 2) * s);
-  const long p1 = Pv.idx(i, j, k);
-  const long p2 = Pv.idx(i - (d == 0) * s, j - (d == 1) * s, k - (d == 2) * s);
-  up[pg] = (8.0 / 15.0) * ut + (2.0 / 3.0) * up[p1] - (1.0 / 5.0) * up[p2];
+  gt[Pv.idx(i + (d == 0) * s, j + (d == 1) * s, k + (d == 2) * s)] = (8.0 / 15.0) * ut;
+}
+
+// A coarse-fine ghost: the quadratic through the base solution and the two
+// patch cells inward, u1 the cell next to the ghost and u2 behind it.
+__device__ __forceinline__ double amr_cf_ghost(double gt, double u1, double u2) {
+  return gt + (2.0 / 3.0) * u1 - (1.0 / 5.0) * u2;
 }
 
 // ------------------------------------------------------------ patch level
 
-// Scalar operator of the patch with every neighbour read from memory (the
-// ghosts are materialised: boundary rules or coarse-fine values); D gets
-// dL/du at the cell, ghosts held fixed.
-template <int G, int KIND>
-__device__ __forceinline__ double amr_op(const LevelView<double>& L, const double* __restrict__ u,
-                                         const double* __restrict__ s0, const double* __restrict__ s1, int i, int j,
-                                         long p, double& D) {
-  double Lu = lap_ghosted<double, G>(L, u, i, j, p, D);
-  if (KIND == EQ_PSI) {
-    const double ip = 1.0 / (1.0 + u[p]);
-    const double ip2 = ip * ip;
-    const double ip7 = ip2 * ip2 * ip2 * ip;
-    const double a = 2.0 * PI_D * s0[p], b = s1[p];
-    Lu += a * ip + 0.125 * b * ip7;
-    D -= a * ip2 + 0.875 * b * ip7 * ip;
-  } else if (s1) {
-    Lu -= s1[p] * u[p];
-    D -= s1[p];
+// Neighbours of a patch cell: coarse-fine ghosts from gt and the patch cells
+// inward, outer ghosts from the boundary rule, the cell itself across the
+// origin and at the poles (their face areas vanish), phi wrapped.  Evaluated
+// where they are read, so no launch refills ghosts between colour passes (16
+// fills and 8 coarse-fine fills per cycle before, ~2.5 us each).
+template <int G>
+__device__ __forceinline__ Nb6<double> amr_neighbours(const LevelView<double>& L, int cf,
+                                                      const double* __restrict__ u, const double* __restrict__ gt,
+                                                      int i, int j, int k, long p, double uc) {
+  Nb6<double> nb;
+  const long sx = L.sx, sy = L.sy;
+  if (i < L.n0 - 1)
+    nb.e = u[p + 1];
+  else
+    nb.e = amr_cf(cf, 0, 1) ? amr_cf_ghost(gt[p + 1], uc, u[p - 1]) : outer_factor(L, L.n0, j, k, L.n0 - 1, j, k) * uc;
+  if (i > 0)
+    nb.w = u[p - 1];
+  else if (amr_cf(cf, 0, -1))
+    nb.w = amr_cf_ghost(gt[p - 1], uc, u[p + 1]);
+  else
+    nb.w = G == CART ? outer_factor(L, -1, j, k, 0, j, k) * uc : uc;
+  if (j < L.n1 - 1)
+    nb.n = u[p + sx];
+  else if (G == SPH)
+    nb.n = uc;
+  else
+    nb.n = amr_cf(cf, 1, 1) ? amr_cf_ghost(gt[p + sx], uc, u[p - sx])
+                            : outer_factor(L, i, L.n1, k, i, L.n1 - 1, k) * uc;
+  if (j > 0)
+    nb.s = u[p - sx];
+  else if (G == SPH)
+    nb.s = uc;
+  else
+    nb.s = amr_cf(cf, 1, -1) ? amr_cf_ghost(gt[p - sx], uc, u[p + sx]) : outer_factor(L, i, -1, k, i, 0, k) * uc;
+  nb.up = nb.dn = uc;
+  if (L.three) {
+    if (k < L.n2 - 1)
+      nb.up = u[p + sy];
+    else if (G != CART)
+      nb.up = u[p - (long)(L.n2 - 1) * sy];
+    else
+      nb.up = amr_cf(cf, 2, 1) ? amr_cf_ghost(gt[p + sy], uc, u[p - sy])
+                               : outer_factor(L, i, j, L.n2, i, j, L.n2 - 1) * uc;
+    if (k > 0)
+      nb.dn = u[p - sy];
+    else if (G != CART)
+      nb.dn = u[p + (long)(L.n2 - 1) * sy];
+    else
+      nb.dn = amr_cf(cf, 2, -1) ? amr_cf_ghost(gt[p - sy], uc, u[p + sy]) : outer_factor(L, i, j, -1, i, j, 0) * uc;
+  }
+  return nb;
+}
+template <int G>
+__device__ __noinline__ Nb6<double> amr_edge_neighbours(const LevelView<double>& L, int cf,
+                                                        const double* __restrict__ u, const double* __restrict__ gt,
+                                                        int i, int j, int k, long p, double uc) {
+  return amr_neighbours<G>(L, cf, u, gt, i, j, k, p, uc);
+}
+
+// Flux-form Laplacian of the patch and its diagonal (as lap_scalar).
+template <int G>
+__device__ __forceinline__ double amr_lap(const LevelView<double>& L, int cf, const double* __restrict__ u,
+                                          const double* __restrict__ gt, int i, int j, int k, long p, double uc,
+                                          double& D) {
+  Nb6<double> nb;
+  if (i > 0 && i < L.n0 - 1 && j > 0 && j < L.n1 - 1 && (!L.three || (k > 0 && k < L.n2 - 1))) {
+    nb.e = u[p + 1];
+    nb.w = u[p - 1];
+    nb.n = u[p + L.sx];
+    nb.s = u[p - L.sx];
+    nb.up = L.three ? u[p + L.sy] : uc;
+    nb.dn = L.three ? u[p - L.sy] : uc;
+  } else {
+    nb = amr_edge_neighbours<G>(L, cf, u, gt, i, j, k, p, uc);
+  }
+  const double cE = L.TI(TI_CE, i), cW = L.TI(TI_CW, i);
+  double Lu = cE * (nb.e - uc) - cW * (uc - nb.w);
+  D = -(cE + cW);
+  if (G == SPH) {
+    const double ir2 = L.TI(TI_IX2, i);
+    const double tN = L.TJ(TJ_TN, j), tS = L.TJ(TJ_TS, j);
+    Lu += ir2 * (tN * (nb.n - uc) - tS * (uc - nb.s));
+    D -= ir2 * (tN + tS);
+  } else {
+    Lu += L.ih1s * (nb.n - 2.0 * uc + nb.s);
+    D -= 2.0 * L.ih1s;
+  }
+  if (L.three) {
+    const double c = (G == CART) ? L.ih2s : (G == CYL ? L.TI(TI_PHI, i) : L.TI(TI_IX2, i) * L.TJ(TJ_PF, j));
+    Lu += c * (nb.up - 2.0 * uc + nb.dn);
+    D -= 2.0 * c;
   }
   return Lu;
 }
 
+// One colour of the patch's red-black sweep; eq. psi with one division, as
+// scalar_update.
 template <int G, int KIND>
-__global__ void k_amr_smooth(LevelView<double> L, double* __restrict__ u, const double* __restrict__ f,
-                             const double* __restrict__ s0, const double* __restrict__ s1, int colour) {
+__global__ void k_amr_smooth(LevelView<double> L, int cf, double* u, const double* __restrict__ gt,
+                             const double* __restrict__ f, const double* __restrict__ s0,
+                             const double* __restrict__ s1, int colour) {
   pdl_entry();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -204,16 +284,27 @@ __global__ void k_amr_smooth(LevelView<double> L, double* __restrict__ u, const 
   if (2 * t >= L.n0 || j >= L.n1 || k >= L.n2) return;
   const int i = 2 * t + ((j + k + colour) & 1);
   const long p = L.idx(i, j, k);
+  const double uc = u[p];
   double D;
-  const double Lu = amr_op<G, KIND>(L, u, s0, s1, i, j, p, D);
-  u[p] = u[p] - (Lu - f[p]) / D;
+  const double lap = amr_lap<G>(L, cf, u, gt, i, j, k, p, uc, D);
+  if (KIND == EQ_PSI) {
+    const double q = 1.0 + uc, q2 = q * q, q4 = q2 * q2, q6 = q4 * q2, q8 = q4 * q4;
+    const double a = 2.0 * PI_D * s0[p], b = s1[p];
+    const double num = (lap - f[p]) * q8 + a * q6 * q + 0.125 * b * q;
+    const double den = D * q8 - a * q6 - 0.875 * b;
+    u[p] = uc - num / den;
+  } else {
+    const double c = s1 ? s1[p] : 0.0;
+    u[p] = uc - (lap - c * uc - f[p]) / (D - c);
+  }
 }
 
 // r = f - L(u) on the patch (apply: r = L(u)); red (nullable) gets max |r|
 // (slot 0), max |w r| (slot 1) and max |w S| (slot 2), w = r^2 sin(theta) /
 // R / 1, S the source as the paper writes the right-hand side.
 template <int G, int KIND>
-__global__ void k_amr_patch_resid(LevelView<double> L, const double* __restrict__ u, const double* __restrict__ f,
+__global__ void k_amr_patch_resid(LevelView<double> L, int cf, const double* __restrict__ u,
+                                  const double* __restrict__ gt, const double* __restrict__ f,
                                   const double* __restrict__ s0, const double* __restrict__ s1,
                                   double* __restrict__ r, unsigned long long* red, int apply) {
   pdl_entry();
@@ -223,23 +314,26 @@ __global__ void k_amr_patch_resid(LevelView<double> L, const double* __restrict_
   unsigned long long m[3] = {0ULL, 0ULL, 0ULL};
   if (i < L.n0 && j < L.n1 && k < L.n2) {
     const long p = L.idx(i, j, k);
-    double D;
-    const double Lu = amr_op<G, KIND>(L, u, s0, s1, i, j, p, D);
-    const double fv = f ? f[p] : 0.0;
+    const double uc = u[p], fv = f ? f[p] : 0.0;
+    double D, S;
+    double Lu = amr_lap<G>(L, cf, u, gt, i, j, k, p, uc, D);
+    if (KIND == EQ_PSI) {
+      const double ip = 1.0 / (1.0 + uc), ip2 = ip * ip;
+      S = -2.0 * PI_D * s0[p] * ip - 0.125 * s1[p] * (ip2 * ip2 * ip2 * ip);
+      Lu -= S;
+    } else {
+      const double cu = s1 ? s1[p] * uc : 0.0;
+      S = fv + cu;
+      Lu -= cu;
+    }
     const double rv = fv - Lu;
     if (r) r[p] = apply ? Lu : rv;
-    double S;
-    if (KIND == EQ_PSI) {
-      const double ip = 1.0 / (1.0 + u[p]);
-      const double ip2 = ip * ip;
-      S = -2.0 * PI_D * s0[p] * ip - 0.125 * s1[p] * (ip2 * ip2 * ip2 * ip);
-    } else {
-      S = fv + (s1 ? s1[p] * u[p] : 0.0);
+    if (red) {
+      const double w = norm_weight(L, i, j);
+      m[0] = abs_bits(rv);
+      m[1] = abs_bits(w * rv);
+      m[2] = abs_bits(w * S);
     }
-    const double w = norm_weight(L, i, j);
-    m[0] = abs_bits(rv);
-    m[1] = abs_bits(w * rv);
-    m[2] = abs_bits(w * S);
   }
   if (red) block_max_bits<3>(m, red);
 }
@@ -274,11 +368,12 @@ __global__ void k_amr_restrict(LevelView<double> Pv, LevelView<double> B, AmrBox
 }
 
 // The composite operator minus the base operator at the uncovered base cells
-// next to the patch (corr zero elsewhere; zeroed before): one thread per
+// next to the patch (corr zero elsewhere; zeroed once): one thread per
 // coarse cell of a coarse-fine face, faces enumerated as in amr_face over
 // the box's tangential extent.
 __global__ void k_amr_flux_corr(LevelView<double> Pv, LevelView<double> B, AmrBox box, const double* __restrict__ up,
-                                const double* __restrict__ ub, double* __restrict__ corr) {
+                                const double* __restrict__ gt, const double* __restrict__ ub,
+                                double* __restrict__ corr) {
   pdl_entry();
   const int nd = B.three ? 3 : 2;
   const int a0 = box.a[0], a1 = box.a[1], a2 = box.a[2], b0 = box.b[0], b1 = box.b[1], b2 = box.b[2];
@@ -323,8 +418,9 @@ __global__ void k_amr_flux_corr(LevelView<double> Pv, LevelView<double> B, AmrBo
       if (!Pv.three) fk = 0;
       const long pf = Pv.idx(fi, fj, fk);
       const long pg = Pv.idx(fi + (d == 0) * s, fj + (d == 1) * s, fk + (d == 2) * s);
+      const long p2 = 2 * pf - pg;  // the patch cell behind
       const double Af = amr_area(Pv, d, s, fi, fj);
-      fsum += Af * (up[pf] - up[pg]) / hp;
+      fsum += Af * (up[pf] - amr_cf_ghost(gt[pg], up[pf], up[p2])) / hp;
     }
   corr[B.idx(QI, QJ, QK)] = (fsum - Ac * Dc) / amr_volume(B, QI, QJ);
 }
@@ -386,11 +482,12 @@ __global__ void k_amr_base(LevelView<double> B, AmrBox box, const double* __rest
   if (mode == 1) block_max_bits<3>(m, red);
 }
 
-// Kwak prolongation (Sec. 2.7.3) of the base change e (ghosts filled with
-// the homogeneous rules) onto the patch: parent a + (i, j, k) / 2 and, per
-// dimension, the parent's neighbour on the fine cell's side.
-__global__ void k_amr_prolong(LevelView<double> Pv, LevelView<double> B, AmrBox box, const double* __restrict__ e,
-                              double* __restrict__ up) {
+// Kwak prolongation (Sec. 2.7.3) of the base change e = u - uh onto the
+// patch: parent a + (i, j, k) / 2 and, per dimension, the parent's neighbour
+// on the fine cell's side (the rules across the boundary are linear, so they
+// hold for a change).
+__global__ void k_amr_prolong(LevelView<double> Pv, LevelView<double> B, AmrBox box, const double* __restrict__ u,
+                              const double* __restrict__ uh, double* __restrict__ up) {
   pdl_entry();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -398,11 +495,11 @@ __global__ void k_amr_prolong(LevelView<double> Pv, LevelView<double> B, AmrBox 
   if (i >= Pv.n0 || j >= Pv.n1 || k >= Pv.n2) return;
   const int I = box.a[0] + (i >> 1), J = box.a[1] + (j >> 1), K = Pv.three ? box.a[2] + (k >> 1) : 0;
   const int si = (i & 1) ? 1 : -1, sj = (j & 1) ? 1 : -1, sk = (k & 1) ? 1 : -1;
-  const double ec = e[B.idx(I, J, K)];
-  const double ex = e[B.idx(I + si, J, K)], ey = e[B.idx(I, J + sj, K)];
+  const double ec = coarse_corr(B, u, uh, -1, I, J, K);
+  const double ex = coarse_corr(B, u, uh, -1, I + si, J, K), ey = coarse_corr(B, u, uh, -1, I, J + sj, K);
   double add;
   if (Pv.three)
-    add = 0.25 * (ec + ex + ey + e[B.idx(I, J, K + sk)]);
+    add = 0.25 * (ec + ex + ey + coarse_corr(B, u, uh, -1, I, J, K + sk));
   else
     add = 0.25 * (2.0 * ec + ex + ey);
   up[Pv.idx(i, j, k)] += add;
@@ -431,98 +528,82 @@ __global__ void k_amr_flat(LevelView<double> Pv, LevelView<double> B, AmrBox box
   }
 }
 
-__global__ void k_amr_diff(LevelView<double> L, const double* __restrict__ a, const double* __restrict__ b,
-                           double* __restrict__ out) {
-  pdl_entry();
-  const long n = (long)L.n0 * L.n1 * L.n2;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-    int i, j, k;
-    L.cell(q, i, j, k);
-    const long p = L.idx(i, j, k);
-    out[p] = a[p] - b[p];
-  }
-}
-
 // ---------------------------------------------------------------- launchers
 
-void launch_amr_diff(const LevelView<double>& L, const double* a, const double* b, double* out, cudaStream_t st) {
-  count_launch();
-  const long n = (long)L.n0 * L.n1 * L.n2;
-  long g = cdiv_u(n, 256);
-  if (g > 4096) g = 4096;
-  launch_k(k_amr_diff, (unsigned)g, 256, 0, st, L, a, b, out);
-}
-
-static dim3 amr_block(int three) { return three ? dim3(32, 4, 2) : dim3(32, 8, 1); }
-
-void launch_amr_cf_ghosts(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, double* up,
-                          const double* ub, cudaStream_t st) {
+void launch_amr_cf_base(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, double* gt,
+                        const double* ub, cudaStream_t st) {
   count_launch();
   const long n = 2L * ((long)Pv.n1 * Pv.n2 + (long)Pv.n0 * Pv.n2 + (Pv.three ? (long)Pv.n0 * Pv.n1 : 0L));
-  launch_k(k_amr_cf_ghosts, cdiv_u(n, 256), 256, 0, st, Pv, B, box, up, ub);
+  const unsigned t = spread_threads(n, 32);
+  launch_k(k_amr_cf_base, cdiv_u(n, t), t, 0, st, Pv, B, box, gt, ub);
 }
 
 template <int G>
-static void amr_smooth_g(const LevelView<double>& L, int kind, double* u, const double* f, const double* s0,
-                         const double* s1, int colour, cudaStream_t st) {
-  const dim3 b = amr_block(L.three), g(cdiv_u(L.n0 / 2, b.x), cdiv_u(L.n1, b.y), cdiv_u(L.n2, b.z));
+static void amr_smooth_g(const LevelView<double>& L, int cf, int kind, double* u, const double* gt, const double* f,
+                         const double* s0, const double* s1, int colour, cudaStream_t st) {
+  const dim3 b = colour_block(L), g(cdiv_u(L.n0 / 2, b.x), cdiv_u(L.n1, b.y), cdiv_u(L.n2, b.z));
   if (kind == EQ_PSI)
-    launch_k(k_amr_smooth<G, EQ_PSI>, g, b, 0, st, L, u, f, s0, s1, colour);
+    launch_k(k_amr_smooth<G, EQ_PSI>, g, b, 0, st, L, cf, u, gt, f, s0, s1, colour);
   else
-    launch_k(k_amr_smooth<G, EQ_LIN>, g, b, 0, st, L, u, f, s0, s1, colour);
+    launch_k(k_amr_smooth<G, EQ_LIN>, g, b, 0, st, L, cf, u, gt, f, s0, s1, colour);
 }
-void launch_amr_smooth(const LevelView<double>& L, int kind, double* u, const double* f, const double* s0,
-                       const double* s1, int colour, cudaStream_t st) {
+void launch_amr_smooth(const LevelView<double>& L, int cf, int kind, double* u, const double* gt, const double* f,
+                       const double* s0, const double* s1, int colour, cudaStream_t st) {
   count_launch();
   if (L.geom == CART)
-    amr_smooth_g<CART>(L, kind, u, f, s0, s1, colour, st);
+    amr_smooth_g<CART>(L, cf, kind, u, gt, f, s0, s1, colour, st);
   else if (L.geom == CYL)
-    amr_smooth_g<CYL>(L, kind, u, f, s0, s1, colour, st);
+    amr_smooth_g<CYL>(L, cf, kind, u, gt, f, s0, s1, colour, st);
   else
-    amr_smooth_g<SPH>(L, kind, u, f, s0, s1, colour, st);
+    amr_smooth_g<SPH>(L, cf, kind, u, gt, f, s0, s1, colour, st);
 }
 
 template <int G>
-static void amr_resid_g(const LevelView<double>& L, int kind, const double* u, const double* f, const double* s0,
-                        const double* s1, double* r, unsigned long long* red, int apply, cudaStream_t st) {
-  const dim3 b = amr_block(L.three), g(cdiv_u(L.n0, b.x), cdiv_u(L.n1, b.y), cdiv_u(L.n2, b.z));
+static void amr_resid_g(const LevelView<double>& L, int cf, int kind, const double* u, const double* gt,
+                        const double* f, const double* s0, const double* s1, double* r, unsigned long long* red,
+                        int apply, cudaStream_t st) {
+  const dim3 b = red ? norm_block(L, 1) : cells_block(L), g(cdiv_u(L.n0, b.x), cdiv_u(L.n1, b.y), cdiv_u(L.n2, b.z));
   if (kind == EQ_PSI)
-    launch_k(k_amr_patch_resid<G, EQ_PSI>, g, b, 0, st, L, u, f, s0, s1, r, red, apply);
+    launch_k(k_amr_patch_resid<G, EQ_PSI>, g, b, 0, st, L, cf, u, gt, f, s0, s1, r, red, apply);
   else
-    launch_k(k_amr_patch_resid<G, EQ_LIN>, g, b, 0, st, L, u, f, s0, s1, r, red, apply);
+    launch_k(k_amr_patch_resid<G, EQ_LIN>, g, b, 0, st, L, cf, u, gt, f, s0, s1, r, red, apply);
 }
-void launch_amr_patch_resid(const LevelView<double>& L, int kind, const double* u, const double* f, const double* s0,
-                            const double* s1, double* r, unsigned long long* red, int apply, cudaStream_t st) {
+void launch_amr_patch_resid(const LevelView<double>& L, int cf, int kind, const double* u, const double* gt,
+                            const double* f, const double* s0, const double* s1, double* r, unsigned long long* red,
+                            int apply, cudaStream_t st) {
   count_launch();
   if (L.geom == CART)
-    amr_resid_g<CART>(L, kind, u, f, s0, s1, r, red, apply, st);
+    amr_resid_g<CART>(L, cf, kind, u, gt, f, s0, s1, r, red, apply, st);
   else if (L.geom == CYL)
-    amr_resid_g<CYL>(L, kind, u, f, s0, s1, r, red, apply, st);
+    amr_resid_g<CYL>(L, cf, kind, u, gt, f, s0, s1, r, red, apply, st);
   else
-    amr_resid_g<SPH>(L, kind, u, f, s0, s1, r, red, apply, st);
+    amr_resid_g<SPH>(L, cf, kind, u, gt, f, s0, s1, r, red, apply, st);
 }
 
 void launch_amr_restrict(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, const double* up,
                          const double* rp, double* ub, double* rr, cudaStream_t st) {
   count_launch();
   const int m0 = box.b[0] - box.a[0], m1 = box.b[1] - box.a[1], m2 = box.b[2] - box.a[2];
-  const dim3 b = amr_block(Pv.three), g(cdiv_u(m0, b.x), cdiv_u(m1, b.y), cdiv_u(m2, b.z));
+  const dim3 b = fit_block(m0, m1, m2, spread_threads((long)m0 * m1 * m2, 32));
+  const dim3 g(cdiv_u(m0, b.x), cdiv_u(m1, b.y), cdiv_u(m2, b.z));
   launch_k(k_amr_restrict, g, b, 0, st, Pv, B, box, up, rp, ub, rr);
 }
 
 void launch_amr_flux_corr(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box,
-                          const double* up, const double* ub, double* corr, cudaStream_t st) {
+                          const double* up, const double* gt, const double* ub, double* corr, cudaStream_t st) {
   count_launch();
   const long m0 = box.b[0] - box.a[0], m1 = box.b[1] - box.a[1], m2 = B.three ? box.b[2] - box.a[2] : 1;
   const long n = 2L * (m1 * m2 + m0 * m2 + (B.three ? m0 * m1 : 0L));
-  launch_k(k_amr_flux_corr, cdiv_u(n, 256), 256, 0, st, Pv, B, box, up, ub, corr);
+  const unsigned t = spread_threads(n, 32);
+  launch_k(k_amr_flux_corr, cdiv_u(n, t), t, 0, st, Pv, B, box, up, gt, ub, corr);
 }
 
 template <int G>
 static void amr_base_g(const LevelView<double>& B, const AmrBox& box, int kind, const double* u, const double* s0,
                        const double* s1, const double* f0, const double* rr, const double* corr, double* f,
                        unsigned long long* red, int mode, cudaStream_t st) {
-  const dim3 b = amr_block(B.three), g(cdiv_u(B.n0, b.x), cdiv_u(B.n1, b.y), cdiv_u(B.n2, b.z));
+  const dim3 b = mode == 1 ? norm_block(B, 1) : cells_block(B);
+  const dim3 g(cdiv_u(B.n0, b.x), cdiv_u(B.n1, b.y), cdiv_u(B.n2, b.z));
   if (kind == EQ_PSI)
     launch_k(k_amr_base<G, EQ_PSI>, g, b, 0, st, B, box, u, s0, s1, f0, rr, corr, f, red, mode);
   else
@@ -540,11 +621,11 @@ void launch_amr_base(const LevelView<double>& B, const AmrBox& box, int kind, co
     amr_base_g<SPH>(B, box, kind, u, s0, s1, f0, rr, corr, f, red, mode, st);
 }
 
-void launch_amr_prolong(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, const double* e,
-                        double* up, cudaStream_t st) {
+void launch_amr_prolong(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, const double* u,
+                        const double* uh, double* up, cudaStream_t st) {
   count_launch();
-  const dim3 b = amr_block(Pv.three), g(cdiv_u(Pv.n0, b.x), cdiv_u(Pv.n1, b.y), cdiv_u(Pv.n2, b.z));
-  launch_k(k_amr_prolong, g, b, 0, st, Pv, B, box, e, up);
+  const dim3 b = cells_block(Pv), g(cdiv_u(Pv.n0, b.x), cdiv_u(Pv.n1, b.y), cdiv_u(Pv.n2, b.z));
+  launch_k(k_amr_prolong, g, b, 0, st, Pv, B, box, u, uh, up);
 }
 
 void launch_amr_flat(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, double* up,

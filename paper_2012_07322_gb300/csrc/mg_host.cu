@@ -1912,31 +1912,34 @@ int ensure_amr_aa(mg_hierarchy* H, int m) {
 
 // Arrays of the composite iteration on the finest base level (scalar
 // equations leave components 1 and 2 free): the original right-hand side,
-// the flux correction, the restricted patch residual, the base state before
-// the base V-cycle and its change.
+// the flux correction, the restricted patch residual and the base state
+// before the base V-cycle.
 struct AmrArrays {
-  double *f0, *corr, *rr, *uh, *eb;
+  double *f0, *corr, *rr, *uh;
 };
 AmrArrays amr_arrays(mg_hierarchy* H, const Eq& e) {
   Level& L0 = H->L[0];
-  return AmrArrays{e.kind == EQ_LIN ? L0.f[1] : nullptr, L0.f[2], L0.r[1], L0.u[2], L0.r[2]};
+  return AmrArrays{e.kind == EQ_LIN ? L0.f[1] : nullptr, L0.f[2], L0.r[1], L0.u[2]};
 }
 
-// Base ghosts, patch ghosts (boundary rules, then the coarse-fine values)
-// and the flux correction of the uncovered interface cells.
-void amr_refresh(mg_hierarchy* H, const Eq& e, bool corr) {
+// Base ghosts and the base's share of the patch's coarse-fine ghosts (kept
+// in the ghosts of the patch's right-hand side): current while the uncovered
+// base cells do not change.
+void amr_refresh(mg_hierarchy* H, const Eq& e) {
   auto& A = H->amr;
   Level& L0 = H->L[0];
   const auto vb = with_bc(L0.v64, e.bc);
-  const auto vp = with_bc(A.v, e.bc);
   launch_fill_ghosts(vb, L0.u[0], -1, H->st);
-  launch_fill_ghosts(vp, A.u, -1, H->st);
-  launch_amr_cf_ghosts(vp, vb, A.box, A.u, L0.u[0], H->st);
-  if (corr) {
-    const AmrArrays W = amr_arrays(H, e);
-    cudaMemsetAsync(W.corr, 0, sizeof(double) * L0.ng, H->st);
-    launch_amr_flux_corr(vp, vb, A.box, A.u, L0.u[0], W.corr, H->st);
-  }
+  launch_amr_cf_base(with_bc(A.v, e.bc), vb, A.box, A.f, L0.u[0], H->st);
+}
+
+// The flux correction of the uncovered interface cells (the others' stays
+// zero from the start of the solve).
+void amr_correct(mg_hierarchy* H, const Eq& e) {
+  auto& A = H->amr;
+  Level& L0 = H->L[0];
+  launch_amr_flux_corr(with_bc(A.v, e.bc), with_bc(L0.v64, e.bc), A.box, A.u, A.f, L0.u[0], amr_arrays(H, e).corr,
+                       H->st);
 }
 
 // Relative weighted residual over the composite cells (stopping rule).
@@ -1944,11 +1947,12 @@ int amr_norm(mg_hierarchy* H, const Eq& e, double* rel) {
   auto& A = H->amr;
   Level& L0 = H->L[0];
   const AmrArrays W = amr_arrays(H, e);
-  amr_refresh(H, e, true);
+  amr_refresh(H, e);
+  amr_correct(H, e);
   CK(cudaMemsetAsync(H->d_red, 0, sizeof(unsigned long long) * 3, H->st));
   const double* s0p = e.kind == EQ_PSI ? A.s0 : nullptr;
   const double* s1p = (e.kind == EQ_PSI || e.has_c) ? A.s1 : nullptr;
-  launch_amr_patch_resid(with_bc(A.v, e.bc), e.kind, A.u, A.f, s0p, s1p, nullptr, H->d_red, 0, H->st);
+  launch_amr_patch_resid(with_bc(A.v, e.bc), A.box.cf, e.kind, A.u, A.f, A.f, s0p, s1p, nullptr, H->d_red, 0, H->st);
   launch_amr_base(with_bc(L0.v64, e.bc), A.box, e.kind, L0.u[0], s0ptr(H, e, 0), s1ptr(H, e, 0), W.f0, nullptr,
                   W.corr, nullptr, H->d_red, 1, H->st);
   CK(cudaGetLastError());
@@ -1962,25 +1966,20 @@ int amr_norm(mg_hierarchy* H, const Eq& e, double* rel) {
   return MG_OK;
 }
 
-// Red-black Newton-Gauss-Seidel sweeps of the patch, its ghosts refilled
-// before each colour (the base ghosts are current).
+// Red-black Newton-Gauss-Seidel sweeps of the patch (amr_refresh is current).
 void amr_patch_sweeps(mg_hierarchy* H, const Eq& e, int nsweeps) {
   auto& A = H->amr;
-  Level& L0 = H->L[0];
-  const auto vb = with_bc(L0.v64, e.bc);
   const auto vp = with_bc(A.v, e.bc);
   const double* s0p = e.kind == EQ_PSI ? A.s0 : nullptr;
   const double* s1p = (e.kind == EQ_PSI || e.has_c) ? A.s1 : nullptr;
-  for (int sw = 0; sw < nsweeps; ++sw)
-    for (int colour = 0; colour < 2; ++colour) {
-      launch_fill_ghosts(vp, A.u, -1, H->st);
-      launch_amr_cf_ghosts(vp, vb, A.box, A.u, L0.u[0], H->st);
-      launch_amr_smooth(vp, e.kind, A.u, A.f, s0p, s1p, colour, H->st);
-    }
+  for (int h = 0; h < 2 * nsweeps; ++h)
+    launch_amr_smooth(vp, A.box.cf, e.kind, A.u, A.f, A.f, s0p, s1p, h & 1, H->st);
   H->updates += (int64_t)nsweeps * (int64_t)A.n[0] * A.n[1] * A.n[2];
 }
 
-// One composite FAS V(nu1, nu2) cycle.
+// One composite FAS V(nu1, nu2) cycle, after amr_norm of the same state
+// (whose amr_refresh still holds: the restriction changes covered base cells
+// only, which neither the ghosts' interpolation nor its boundary rules read).
 void amr_cycle(mg_hierarchy* H, const Eq& e) {
   auto& A = H->amr;
   Level& L0 = H->L[0];
@@ -1989,21 +1988,16 @@ void amr_cycle(mg_hierarchy* H, const Eq& e) {
   const AmrArrays W = amr_arrays(H, e);
   const double* s0p = e.kind == EQ_PSI ? A.s0 : nullptr;
   const double* s1p = (e.kind == EQ_PSI || e.has_c) ? A.s1 : nullptr;
-  launch_fill_ghosts(vb, L0.u[0], -1, H->st);
   amr_patch_sweeps(H, e, H->d.nu1);
-  launch_fill_ghosts(vp, A.u, -1, H->st);
-  launch_amr_cf_ghosts(vp, vb, A.box, A.u, L0.u[0], H->st);
-  launch_amr_patch_resid(vp, e.kind, A.u, A.f, s0p, s1p, A.r, nullptr, 0, H->st);
+  launch_amr_patch_resid(vp, A.box.cf, e.kind, A.u, A.f, A.f, s0p, s1p, A.r, nullptr, 0, H->st);
   launch_amr_restrict(vp, vb, A.box, A.u, A.r, L0.u[0], W.rr, H->st);
   cudaMemcpyAsync(W.uh, L0.u[0], sizeof(double) * L0.ng, cudaMemcpyDeviceToDevice, H->st);
-  amr_refresh(H, e, true);
+  amr_correct(H, e);
   launch_amr_base(vb, A.box, e.kind, L0.u[0], s0ptr(H, e, 0), s1ptr(H, e, 0), W.f0, W.rr, W.corr, L0.f[0], nullptr,
                   0, H->st);
   vcycle64(H, e, 0);
-  launch_amr_diff(vb, L0.u[0], W.uh, W.eb, H->st);
-  launch_fill_ghosts(vb, W.eb, -1, H->st);  // the rules are linear: homogeneous for a change
-  launch_amr_prolong(vp, vb, A.box, W.eb, A.u, H->st);
-  launch_fill_ghosts(vb, L0.u[0], -1, H->st);
+  launch_amr_prolong(vp, vb, A.box, L0.u[0], W.uh, A.u, H->st);
+  amr_refresh(H, e);
   amr_patch_sweeps(H, e, H->d.nu2);
 }
 
@@ -2057,6 +2051,7 @@ int run_solve_amr(mg_hierarchy* H, const Eq& e, mg_solve_report* rep) {
   const int m = d.accel_depth;
   H->updates = 0;
   restrict_sources(H, e);
+  CK(cudaMemsetAsync(amr_arrays(H, e).corr, 0, sizeof(double) * L0.ng, H->st));
   const long nfl = A.flat.n0;
   double *ag = nullptr, *ax = nullptr, *afp = nullptr, *agp = nullptr, *adF = nullptr, *adG = nullptr;
   if (m > 0) {
@@ -3205,10 +3200,12 @@ int mg_apply_amr(mg_hierarchy* H, const int box_lo[3], const int box_hi[3], int 
   Level& L0 = H->L[0];
   const AmrArrays W = amr_arrays(H, e);
   restrict_sources(H, e);
-  amr_refresh(H, e, true);
+  amr_refresh(H, e);
+  CK(cudaMemsetAsync(W.corr, 0, sizeof(double) * L0.ng, H->st));
+  amr_correct(H, e);
   const double* s0p = e.kind == EQ_PSI ? A.s0 : nullptr;
   const double* s1p = (e.kind == EQ_PSI || e.has_c) ? A.s1 : nullptr;
-  launch_amr_patch_resid(with_bc(A.v, e.bc), e.kind, A.u, nullptr, s0p, s1p, A.r, nullptr, 1, H->st);
+  launch_amr_patch_resid(with_bc(A.v, e.bc), A.box.cf, e.kind, A.u, A.f, nullptr, s0p, s1p, A.r, nullptr, 1, H->st);
   launch_amr_base(with_bc(L0.v64, e.bc), A.box, e.kind, L0.u[0], s0ptr(H, e, 0), s1ptr(H, e, 0), nullptr, nullptr,
                   W.corr, L0.r[0], nullptr, 2, H->st);
   copy_out(H, L0.r[0], out);

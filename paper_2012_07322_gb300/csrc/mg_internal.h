@@ -3,6 +3,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "mg_dev.cuh"
@@ -74,6 +75,60 @@ template <typename T>
 inline long ghost_count_host(const LevelView<T>& L) {
   const long nk = L.n2 + 2 * L.three;
   return 2L * (L.n1 + 2) * nk + 2L * L.n0 * nk + (L.three ? 2L * L.n0 * L.n1 : 0L);
+}
+
+// ------------------------------------------------------- launch shapes
+
+extern int g_sms;  // multiprocessors of the device, set when a hierarchy is created
+inline int sm_count() { return g_sms > 0 ? g_sms : 152; }
+
+// Threads per block of a pass with one thread per item over n items: the
+// smallest of lo .. 256 that needs at most 8 blocks per multiprocessor.  The
+// FP64 pipe takes ~16 cycles per warp instruction, so a level of a few
+// thousand cells in 256-thread blocks keeps a few SMs busy for microseconds
+// while the others idle: the FP64 vector colour pass took ~11 us on every
+// level of a 64x32x32 hierarchy, down to 128 cells, before the blocks were
+// made small enough to spread over the device.
+inline unsigned spread_threads(long n, unsigned lo) {
+  unsigned t = lo;
+  while (t < 256 && n > 8L * sm_count() * t) t *= 2;
+  return t;
+}
+// Block of at most t threads (a power of two) that tiles nx x ny x nz items
+// (powers of two) without idle threads, z planes deep at least: the FP64
+// pipe spends a whole instruction slot on a warp with idle lanes too.
+inline dim3 fit_block(int nx, int ny, int nz, unsigned t, unsigned z = 1) {
+  dim3 b(1, 1, z);
+  t = t > z ? t / z : 1;
+  b.x = std::min<unsigned>({(unsigned)nx, 32u, t});
+  t /= b.x;
+  b.y = std::min<unsigned>((unsigned)ny, t);
+  t /= b.y;
+  b.z *= std::max<unsigned>(1u, std::min<unsigned>((unsigned)nz / z, t));
+  return b;
+}
+template <typename T>
+inline long ncells(const LevelView<T>& L) {
+  return (long)L.n0 * L.n1 * L.n2;
+}
+// Blocks of a pass over all cells, and of one over the cells of one colour.
+// FP32 passes are not bound by their pipe: larger blocks.
+template <typename T>
+inline dim3 cells_block(const LevelView<T>& L) {
+  return fit_block(L.n0, L.n1, L.n2, spread_threads(ncells(L), sizeof(T) == 8 ? 32 : 128));
+}
+template <typename T>
+inline dim3 colour_block(const LevelView<T>& L) {
+  return fit_block(L.n0 / 2, L.n1, L.n2, spread_threads(ncells(L) / 2, sizeof(T) == 8 ? 32 : 128));
+}
+// Passes that end in block maxima and atomics: at most 512 blocks until
+// they have 256 threads.
+template <typename T>
+inline dim3 norm_block(const LevelView<T>& L, long per_thread, unsigned z = 1) {
+  const long n = ncells(L) / per_thread;
+  unsigned t = 32;
+  while (t < 256 && n > 512L * t) t *= 2;
+  return fit_block(L.n0, L.n1, std::max(1, (int)(L.n2 / per_thread)), t, z);
 }
 
 void count_launch(int n = 1);
@@ -315,31 +370,33 @@ struct AmrBox {
   int a[3], b[3];
   int cf;
 };
-void launch_amr_cf_ghosts(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, double* up,
-                          const double* ub, cudaStream_t st);
-void launch_amr_smooth(const LevelView<double>& L, int kind, double* u, const double* f, const double* s0,
-                       const double* s1, int colour, cudaStream_t st);
+// The base's share of the coarse-fine ghosts into their places in gt, which
+// the patch's smoother, residual and the flux correction complete.
+void launch_amr_cf_base(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, double* gt,
+                        const double* ub, cudaStream_t st);
+void launch_amr_smooth(const LevelView<double>& L, int cf, int kind, double* u, const double* gt, const double* f,
+                       const double* s0, const double* s1, int colour, cudaStream_t st);
 // r = f - L(u) on the patch (f nullable; apply: r = L(u)), norms into red.
-void launch_amr_patch_resid(const LevelView<double>& L, int kind, const double* u, const double* f, const double* s0,
-                            const double* s1, double* r, unsigned long long* red, int apply, cudaStream_t st);
+void launch_amr_patch_resid(const LevelView<double>& L, int cf, int kind, const double* u, const double* gt,
+                            const double* f, const double* s0, const double* s1, double* r, unsigned long long* red,
+                            int apply, cudaStream_t st);
 void launch_amr_restrict(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, const double* up,
                          const double* rp, double* ub, double* rr, cudaStream_t st);
 void launch_amr_flux_corr(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box,
-                          const double* up, const double* ub, double* corr, cudaStream_t st);
+                          const double* up, const double* gt, const double* ub, double* corr, cudaStream_t st);
 // Base level of the composite grid: mode 0 the FAS right-hand side f, 1 the
 // composite residual norms of the uncovered cells into red, 2 the composite
 // operator into f (0 on covered cells).
 void launch_amr_base(const LevelView<double>& B, const AmrBox& box, int kind, const double* u, const double* s0,
                      const double* s1, const double* f0, const double* rr, const double* corr, double* f,
                      unsigned long long* red, int mode, cudaStream_t st);
-void launch_amr_prolong(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, const double* e,
-                        double* up, cudaStream_t st);
+// up += P (u - uh), u and uh on the base.
+void launch_amr_prolong(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, const double* u,
+                        const double* uh, double* up, cudaStream_t st);
 // Composite unknowns <-> flat vector x (patch cells, then the uncovered
 // base cells at the ghosted offsets bmap[0 .. nbase - 1]).
 void launch_amr_flat(const LevelView<double>& Pv, const LevelView<double>& B, const AmrBox& box, double* up,
                      double* ub, const int* bmap, long nbase, double* x, int to_flat, cudaStream_t st);
-// out = a - b over the interior (ghosted arrays of L).
-void launch_amr_diff(const LevelView<double>& L, const double* a, const double* b, double* out, cudaStream_t st);
 
 // Anderson mixing (mg_accel.cu): live ring slots of the difference columns
 // in age order (the newest last).

@@ -20,57 +20,7 @@ unsigned long long launch_count() { return g_launches.load(std::memory_order_rel
 static inline dim3 block_for(int three) { return three ? dim3(32, 4, 2) : dim3(32, 8, 1); }
 static inline unsigned cdiv(long a, long b) { return (unsigned)((a + b - 1) / b); }
 
-static int g_sms = 0;  // multiprocessors of the device, set when a hierarchy is created
-static inline int sm_count() { return g_sms > 0 ? g_sms : 152; }
-
-// Threads per block of a pass with one thread per item over n items: the
-// smallest of lo .. 256 that needs at most 8 blocks per multiprocessor.  The
-// FP64 pipe takes ~16 cycles per warp instruction, so a level of a few
-// thousand cells in 256-thread blocks keeps a few SMs busy for microseconds
-// while the others idle: the FP64 vector colour pass took ~11 us on every
-// level of a 64x32x32 hierarchy, down to 128 cells, before the blocks were
-// made small enough to spread over the device.
-static inline unsigned spread_threads(long n, unsigned lo) {
-  unsigned t = lo;
-  while (t < 256 && n > 8L * sm_count() * t) t *= 2;
-  return t;
-}
-// Block of at most t threads (a power of two) that tiles nx x ny x nz items
-// (powers of two) without idle threads, z planes deep at least: the FP64
-// pipe spends a whole instruction slot on a warp with idle lanes too.
-static inline dim3 fit_block(int nx, int ny, int nz, unsigned t, unsigned z = 1) {
-  dim3 b(1, 1, z);
-  t = t > z ? t / z : 1;
-  b.x = std::min<unsigned>({(unsigned)nx, 32u, t});
-  t /= b.x;
-  b.y = std::min<unsigned>((unsigned)ny, t);
-  t /= b.y;
-  b.z *= std::max<unsigned>(1u, std::min<unsigned>((unsigned)nz / z, t));
-  return b;
-}
-template <typename T>
-static inline long ncells(const LevelView<T>& L) {
-  return (long)L.n0 * L.n1 * L.n2;
-}
-// Blocks of a pass over all cells, and of one over the cells of one colour.
-// FP32 passes are not bound by their pipe: larger blocks.
-template <typename T>
-static inline dim3 cells_block(const LevelView<T>& L) {
-  return fit_block(L.n0, L.n1, L.n2, spread_threads(ncells(L), sizeof(T) == 8 ? 32 : 128));
-}
-template <typename T>
-static inline dim3 colour_block(const LevelView<T>& L) {
-  return fit_block(L.n0 / 2, L.n1, L.n2, spread_threads(ncells(L) / 2, sizeof(T) == 8 ? 32 : 128));
-}
-// Passes that end in block maxima and atomics: at most 512 blocks until
-// they have 256 threads.
-template <typename T>
-static inline dim3 norm_block(const LevelView<T>& L, long per_thread, unsigned z = 1) {
-  const long n = ncells(L) / per_thread;
-  unsigned t = 32;
-  while (t < 256 && n > 512L * t) t *= 2;
-  return fit_block(L.n0, L.n1, std::max(1, (int)(L.n2 / per_thread)), t, z);
-}
+int g_sms = 0;
 
 // ------------------------------------------------------------ smoothers
 
