@@ -383,12 +383,16 @@ __global__ void k_loop_decide(LoopState* __restrict__ S, const unsigned long lon
                               cudaGraphConditionalHandle h, int first) {
   pdl_entry();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const double num = __longlong_as_double((long long)red[1]), den = __longlong_as_double((long long)red[2]);
-  double rel;
-  if (isinf(num) || isinf(den) || isnan(num) || isnan(den))
-    rel = __longlong_as_double(0x7ff8000000000000LL);
-  else
-    rel = num / (den > 1e-300 ? den : 1e-300);
+  double rel = 0.0;
+  for (int b = 0; b < P.nb; ++b) {
+    const double num = __longlong_as_double((long long)red[3 * b + 1]);
+    const double den = __longlong_as_double((long long)red[3 * b + 2]);
+    const double q = num / (den > 1e-300 ? den : 1e-300);
+    if (isinf(num) || isinf(den) || isnan(num) || isnan(den))
+      rel = __longlong_as_double(0x7ff8000000000000LL);
+    else if (!(q <= rel))
+      rel = rel != rel ? rel : q;
+  }
   if (first) {
     S->cyc = 0;
     S->ncol = 0;

@@ -17,7 +17,7 @@ template <int G, bool VEC>
 __global__ void __launch_bounds__(BC_THREADS, 1) k_block_vcycle32(const __grid_constant__ BlockCycle32 P) {
   bc_stage_tables(P);  // fixed for the hierarchy: fetched before waiting for the preceding launch
   pdl_entry();
-  bc_run<G, VEC, false, true>(P);
+  bc_run<G, VEC, false, true>(P, blockIdx.x * P.ng0);
 }
 
 // Column col of the coarsest vector operator (lap V + 1/3 grad div V with
@@ -103,7 +103,7 @@ static void launch_g(const BlockCycle32& P, cudaStream_t st) {
   if (P.vec)
     launch_k(k_block_vcycle32<G, true>, 1, BC_THREADS, P.smem, st, P);
   else
-    launch_k(k_block_vcycle32<G, false>, 1, BC_THREADS, P.smem, st, P);
+    launch_k(k_block_vcycle32<G, false>, P.nb, BC_THREADS, P.smem, st, P);
 }
 
 void launch_block_vcycle32(const BlockCycle32& P, int geom, cudaStream_t st) {

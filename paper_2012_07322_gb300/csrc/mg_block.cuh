@@ -558,10 +558,11 @@ __device__ void bc_coarse(const BlockCycle32& P, const BcLevel& B) {
 // The whole cycle from level l0 of P: its right-hand side in from P.f_in,
 // the correction out to P.e_out (ghosts included).  No barrier after the
 // final stores.  DENSE_ONLY: P carries the dense coarsest operator (cA) or
-// its inverse (cinv).  TABLES: the coefficient tables are on their way to
+// its inverse (cinv).  problem_at: offset of the block's problem in them.
+// TABLES: the coefficient tables are on their way to
 // shared memory already (bc_stage_tables).
 template <int G, bool VEC, bool DENSE_ONLY = false, bool TABLES = false>
-__device__ void bc_run(const BlockCycle32& P) {
+__device__ void bc_run(const BlockCycle32& P, long problem_at = 0) {
   constexpr int nc = VEC ? 3 : 1;
   if (!TABLES) bc_stage_tables(P);
   {
@@ -570,7 +571,7 @@ __device__ void bc_run(const BlockCycle32& P) {
     const BcLevel B = bc_level<VEC>(P, 0);
 #pragma unroll
     for (int c = 0; c < nc; ++c) {
-      for (int q = threadIdx.x; q < (int)P.ng0 / 4; q += BC_THREADS) bc_cp16(B.f[c] + 4 * q, P.f_in[c] + 4 * q);
+      for (int q = threadIdx.x; q < (int)P.ng0 / 4; q += BC_THREADS) bc_cp16(B.f[c] + 4 * q, P.f_in[c] + problem_at + 4 * q);
       for (int q = threadIdx.x; q < (int)P.ng0; q += BC_THREADS) B.e[c][q] = 0.0f;
     }
     if (!VEC)
@@ -603,7 +604,7 @@ __device__ void bc_run(const BlockCycle32& P) {
 #pragma unroll
   for (int c = 0; c < nc; ++c)
     for (int q = threadIdx.x; q < (int)P.ng0 / 4; q += BC_THREADS)
-      reinterpret_cast<float4*>(P.e_out[c])[q] = reinterpret_cast<const float4*>(B.e[c])[q];
+      reinterpret_cast<float4*>(P.e_out[c] + problem_at)[q] = reinterpret_cast<const float4*>(B.e[c])[q];
 }
 
 }  // namespace gmg

@@ -8,8 +8,6 @@
 
 namespace gmg {
 
-static inline unsigned cdiv_u(long a, long b) { return (unsigned)((a + b - 1) / b); }
-
 // ------------------------------------------------------- FP64 residual
 
 // r = f - lap u of every cell of a level with equal spacings (r, r32
@@ -26,7 +24,13 @@ __global__ void __launch_bounds__(256)
   pdl_entry();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k0 = (blockIdx.z * blockDim.z + threadIdx.z) * KZ;
+  int b;
+  const int k0 = (L.z_block(b) * blockDim.z + threadIdx.z) * KZ;
+  u += b * L.bst;
+  if (f) f += b * L.bst;
+  if (r) r += b * L.bst;
+  if (r32) r32 += b * L.bst;
+  if (red) red += 3 * b;
   const long sx = L.sx, sy = L.sy;
   const bool neumann = L.bc == BC_NEUMANN;
   const bool edge_ij = i == 0 || i == L.n0 - 1 || j == 0 || j == L.n1 - 1;
@@ -77,7 +81,7 @@ void launch_resid_cart(const LevelView<double>& L, const double* u, const double
   // the device that way take two planes per thread
   const bool big = (long)L.n0 * L.n1 * L.n2 >= (1L << 21);
   const dim3 b(32, 8, 1);
-  const dim3 g(L.n0 / 32, L.n1 / 8, L.n2 / (big ? 8 : 2));
+  const dim3 g(L.n0 / 32, L.n1 / 8, L.nb * (L.n2 / (big ? 8 : 2)));
   if (big)
     launch_k(k_resid_cart<8>, g, b, 0, st, L, u, f, r, r32, red, weighted);
   else
@@ -98,7 +102,11 @@ __global__ void __launch_bounds__(256)
                           const float* __restrict__ f, float* __restrict__ fc, float* __restrict__ ec) {
   pdl_entry();
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
-  const int K0 = (blockIdx.z * blockDim.z + threadIdx.z) * KC;
+  int bq;
+  const int K0 = (F.z_block(bq) * blockDim.z + threadIdx.z) * KC;
+  e += bq * F.bst;
+  f += bq * F.bst;
+  fc += bq * C.bst;
   const int i = 2 * I, j = 2 * J;
   const long sx = F.sx, sy = F.sy;
   const bool ie = i + 2 == F.n0, iw = i == 0, jn = j + 2 == F.n1, js = j == 0;
@@ -163,7 +171,7 @@ __global__ void __launch_bounds__(256)
     }
     fc[C.idx(I, J, K)] = s * 0.125f;
   }
-  const long nz = C.sy * (C.n2 + 2) / 4;
+  const long nz = C.nb * (C.sy * (C.n2 + 2) / 4);
   const long nb = (long)blockDim.x * blockDim.y * blockDim.z;
   const long gt = threadIdx.x + (long)blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z) +
                   nb * (blockIdx.x + gridDim.x * (blockIdx.y + (long)gridDim.y * blockIdx.z));
@@ -182,7 +190,11 @@ __global__ void __launch_bounds__(256)
                    const T* __restrict__ uhH) {
   pdl_entry();
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
-  const int K = blockIdx.z * blockDim.z + threadIdx.z;
+  int b;
+  const int K = F.z_block(b) * blockDim.z + threadIdx.z;
+  u += b * F.bst;
+  uH += b * C.bst;
+  if (uhH) uhH += b * C.bst;
   const long q = C.idx(I, J, K);
   auto e = [&](long p) { return uhH ? uH[p] - uhH[p] : uH[p]; };
   const T ec = e(q);
@@ -218,20 +230,20 @@ void launch_resid_restrict_cart(const LevelView<float>& F, const LevelView<float
   count_launch();
   const dim3 b(32, 8, 1);
   if ((long)F.n0 * F.n1 * F.n2 >= (1L << 23))
-    launch_k(k_resid_restrict_cart<4>, dim3(C.n0 / 32, C.n1 / 8, C.n2 / 4), b, 0, st, F, C, e, f, fc, ec);
+    launch_k(k_resid_restrict_cart<4>, dim3(C.n0 / 32, C.n1 / 8, C.nb * (C.n2 / 4)), b, 0, st, F, C, e, f, fc, ec);
   else
-    launch_k(k_resid_restrict_cart<1>, dim3(C.n0 / 32, C.n1 / 8, C.n2), b, 0, st, F, C, e, f, fc, ec);
+    launch_k(k_resid_restrict_cart<1>, dim3(C.n0 / 32, C.n1 / 8, C.nb * C.n2), b, 0, st, F, C, e, f, fc, ec);
 }
 
 void launch_prolong_cart(const LevelView<float>& F, const LevelView<float>& C, float* u, const float* uH,
                          const float* uhH, cudaStream_t st) {
   count_launch();
-  launch_k(k_prolong_cart<float, float2>, dim3(C.n0 / 32, C.n1 / 8, C.n2), dim3(32, 8, 1), 0, st, F, C, u, uH, uhH);
+  launch_k(k_prolong_cart<float, float2>, dim3(C.n0 / 32, C.n1 / 8, C.nb * C.n2), dim3(32, 8, 1), 0, st, F, C, u, uH, uhH);
 }
 void launch_prolong_cart(const LevelView<double>& F, const LevelView<double>& C, double* u, const double* uH,
                          const double* uhH, cudaStream_t st) {
   count_launch();
-  launch_k(k_prolong_cart<double, double2>, dim3(C.n0 / 32, C.n1 / 8, C.n2), dim3(32, 8, 1), 0, st, F, C, u, uH, uhH);
+  launch_k(k_prolong_cart<double, double2>, dim3(C.n0 / 32, C.n1 / 8, C.nb * C.n2), dim3(32, 8, 1), 0, st, F, C, u, uH, uhH);
 }
 template bool transfer_cart_applies<float>(const LevelView<float>&);
 template bool transfer_cart_applies<double>(const LevelView<double>&);

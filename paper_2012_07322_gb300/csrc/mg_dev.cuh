@@ -57,6 +57,8 @@ struct LevelView {
   int ln0, ln1;        // log2 of n0, n1 (all sizes are powers of two)
   const T* ti;         // NTI tables of n0 + 2
   const T* tj;         // NTJ tables of n1 + 2
+  int nb;              // independent problems the level's arrays hold (1 but for the classes of MG_DIVB_EXACT)
+  long bst;            // ... one after the other, this many values apart
   const T* vc;         // VC_N per-(i, j) coefficients of the vector operator, or null
   __device__ __forceinline__ long idx(int i, int j, int k) const { return off + i + j * sx + (long)k * sy; }
   __device__ __forceinline__ T TI(int s, int i) const { return ti[s * (n0 + 2) + i + 1]; }
@@ -76,6 +78,16 @@ struct LevelView {
     j = (int)(jk & (n1 - 1));
     k = (int)(jk >> ln1);
     i = 2 * t + ((j + k + colour) & 1);
+  }
+  // The z block index of a launch over all problems (grid.z = problems x
+  // blocks of one), split into the block within a problem (returned) and the
+  // problem's offset in this level's arrays.
+  __device__ __forceinline__ int z_block(int& b) const {
+    b = 0;
+    if (nb == 1) return blockIdx.z;
+    const int gz = gridDim.z / nb;
+    b = blockIdx.z / gz;
+    return blockIdx.z - b * gz;
   }
   __device__ __forceinline__ T xc0(int i) const { return lo0 + (T(i) + T(0.5)) * h0; }
   __device__ __forceinline__ T xc1(int j) const { return lo1 + (T(j) + T(0.5)) * h1; }

@@ -20,6 +20,7 @@ using namespace gmg;
 namespace {
 
 constexpr int MAX_LEVELS = 16;
+constexpr int RED_SLOTS = 32;
 constexpr int NPARTS = 1024;           // blocks of the deterministic sums
 constexpr int COARSE_SWEEPS = 16;      // coarsest-grid sweep cap (Sec. 2.7.2)
 // Sweep cap of the coarsest scalar correction equation inside the FP32
@@ -75,8 +76,11 @@ struct mg_hierarchy {
   // level-0 arrays of the xCFC sequence (ghosted)
   double *Xg[3] = {}, *dpsi = nullptr, *dap = nullptr, *sg = nullptr, *Ug = nullptr, *Sg = nullptr,
          *Sig[3] = {};
-  unsigned long long* d_red = nullptr;   // 8 reduction slots
+  int nb = 1;  // problems the hierarchy solves together (MG_DIVB_EXACT's classes)
+  // 8 reduction slots, then 3 per problem when there are several
+  unsigned long long* d_red = nullptr;
   unsigned long long* h_red = nullptr;   // pinned mirror
+  unsigned long long* norm_red() const { return nb > 1 ? d_red + 8 : d_red; }
   double* d_part = nullptr;
   char* arena = nullptr;
   size_t arena_bytes = 0;
@@ -262,6 +266,21 @@ int validate(const mg_grid_desc* d) {
 // Descriptor of the parity-class problems of the exact-projection cleaning:
 // n / 2 cells per dimension over the same domain (spacing 2 h), the same
 // solver settings.
+int level_sizes(const mg_grid_desc* d, int n[][3], double h[][3]);
+
+// Problems the class hierarchy solves together: all of them in mixed
+// precision (V-cycles without mixing, a coarsest level the one-block cycle
+// takes), whose 64^3-sized cycle is a chain of launches too small to fill the
+// device; else one after the other.
+int class_batch(const mg_grid_desc* c) {
+  if (c->precision != MG_MIXED || c->accel_depth != 0 || c->cycle != MG_CYCLE_V) return 1;
+  int n[MAX_LEVELS][3];
+  double h[MAX_LEVELS][3];
+  const int nl = level_sizes(c, n, h);
+  if ((long)n[nl - 1][0] * n[nl - 1][1] * n[nl - 1][2] > 512) return 1;
+  return c->ndim == 3 ? 8 : 4;
+}
+
 mg_grid_desc class_desc(const mg_grid_desc* d) {
   mg_grid_desc c = *d;
   for (int k = 0; k < d->ndim; ++k) c.n[k] = d->n[k] / 2;
@@ -294,7 +313,9 @@ int level_sizes(const mg_grid_desc* d, int n[][3], double h[][3]) {
 }
 
 // Walk the arena layout; with base == nullptr only sizes are summed.
-size_t layout(mg_hierarchy* H, const mg_grid_desc* d, char* base) {
+// nb problems: the arrays of the mixed Poisson cycle (u, f, e, its scratch
+// and its right-hand side, component 0) hold nb of them one after the other.
+size_t layout(mg_hierarchy* H, const mg_grid_desc* d, char* base, int nb = 1) {
   size_t off = 0;
   auto take = [&](size_t bytes) -> char* {
     off = (off + 255) & ~size_t(255);
@@ -333,17 +354,17 @@ size_t layout(mg_hierarchy* H, const mg_grid_desc* d, char* base) {
     }
     t32(L ? &L->tj32 : &dummy32, sizeof(float) * NTJ * (n[l][1] + 2));
     for (int c = 0; c < 3; ++c) {
-      t64(L ? &L->u[c] : &dummy64, b64);
+      t64(L ? &L->u[c] : &dummy64, c == 0 ? nb * b64 : b64);
       if (l > 0) t64(L ? &L->uh[c] : &dummy64, b64);
-      t64(L ? &L->f[c] : &dummy64, b64);
+      t64(L ? &L->f[c] : &dummy64, c == 0 ? nb * b64 : b64);
       t64(L ? &L->r[c] : &dummy64, b64);
     }
     t64(L ? &L->s0 : &dummy64, b64);
     t64(L ? &L->s1 : &dummy64, b64);
     if (mixed) {
       for (int c = 0; c < 3; ++c) {
-        t32(L ? &L->e[c] : &dummy32, b32);
-        t32(L ? &L->f32[c] : &dummy32, b32);
+        t32(L ? &L->e[c] : &dummy32, c < 2 ? nb * b32 : b32);
+        t32(L ? &L->f32[c] : &dummy32, c == 0 ? nb * b32 : b32);
       }
       t32(L ? &L->k32 : &dummy32, b32);
     }
@@ -363,7 +384,7 @@ size_t layout(mg_hierarchy* H, const mg_grid_desc* d, char* base) {
       }
     }
   }
-  char* p = take(sizeof(unsigned long long) * 8);
+  char* p = take(sizeof(unsigned long long) * RED_SLOTS);
   if (H) H->d_red = (unsigned long long*)p;
   p = take(sizeof(double) * 2 * NPARTS);  // two sets of block sums
   if (H) H->d_part = (double*)p;
@@ -592,6 +613,8 @@ LevelView<T> make_view(const mg_grid_desc* d, const Level& L, const T* ti, const
   v.ti = ti;
   v.tj = tj;
   v.vc = nullptr;
+  v.nb = 1;
+  v.bst = L.ng;
   return v;
 }
 
@@ -800,7 +823,8 @@ double bits_to_double(unsigned long long b) {
 int finest_residual(mg_hierarchy* H, const Eq& e) {
   Level& L = H->L[0];
   auto v = with_bc(L.v64, e.bc);
-  CK(cudaMemsetAsync(H->d_red, 0, sizeof(unsigned long long) * 3, H->st));
+  unsigned long long* const red = H->norm_red();
+  CK(cudaMemsetAsync(red, 0, sizeof(unsigned long long) * 3 * H->nb, H->st));
   long tok = prof_begin(H, 0,
                         e.kind == EQ_VEC ? MG_PROF_RESID64_VEC
                                          : (e.kind == EQ_PSI ? MG_PROF_RESID64_PSI : MG_PROF_RESID64_SCALAR),
@@ -810,12 +834,12 @@ int finest_residual(mg_hierarchy* H, const Eq& e) {
   const bool mixed = H->d.precision == MG_MIXED;
   if (e.kind != EQ_VEC) {
     launch_residual_scalar(v, e.kind, L.u[0], fptr(H, e, 0, 0), s0ptr(H, e, 0), s1ptr(H, e, 0),
-                           (double*)nullptr, H->d_red, 1, H->st, mixed ? L.f32[0] : nullptr,
+                           (double*)nullptr, red, 1, H->st, mixed ? L.f32[0] : nullptr,
                            (mixed && e.kind == EQ_PSI) ? L.k32 : nullptr);
   } else {
     const double* f[3] = {L.f[0], L.f[1], L.f[2]};
     double* const none[3] = {nullptr, nullptr, nullptr};
-    launch_residual_vec(v, L.u, f, none, H->d_red, 1, H->st, mixed ? L.f32 : nullptr);
+    launch_residual_vec(v, L.u, f, none, red, 1, H->st, mixed ? L.f32 : nullptr);
   }
   prof_end(H, tok);
   CK(cudaGetLastError());
@@ -826,13 +850,16 @@ int finest_residual(mg_hierarchy* H, const Eq& e) {
 int finest_norm(mg_hierarchy* H, const Eq& e, double* rel) {
   if (int st = finest_residual(H, e)) return st;
   // slot 3: status of this cycle's mixing solve (read by run_solve)
-  CK(cudaMemcpyAsync(H->h_red, H->d_red, sizeof(unsigned long long) * 4, cudaMemcpyDeviceToHost, H->st));
+  CK(cudaMemcpyAsync(H->h_red, H->norm_red(), sizeof(unsigned long long) * (H->nb > 1 ? 3 * H->nb : 4),
+                     cudaMemcpyDeviceToHost, H->st));
   CK(cudaStreamSynchronize(H->st));
-  const double num = bits_to_double(H->h_red[1]), den = bits_to_double(H->h_red[2]);
-  if (std::isinf(num) || std::isinf(den) || std::isnan(num) || std::isnan(den)) {
-    *rel = NAN;
-  } else {
-    *rel = num / (den > 1e-300 ? den : 1e-300);
+  *rel = 0.0;
+  for (int b = 0; b < H->nb; ++b) {
+    const double num = bits_to_double(H->h_red[3 * b + 1]), den = bits_to_double(H->h_red[3 * b + 2]);
+    if (std::isinf(num) || std::isinf(den) || std::isnan(num) || std::isnan(den))
+      *rel = NAN;
+    else if (!std::isnan(*rel))
+      *rel = std::max(*rel, num / (den > 1e-300 ? den : 1e-300));
   }
   return MG_OK;
 }
@@ -888,7 +915,7 @@ void smooth32(mg_hierarchy* H, const Eq& e, int l, int nsweeps) {
       }
     }
   }
-  H->updates += (int64_t)nsweeps * L.cells() * e.ncomp;
+  H->updates += (int64_t)nsweeps * L.cells() * e.ncomp * H->nb;
 }
 
 // Coarsest correction equation solved in FP64 on the level's FP64 scratch.
@@ -1009,7 +1036,8 @@ void block_vcycle32(mg_hierarchy* H, const Eq& e, int l0) {
   // K of eq. psi reached level l0 with the down leg; the block restricts it further
   BlockCycle32 P = block_cycle_params(H, e, l0);
   P.fold_k = H->fold_k32;
-  for (int l = l0; l + 1 < H->nlev; ++l) H->updates += (int64_t)(H->d.nu1 + H->d.nu2) * H->L[l].cells() * e.ncomp;
+  P.nb = H->nb;
+  for (int l = l0; l + 1 < H->nlev; ++l) H->updates += (int64_t)(H->d.nu1 + H->d.nu2) * H->L[l].cells() * e.ncomp * H->nb;
   long tok = prof_begin(H, l0, MG_PROF_BLOCK_CYCLE32, H->L[l0].cells());
   launch_block_vcycle32(P, H->d.geom, H->st);
   prof_end(H, tok);
@@ -1113,7 +1141,7 @@ int cycle_map(mg_hierarchy* H, const Eq& e) {
   } else {
     auto v = with_bc(L0.v64, e.bc);
     // f32 holds the FP32 residual written by the preceding finest_norm
-    for (int c = 0; c < e.ncomp; ++c) CK(cudaMemsetAsync(L0.e[c], 0, sizeof(float) * L0.ng, H->st));
+    for (int c = 0; c < e.ncomp; ++c) CK(cudaMemsetAsync(L0.e[c], 0, sizeof(float) * L0.ng * H->nb, H->st));
     // eq. psi: K = dS/du at this u was written by finest_norm with f32; the
     // V-cycle restricts it level by level on its way down (fold_k32)
     if (e.kind == EQ_PSI && fmg) restrict_k32(H, 1);
@@ -1482,7 +1510,7 @@ int build_loop_graph(mg_hierarchy* H, const Eq& e, int key, double* ax, double* 
     if (top) cudaGraphDestroy(top);
     return LOOP_UNSUPPORTED;
   }
-  const LoopParams P{d.tol, d.max_cycles, d.stall_window, m};
+  const LoopParams P{d.tol, d.max_cycles, d.stall_window, m, H->nb};
   const int64_t u0 = H->updates;
   // The kernels are captured straight into the graph and into the while
   // node's body (no child-graph nodes), so the programmatic edges between
@@ -1506,7 +1534,7 @@ int build_loop_graph(mg_hierarchy* H, const Eq& e, int key, double* ax, double* 
     for (int c = 0; c < e.ncomp; ++c)
       cudaMemcpyAsync(ax + (long)c * stride, L0.u[c], sizeof(double) * L0.ng, cudaMemcpyDeviceToDevice, H->st);
   int st = finest_residual(H, e);
-  launch_loop_decide(H->d_loop, H->d_red, P, hc, 1, H->st);
+  launch_loop_decide(H->d_loop, H->norm_red(), P, hc, 1, H->st);
   const unsigned long long lpre = launch_count() - l0;
   cudaStreamCaptureStatus cs;
   const cudaGraphNode_t* deps = nullptr;
@@ -1560,7 +1588,7 @@ int build_loop_graph(mg_hierarchy* H, const Eq& e, int key, double* ax, double* 
     if (e.kind == EQ_VEC) fill_all64(H, e, 0);
   }
   if (!st) st = finest_residual(H, e);
-  launch_loop_decide(H->d_loop, H->d_red, P, hc, 0, H->st);
+  launch_loop_decide(H->d_loop, H->norm_red(), P, hc, 0, H->st);
   cudaGraph_t body_out = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(H->st, &body_out);
   const unsigned long long lbody = launch_count() - l1;
@@ -1876,7 +1904,7 @@ int ensure_amr(mg_hierarchy* H, const AmrBox& box) {
   while (nf < A.nvec) nf <<= 1, ++lg;
   A.flat = LevelView<double>{};
   A.flat.n0 = (int)nf;
-  A.flat.n1 = A.flat.n2 = 1;
+  A.flat.n1 = A.flat.n2 = A.flat.nb = 1;
   A.flat.three = 0;
   A.flat.sx = A.flat.sy = nf;
   A.flat.off = 0;
@@ -2212,6 +2240,14 @@ const char* mg_strerror(int s) {
 
 const char* mg_last_error(void) { return g_last_error; }
 
+}  // extern "C"
+
+namespace {
+int create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, int nb, mg_hierarchy** out);
+}
+
+extern "C" {
+
 int mg_hierarchy_bytes(const mg_grid_desc* desc, size_t* bytes) {
   int st = validate(desc);
   if (st) return st;
@@ -2219,18 +2255,27 @@ int mg_hierarchy_bytes(const mg_grid_desc* desc, size_t* bytes) {
   *bytes = layout(nullptr, desc, nullptr);
   if (desc->divb_variant == MG_DIVB_EXACT) {
     const mg_grid_desc c = class_desc(desc);
-    *bytes += layout(nullptr, &c, nullptr);
+    *bytes += layout(nullptr, &c, nullptr, class_batch(&c));
   }
   return MG_OK;
 }
 
 int mg_create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, mg_hierarchy** out) {
+  return create_hierarchy(desc, cuda_stream, 1, out);
+}
+
+}  // extern "C"
+
+namespace {
+
+int create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, int nb, mg_hierarchy** out) {
   int st = validate(desc);
   if (st) return st;
   if (!out) return fail(MG_ERR_INVALID, "null output");
   mg_hierarchy* H = new (std::nothrow) mg_hierarchy();
   if (!H) return fail(MG_ERR_OOM, "host allocation failed");
   H->d = *desc;
+  H->nb = nb;
   if (H->d.ndim == 2) {
     H->d.n[2] = 1;
     H->d.lo[2] = 0.0;
@@ -2253,15 +2298,15 @@ int mg_create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, mg_hierarch
   int n[MAX_LEVELS][3];
   double h[MAX_LEVELS][3];
   H->nlev = level_sizes(&H->d, n, h);
-  const size_t bytes = layout(nullptr, &H->d, nullptr);
+  const size_t bytes = layout(nullptr, &H->d, nullptr, nb);
   if (cudaMalloc(&H->arena, bytes) != cudaSuccess) {
     H->arena = nullptr;
     mg_destroy_hierarchy(H);
     return fail(MG_ERR_OOM, "arena allocation failed");
   }
   H->arena_bytes = bytes;
-  layout(H, &H->d, H->arena);
-  if (cudaMallocHost(&H->h_red, sizeof(unsigned long long) * 8) != cudaSuccess) {
+  layout(H, &H->d, H->arena, nb);
+  if (cudaMallocHost(&H->h_red, sizeof(unsigned long long) * RED_SLOTS) != cudaSuccess) {
     H->h_red = nullptr;
     mg_destroy_hierarchy(H);
     return fail(MG_ERR_OOM, "pinned allocation failed");
@@ -2316,8 +2361,10 @@ int mg_create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, mg_hierarch
     }
     L.v64 = make_view<double>(&H->d, L, L.ti64, L.tj64);
     L.v64.vc = L.vc64;
+    L.v64.nb = nb;
     L.v32 = make_view<float>(&H->d, L, L.ti32, L.tj32);
     L.v32.vc = L.vc32;
+    L.v32.nb = nb;
     if (H->d.precision == MG_MIXED && sweep_uses_maps(L.v32)) {
       bool ok = true;
       for (int leg = 0; leg < 2; ++leg) {
@@ -2334,7 +2381,7 @@ int mg_create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, mg_hierarch
   }
   if (H->d.divb_variant == MG_DIVB_EXACT) {
     const mg_grid_desc c = class_desc(&H->d);
-    const int sst = mg_create_hierarchy(&c, (void*)H->st, &H->sub);
+    const int sst = create_hierarchy(&c, (void*)H->st, class_batch(&c), &H->sub);
     if (sst != MG_OK) {
       H->sub = nullptr;
       mg_destroy_hierarchy(H);
@@ -2344,6 +2391,10 @@ int mg_create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, mg_hierarch
   *out = H;
   return MG_OK;
 }
+
+}  // namespace
+
+extern "C" {
 
 uint64_t mg_kernel_launches(void) { return (uint64_t)launch_count(); }
 
@@ -2850,6 +2901,25 @@ int mg_solve_cfc_batch(mg_hierarchy* const* hs, int count, const mg_cfc_sources*
   return status;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The Neumann problems lap Phi = f (zero mean) of a hierarchy that holds
+// several, f and Phi ghost-free one after the other, from a zero start.
+int solve_classes(mg_hierarchy* H, const double* f, double* phi, mg_solve_report* rep) {
+  Level& L0 = H->L[0];
+  copy_in(H, f, L0.f[0]);
+  CK(cudaMemsetAsync(L0.u[0], 0, sizeof(double) * L0.ng * H->nb, H->st));
+  const int st = run_solve(H, Eq{MG_EQ_LIN, MG_BC_NEUMANN, 1, 1, false}, rep);
+  copy_out(H, L0.u[0], phi);
+  return st;
+}
+
+}  // namespace
+
+extern "C" {
+
 int mg_clean_divB(mg_hierarchy* H, double* B[3], double* phi_out, int flags, mg_divb_report* rep) {
   if (!H || !B) return fail(MG_ERR_INVALID, "null argument");
   const int nd = H->d.ndim;
@@ -2922,7 +2992,13 @@ int mg_clean_divB(mg_hierarchy* H, double* B[3], double* phi_out, int flags, mg_
     launch_class_gather(v, L0.r[0], H->d_part, NPARTS / 8, L0.r[1], H->st);
     CK(cudaMemsetAsync(L0.r[2], 0, sizeof(double) * L0.cells(), H->st));
     mg_solve_report agg{};
-    for (int q = 0; q < ncl; ++q) {
+    if (H->sub->nb > 1) {
+      // all classes together: the report is the largest residual's
+      const int sq = solve_classes(H->sub, L0.r[1], L0.r[2], &agg);
+      if (sq == MG_ERR_CUDA || sq == MG_ERR_INVALID || sq == MG_ERR_OOM) return sq;
+      st = sq;
+    }
+    for (int q = 0; q < ncl && H->sub->nb == 1; ++q) {
       mg_solve_report r{};
       const int sq = mg_solve_scalar(H->sub, MG_EQ_LIN, MG_BC_NEUMANN, 1, nullptr, nullptr, nullptr,
                                      L0.r[1] + q * M, L0.r[2] + q * M, &r);

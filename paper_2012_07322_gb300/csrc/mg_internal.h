@@ -109,23 +109,23 @@ inline dim3 fit_block(int nx, int ny, int nz, unsigned t, unsigned z = 1) {
 }
 template <typename T>
 inline long ncells(const LevelView<T>& L) {
-  return (long)L.n0 * L.n1 * L.n2;
+  return (long)L.n0 * L.n1 * L.n2;  // of one problem
 }
 // Blocks of a pass over all cells, and of one over the cells of one colour.
 // FP32 passes are not bound by their pipe: larger blocks.
 template <typename T>
 inline dim3 cells_block(const LevelView<T>& L) {
-  return fit_block(L.n0, L.n1, L.n2, spread_threads(ncells(L), sizeof(T) == 8 ? 32 : 128));
+  return fit_block(L.n0, L.n1, L.n2, spread_threads(L.nb * ncells(L), sizeof(T) == 8 ? 32 : 128));
 }
 template <typename T>
 inline dim3 colour_block(const LevelView<T>& L) {
-  return fit_block(L.n0 / 2, L.n1, L.n2, spread_threads(ncells(L) / 2, sizeof(T) == 8 ? 32 : 128));
+  return fit_block(L.n0 / 2, L.n1, L.n2, spread_threads(L.nb * ncells(L) / 2, sizeof(T) == 8 ? 32 : 128));
 }
 // Passes that end in block maxima and atomics: at most 512 blocks until
 // they have 256 threads.
 template <typename T>
 inline dim3 norm_block(const LevelView<T>& L, long per_thread, unsigned z = 1) {
-  const long n = ncells(L) / per_thread;
+  const long n = L.nb * ncells(L) / per_thread;
   unsigned t = 32;
   while (t < 256 && n > 512L * t) t *= 2;
   return fit_block(L.n0, L.n1, std::max(1, (int)(L.n2 / per_thread)), t, z);
@@ -453,6 +453,7 @@ struct LoopState {
 struct LoopParams {
   double tol;
   int max_cycles, stall_window, m;
+  int nb;  // problems: the norms of problem b in slots 3 b .. 3 b + 2, all of them within tol
 };
 void launch_loop_decide(LoopState* S, const unsigned long long* red, const LoopParams& P,
                         cudaGraphConditionalHandle h, int first, cudaStream_t st);
@@ -477,6 +478,7 @@ struct BlockLevel32 {
 };
 struct BlockCycle32 {
   int nl, vec, nu1, nu2, coarse_sweeps;
+  int nb;      // problems, one block each, ng0 values apart in f_in and e_out (scalar equations without c)
   int fold_k;  // restrict c from level l0 on the way down (else every level's is read from HBM)
   BlockLevel32 lv[BC_MAX];
   LevelView<double> c64;  // the coarsest level, boundary rule applied

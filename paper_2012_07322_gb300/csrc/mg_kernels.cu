@@ -32,10 +32,12 @@ __global__ void k_smooth_scalar(LevelView<T> L, T* __restrict__ u, const T* __re
   pdl_entry();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z * blockDim.z + threadIdx.z;
+  int b;
+  const int k = L.z_block(b) * blockDim.z + threadIdx.z;
   if (2 * t >= L.n0 || j >= L.n1 || k >= L.n2) return;
   const int i = 2 * t + ((j + k + colour) & 1);
-  scalar_update<T, G, KIND>(L, u, f, s0, s1, i, j, k);
+  const long o = b * L.bst;
+  scalar_update<T, G, KIND>(L, u + o, f ? f + o : f, s0, s1, i, j, k);
 }
 
 // One colour of component comp of the vector sweep.  With a ghost-push
@@ -463,7 +465,12 @@ __global__ void __launch_bounds__(RbShape<TX>::THREADS, TX == 128 ? (G == CART ?
   T* sc = sf + RB_NF * BP;
   constexpr int TY = RbShape<TX>::TY;
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
-  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, L.n2);
+  int prob;
+  const int z0 = L.z_block(prob) * zc, z1 = min(z0 + zc, L.n2);
+  uin += prob * L.bst;
+  uout += prob * L.bst;
+  f += prob * L.bst;
+  const int mz = prob * (L.n2 + 2) + 1;  // plane 0 of the problem in the tensor maps
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // coefficients of the lane's cells (uniform on a Cartesian grid)
   RbLaneCoef<T, TX> lc;
@@ -490,10 +497,10 @@ __global__ void __launch_bounds__(RbShape<TX>::THREADS, TX == 128 ? (G == CART ?
           constexpr unsigned PB = (unsigned)(BP * sizeof(T));
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           mbar_expect(&mbar[bu], (uok ? PB : 0u) + (fok ? PB * (HAS_C ? 2u : 1u) : 0u));
-          if (uok) tma_plane(su + bu * BP, &M.u, i0, j0 - 1, wrap(p) + 1, &mbar[bu]);
+          if (uok) tma_plane(su + bu * BP, &M.u, i0, j0 - 1, wrap(p) + mz, &mbar[bu]);
           if (fok) {
-            tma_plane(sf + bf, &M.f, i0, j0 - 1, wrap(pf) + 1, &mbar[bu]);
-            if (HAS_C) tma_plane(sc + bf, &M.c, i0, j0 - 1, wrap(pf) + 1, &mbar[bu]);
+            tma_plane(sf + bf, &M.f, i0, j0 - 1, wrap(pf) + mz, &mbar[bu]);
+            if (HAS_C) tma_plane(sc + bf, &M.c, i0, j0 - 1, wrap(pf) + mz, &mbar[bu]);
           }
         }
         pending |= 1u << bu;
@@ -712,11 +719,18 @@ __global__ void k_residual_scalar(LevelView<T> L, const T* __restrict__ u, const
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   unsigned long long m[3] = {0ULL, 0ULL, 0ULL};
+  int b;
+  const int bz = L.z_block(b);
+  u += b * L.bst;
+  if (f) f += b * L.bst;
+  if (r) r += b * L.bst;
+  if (r32) r32 += b * L.bst;
+  if (red) red += 3 * b;
   if (i < L.n0 && j < L.n1) {
     const double w = weighted ? (double)norm_weight(L, i, j) : 1.0;
 #pragma unroll
     for (int it = 0; it < KZ; ++it) {
-      const int k = (blockIdx.z * KZ + it) * blockDim.z + threadIdx.z;
+      const int k = (bz * KZ + it) * blockDim.z + threadIdx.z;
       if (k >= L.n2) continue;
       const long p = L.idx(i, j, k);
       T Sv, kp;
@@ -911,10 +925,10 @@ __global__ void k_prolong(LevelView<T> F, LevelView<T> Cv, T* __restrict__ u, co
 // columns i0 / 2 - 1 .. (i1 - 1) / 2 + 1, likewise in j and k.  Such blocks
 // run the prolongation and the residual without the boundary rules, which
 // FP32 code otherwise evaluates for every cell.
-__device__ __forceinline__ bool block_coarse_interior(int n0, int n1, int n2, bool three) {
+__device__ __forceinline__ bool block_coarse_interior(int n0, int n1, int n2, bool three, int bz) {
   const int i0 = blockIdx.x * blockDim.x, i1 = i0 + blockDim.x;
   const int j0 = blockIdx.y * blockDim.y, j1 = j0 + blockDim.y;
-  const int k0 = blockIdx.z * blockDim.z, k1 = k0 + blockDim.z;
+  const int k0 = bz * blockDim.z, k1 = k0 + blockDim.z;
   return i0 >= 2 && i1 + 2 <= n0 && j0 >= 2 && j1 + 2 <= n1 && (!three || (k0 >= 2 && k1 + 2 <= n2));
 }
 
@@ -923,15 +937,19 @@ __global__ void k_prolong3(LevelView<T> F, LevelView<T> Cv, Ptr3<T> u, CPtr3<T> 
   pdl_entry();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z * blockDim.z + threadIdx.z;
+  int b;
+  const int bz = F.z_block(b), k = bz * blockDim.z + threadIdx.z;
   if (i >= F.n0 || j >= F.n1 || k >= F.n2) return;
-  if (block_coarse_interior(F.n0, F.n1, F.n2, F.three)) {
+  const long of = b * F.bst, oc = b * Cv.bst;
+  auto at = [&](const T* q) { return q ? q + oc : q; };
+  if (block_coarse_interior(F.n0, F.n1, F.n2, F.three, bz)) {
 #pragma unroll
     for (int c = 0; c < NC; ++c)
-      prolong_cell<T, true>(F, Cv, u.at(c), uH.at(c), uhH.at(c), vec ? c : -1, i, j, k);
+      prolong_cell<T, true>(F, Cv, u.at(c) + of, uH.at(c) + oc, at(uhH.at(c)), vec ? c : -1, i, j, k);
   } else {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) prolong_cell(F, Cv, u.at(c), uH.at(c), uhH.at(c), vec ? c : -1, i, j, k);
+    for (int c = 0; c < NC; ++c)
+      prolong_cell(F, Cv, u.at(c) + of, uH.at(c) + oc, at(uhH.at(c)), vec ? c : -1, i, j, k);
   }
 }
 
@@ -957,18 +975,20 @@ __global__ void __launch_bounds__(256) k_resid_restrict32(LevelView<float> F, Le
   const int t = threadIdx.x + bx * (threadIdx.y + by * threadIdx.z);
   const int i = blockIdx.x * bx + threadIdx.x;
   const int j = blockIdx.y * by + threadIdx.y;
-  const int k = blockIdx.z * bz + threadIdx.z;
+  int prob;
+  const int zb = F.z_block(prob), k = zb * bz + threadIdx.z;
+  const long of = prob * F.bst, oc = prob * Cv.bst;  // scalar levels without K only
   if (i < F.n0 && j < F.n1 && k < F.n2) {
     const long p = F.idx(i, j, k);
     if (VEC) {
 #pragma unroll
       for (int c = 0; c < NC; ++c) rt[c][t] = vec_residual_cell<float, G>(F, e.p[0], e.p[1], e.p[2], f.at(c), c, i, j, p);
-    } else if (block_coarse_interior(F.n0, F.n1, F.n2, F.three)) {
+    } else if (block_coarse_interior(F.n0, F.n1, F.n2, F.three, zb)) {
       float Sv;
-      rt[0][t] = scalar_residual_cell<float, G, EQ_LIN, true>(F, e.p[0], f.p[0], nullptr, K, i, j, k, p, Sv);
+      rt[0][t] = scalar_residual_cell<float, G, EQ_LIN, true>(F, e.p[0] + of, f.p[0] + of, nullptr, K, i, j, k, p, Sv);
     } else {
       float Sv;
-      rt[0][t] = scalar_residual_cell<float, G, EQ_LIN>(F, e.p[0], f.p[0], nullptr, K, i, j, k, p, Sv);
+      rt[0][t] = scalar_residual_cell<float, G, EQ_LIN>(F, e.p[0] + of, f.p[0] + of, nullptr, K, i, j, k, p, Sv);
     }
   }
   __syncthreads();
@@ -977,7 +997,7 @@ __global__ void __launch_bounds__(256) k_resid_restrict32(LevelView<float> F, Le
   for (int w = t; w < NC * ncell; w += bx * by * bz) {
     const int c = w / ncell, q = w - c * ncell;
     const int ci = q % cx, cj = (q / cx) % cy, ck = q / (cx * cy);
-    const int I = blockIdx.x * cx + ci, J = blockIdx.y * cy + cj, KK = F.three ? blockIdx.z * cz + ck : 0;
+    const int I = blockIdx.x * cx + ci, J = blockIdx.y * cy + cj, KK = F.three ? zb * cz + ck : 0;
     if (I >= Cv.n0 || J >= Cv.n1 || KK >= Cv.n2) continue;
     float wi[2], wj[2];
     wi[0] = F.TI(TI_VW, 2 * I);
@@ -995,7 +1015,7 @@ __global__ void __launch_bounds__(256) k_resid_restrict32(LevelView<float> F, Le
         for (int di = 0; di < 2; ++di)
           sr += wi[di] * wj[dj] * rt[c][(2 * ci + di) + bx * ((2 * cj + dj) + by * (2 * ck + dk))];
     const long qc = Cv.idx(I, J, KK);
-    fc.at(c)[qc] = sr * inv;
+    fc.at(c)[qc + oc] = sr * inv;
     if (c == 0 && Kc) {
       float sk = 0.0f;
       for (int dk = 0; dk < nk; ++dk)
@@ -1005,7 +1025,7 @@ __global__ void __launch_bounds__(256) k_resid_restrict32(LevelView<float> F, Le
       Kc[qc] = sk * inv;
     }
   }
-  const long nz = Cv.sy * (Cv.n2 + 2 * Cv.three);
+  const long nz = Cv.nb * Cv.sy * (Cv.n2 + 2 * Cv.three);
   const long gt = (long)t + (long)bx * by * bz * (blockIdx.x + gridDim.x * (blockIdx.y + (long)gridDim.y * blockIdx.z));
   const long gs = (long)bx * by * bz * gridDim.x * gridDim.y * gridDim.z;
   for (long q = gt; q < nz; q += gs)
@@ -1098,6 +1118,8 @@ __global__ void k_partial_sum(LevelView<T> L, const T* __restrict__ u, double* _
   const long n = (long)L.n0 * L.n1 * L.n2;
   const long stride = (long)gridDim.x * blockDim.x;
   double s = 0.0;
+  u += blockIdx.y * L.bst;
+  part += blockIdx.y * gridDim.x;
   if (L.n0 >= 4) {
     for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n / 4; q += stride) {
       double v[4];
@@ -1114,7 +1136,8 @@ template <typename T>
 __global__ void k_sub_mean(LevelView<T> L, T* __restrict__ u, const double* __restrict__ part, int nparts) {
   pdl_entry();
   const long n = (long)L.n0 * L.n1 * L.n2;
-  const double mean = mean_of(part, nparts, (double)n);
+  const double mean = mean_of(part + blockIdx.y * nparts, nparts, (double)n);
+  u += blockIdx.y * L.bst;
   const long stride = (long)gridDim.x * blockDim.x;
   if (L.n0 >= 4) {
     for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n / 4; q += stride) {
@@ -1137,6 +1160,8 @@ template <typename A, typename B>
 __global__ void k_copy_in(LevelView<B> L, const A* __restrict__ src, B* __restrict__ dst, A shift) {
   pdl_entry();
   const long n = (long)L.n0 * L.n1 * L.n2;
+  src += blockIdx.y * n;
+  dst += blockIdx.y * L.bst;
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
     int i, j, k;
     L.cell(q, i, j, k);
@@ -1147,6 +1172,8 @@ template <typename A, typename B>
 __global__ void k_copy_out(LevelView<A> L, const A* __restrict__ src, B* __restrict__ dst, A shift) {
   pdl_entry();
   const long n = (long)L.n0 * L.n1 * L.n2;
+  src += blockIdx.y * L.bst;
+  dst += blockIdx.y * n;
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
     int i, j, k;
     L.cell(q, i, j, k);
@@ -1184,8 +1211,8 @@ __global__ void k_add_correction(LevelView<double> L, Ptr3<double> u, CPtr3<T> e
   const long stride = (long)gridDim.x * blockDim.x;
   double s = 0.0;
   for (int c = 0; c < ncomp; ++c) {
-    double* __restrict__ uc = u.at(c);
-    const T* __restrict__ ecp = e.at(c);
+    double* __restrict__ uc = u.at(c) + blockIdx.y * L.bst;
+    const T* __restrict__ ecp = e.at(c) + blockIdx.y * L.bst;
     if (L.n0 >= 4) {
       for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n / 4; q += stride) {
         const long p = group4(L, q);
@@ -1211,11 +1238,11 @@ __global__ void k_add_correction(LevelView<double> L, Ptr3<double> u, CPtr3<T> e
 
 template <typename T>
 static dim3 grid_colour(const LevelView<T>& L, dim3 b) {
-  return dim3(cdiv(L.n0 / 2, b.x), cdiv(L.n1, b.y), cdiv(L.n2, b.z));
+  return dim3(cdiv(L.n0 / 2, b.x), cdiv(L.n1, b.y), L.nb * cdiv(L.n2, b.z));
 }
 template <typename T>
 static dim3 grid_cells(const LevelView<T>& L, dim3 b) {
-  return dim3(cdiv(L.n0, b.x), cdiv(L.n1, b.y), cdiv(L.n2, b.z));
+  return dim3(cdiv(L.n0, b.x), cdiv(L.n1, b.y), L.nb * cdiv(L.n2, b.z));
 }
 static unsigned grid_flat(long n, int threads) {
   long g = (n + threads - 1) / threads;
@@ -1304,7 +1331,7 @@ void init_fused_sweep_attributes() {
 // in three runs a single block, the others two blocks of 34 steps).
 template <typename T>
 int fused_sweep_chunk(const LevelView<T>& L, int tx, bool with_c) {
-  const long cols = (long)cdiv(L.n0, tx) * cdiv(L.n1, tx == 128 ? RbShape<128>::TY : RbShape<64>::TY);
+  const long cols = (long)L.nb * cdiv(L.n0, tx) * cdiv(L.n1, tx == 128 ? RbShape<128>::TY : RbShape<64>::TY);
   const long cap = FusedCapacity<T>::blocks[L.geom][tx == 128][with_c];
   const long sms = sm_count();
   int best = 8;
@@ -1327,7 +1354,7 @@ static void launch_rb(const LevelView<T>& L, const T* uin, T* uout, const T* f, 
                       const SweepMaps* maps) {
   const int zc = fused_sweep_chunk(L, TX, c != nullptr);
   constexpr int NT = RbShape<TX>::THREADS;
-  dim3 g(cdiv(L.n0, TX), cdiv(L.n1, RbShape<TX>::TY), cdiv(L.n2, zc));
+  dim3 g(cdiv(L.n0, TX), cdiv(L.n1, RbShape<TX>::TY), L.nb * cdiv(L.n2, zc));
   SweepMaps none;
   std::memset(&none, 0, sizeof(none));
   const SweepMaps& M = (rb_tma<T, G, TX>() && maps) ? *maps : none;
@@ -1396,7 +1423,7 @@ bool sweep_plane_map(CUtensorMap* m, const float* base, const LevelView<float>& 
   if (!enc || !base) return false;
   // (padded row index, row index, plane index) of the ghosted array; cell
   // (i, j, k) sits at (i + ROW_PAD, j + 1, k + 1)
-  const cuuint64_t dims[3] = {(cuuint64_t)L.sx, (cuuint64_t)(L.n1 + 2), (cuuint64_t)(L.n2 + 2)};
+  const cuuint64_t dims[3] = {(cuuint64_t)L.sx, (cuuint64_t)(L.n1 + 2), (cuuint64_t)L.nb * (L.n2 + 2)};
   const cuuint64_t strides[2] = {(cuuint64_t)L.sx * sizeof(float), (cuuint64_t)L.sy * sizeof(float)};
   const cuuint32_t box[3] = {(cuuint32_t)RbShape<128>::BX, (cuuint32_t)RbShape<128>::BY, 1};
   const cuuint32_t es[3] = {1, 1, 1};
@@ -1507,7 +1534,7 @@ void launch_residual_scalar(const LevelView<T>& L, int kind, const T* u, const T
   count_launch();
   if (L.three && ncells(L) >= RES_KZ_CELLS) {
     dim3 b = block_for(L.three), g = grid_cells(L, b);
-    g.z = cdiv(L.n2, (long)b.z * RES_KZ);
+    g.z = L.nb * cdiv(L.n2, (long)b.z * RES_KZ);
     GMG_GEOM_DISPATCH(L.geom, if (kind == EQ_PSI) launch_k(k_residual_scalar<T, GG, EQ_PSI, RES_KZ>, g, b, 0, st, L, u, f, s0, s1, r, r32, k32, red, weighted);
                       else launch_k(k_residual_scalar<T, GG, EQ_LIN, RES_KZ>, g, b, 0, st, L, u, f, s0, s1, r, r32, nullptr, red, weighted));
     return;
@@ -1659,21 +1686,22 @@ void launch_coarse_vec(const LevelView<T>& L, T* V[3], const T* const f[3], int 
 template <typename T>
 void launch_sub_mean(const LevelView<T>& L, T* u, double* part, int nparts, cudaStream_t st, bool have_part) {
   count_launch(have_part ? 1 : 2);
-  if (!have_part) launch_k(k_partial_sum<T>, nparts, 256, 0, st, L, u, part);
-  launch_k(k_sub_mean<T>, nparts, 256, 0, st, L, u, part, nparts);
+  const dim3 g(nparts / L.nb, L.nb);  // block sums of each problem
+  if (!have_part) launch_k(k_partial_sum<T>, g, 256, 0, st, L, u, part);
+  launch_k(k_sub_mean<T>, g, 256, 0, st, L, u, part, nparts / L.nb);
 }
 
 template <typename A, typename B>
 void launch_copy_in(const LevelView<B>& L, const A* src, B* dst, A shift, cudaStream_t st) {
   count_launch();
   long n = (long)L.n0 * L.n1 * L.n2;
-  launch_k(k_copy_in<A, B>, grid_flat(n, 256), 256, 0, st, L, src, dst, shift);
+  launch_k(k_copy_in<A, B>, dim3(grid_flat(n, 256), L.nb), 256, 0, st, L, src, dst, shift);
 }
 template <typename A, typename B>
 void launch_copy_out(const LevelView<A>& L, const A* src, B* dst, A shift, cudaStream_t st) {
   count_launch();
   long n = (long)L.n0 * L.n1 * L.n2;
-  launch_k(k_copy_out<A, B>, grid_flat(n, 256), 256, 0, st, L, src, dst, shift);
+  launch_k(k_copy_out<A, B>, dim3(grid_flat(n, 256), L.nb), 256, 0, st, L, src, dst, shift);
 }
 template <typename A, typename B>
 void launch_convert(const LevelView<A>& L, const A* src, B* dst, cudaStream_t st) {
@@ -1687,7 +1715,7 @@ void launch_add_correction(const LevelView<double>& L, int ncomp, double* const 
   count_launch();
   long n = (long)L.n0 * L.n1 * L.n2;
   const unsigned g = part ? (unsigned)nparts : grid_flat((L.n0 >= 4 ? n / 4 : n) * ncomp, 256);
-  launch_k(k_add_correction<T>, g, 256, 0, st, L, Ptr3<double>::of(u, ncomp), CPtr3<T>::of(e, ncomp), ncomp,
+  launch_k(k_add_correction<T>, dim3(g, L.nb), 256, 0, st, L, Ptr3<double>::of(u, ncomp), CPtr3<T>::of(e, ncomp), ncomp,
            part);
 }
 
