@@ -208,10 +208,12 @@ typedef struct {
 int mg_solve_cfc(mg_hierarchy* h, const mg_cfc_sources* src, mg_cfc_fields* io, int flags,
                  mg_cfc_report* rep);
 
-/* Launch shape of mg_solve_cfc_batch (NULL, or 0 in a field: the default). */
+/* Launch shape of mg_solve_cfc_batch (NULL, or 0 in both fields: chosen from
+ * the batch's sizes; 0 in one field: 2 blocks, 16384 cells).  A problem's
+ * result does not depend on it. */
 typedef struct {
-  int team;            /* blocks of a cluster that run one large problem: 1, 2 (default), 4 or 8 */
-  int64_t team_cells;  /* grids of at least this many cells run on a cluster (default 16384) */
+  int team;            /* blocks of a cluster that run one large problem: 1, 2, 4 or 8 */
+  int64_t team_cells;  /* grids of at least this many cells run on a cluster */
 } mg_batch_opts;
 
 typedef struct {
@@ -488,8 +490,8 @@ int mg_profile_read(mg_hierarchy* h, int klass, int64_t* launches, double* ms, i
 
 /* ------------------------------------------ allocation-free diagnostics */
 
-/* Largest grid (cells) mg_divb_norms_noalloc accepts: the size of its
- * static device scratch (16 MiB on every GPU that loads the library). */
+/* Largest grid (cells) mg_divb_norms_noalloc accepts.  Its static device
+ * scratch takes 16 KiB on every GPU that loads the library. */
 #define MG_NOALLOC_MAX_CELLS 2097152
 
 /*
@@ -508,8 +510,8 @@ int mg_profile_read(mg_hierarchy* h, int klass, int64_t* launches, double* ms, i
  *   cuda_stream       cudaStream_t to run on (NULL: the legacy stream); the
  *                     call synchronises it before returning.
  *   max_div, l2_div   host outputs.
- * It allocates nothing: its scratch (the divergence values, per-block sums
- * and the max word) is a file-scope __device__ array.  The first call on a
+ * It allocates nothing: its scratch (per-block results, a counter and the
+ * combined result) is a file-scope __device__ array.  The first call on a
  * device looks up that array's device address with the device current
  * (cudaGetSymbolAddress); make that first call before any stream capture.
  * Every call shares the array and it keeps the last call's contents (the

@@ -61,7 +61,7 @@ struct BtShared {
   unsigned long long red[3];
   unsigned long long cred[BATCH_TEAM][3];  // rank 0: the team's per-block maxima
   float part[BATCH_THREADS / 32][2 * AA_MAX];
-  float cpart[BATCH_TEAM][2 * AA_MAX];  // rank 0: the team's per-block dot products
+  float cpart[BATCH_TEAM][2 * AA_MAX];  // rank 0: the dot products' parts
   float s[2 * AA_MAX];
   float M[AA_MAX * AA_MAX];  // Gram matrix over ring slots (lives for one equation)
   float gamma[AA_MAX];
@@ -269,6 +269,10 @@ __device__ void bt_vcycle(const Team& T, const BatchItem& I, bool fold) {
 // arrays back to back (the storage at I.aa holds x, f', g' and the m
 // columns of dF and dG in that layout).  Returns the solve's status (0
 // solved, 1 degenerate history; 0 when no column is live).
+// The dot products are summed in BATCH_TEAM parts of the groups, whatever the
+// team's size: block r of s takes parts r, r + s, ..., each part is reduced by
+// itself and the parts are added in order, so a problem's iterates do not
+// depend on the number of blocks that ran it.
 template <int G4>
 __device__ int bt_mix_g(const Team& T, const BatchItem& I, int ncomp, const AACols& cols, BtShared& S) {
   const LevelView<double> L = I.v64;
@@ -288,11 +292,17 @@ __device__ int bt_mix_g(const Team& T, const BatchItem& I, int ncomp, const AACo
   const float* __restrict__ dFr = dF;
   float* __restrict__ dFw = dF + onew;
   float* __restrict__ dGw = dG + onew;
+  constexpr int PART = BATCH_THREADS;  // groups of one part in a stride of BATCH_TEAM parts
+  for (int part = T.rank; part < BATCH_TEAM; part += T.size) {
+  if ((long)part * PART >= nq) {
+    if (nc > 0 && threadIdx.x < 32) T.at0(S.cpart[part])[threadIdx.x] = 0.0f;
+    continue;
+  }
   float v[32];
 #pragma unroll
   for (int a = 0; a < 32; ++a) v[a] = 0.0f;
   for (int c = 0; c < ncomp; ++c)
-  for (long q = T.start(); q < nq; q += T.stride()) {
+  for (long q = (long)part * PART + threadIdx.x; q < nq; q += (long)BATCH_TEAM * PART) {
     double* __restrict__ u = I.u3[c];
     const long pu = aa_pos<G4>(L, q), p = (long)c * ng + pu;
     double g[G4], xv[G4], fp[G4], gp[G4], f[G4];
@@ -332,12 +342,8 @@ __device__ int bt_mix_g(const Team& T, const BatchItem& I, int ncomp, const AACo
       }
     }
   }
-  if (nc == 0) {
-    T.sync();
-    return 0;
-  }
-  // the block's sums (fixed order) into row rank of rank 0's cpart, then
-  // rank 0 adds the rows in rank order and solves
+  if (nc == 0) continue;
+  // the part's sums (fixed order) into its row of rank 0's cpart
   const float w = warp_sum32(v);
   S.part[threadIdx.x >> 5][threadIdx.x & 31] = w;
   __syncthreads();
@@ -345,13 +351,18 @@ __device__ int bt_mix_g(const Team& T, const BatchItem& I, int ncomp, const AACo
     float s = 0.0f;
 #pragma unroll
     for (int b = 0; b < BATCH_THREADS / 32; ++b) s += S.part[b][threadIdx.x];
-    T.at0(S.cpart[T.rank])[threadIdx.x] = s;
+    T.at0(S.cpart[part])[threadIdx.x] = s;
+  }
+  __syncthreads();
   }
   T.sync();
+  if (nc == 0) return 0;
+  // rank 0 adds the parts in order and solves
   if (T.rank == 0 && threadIdx.x < 32) {
     const int t = threadIdx.x;
     float s = 0.0f;
-    for (int r = 0; r < T.size; ++r) s += S.cpart[r][t];
+#pragma unroll
+    for (int r = 0; r < BATCH_TEAM; ++r) s += S.cpart[r][t];
     S.s[t] = s;
     __syncwarp();
     // the newest column's row of the Gram matrix, then the scaled,

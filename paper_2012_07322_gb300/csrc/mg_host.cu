@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <queue>
 #include <thread>
 #include <vector>
 
@@ -2758,11 +2759,71 @@ int64_t cycle_updates(const mg_hierarchy* h) {
 
 }  // namespace
 
+}  // extern "C"
+
+namespace {
+
+// Launch shape of a batch when the caller leaves it open: the cluster size
+// and threshold whose schedule (the kernel's: the problems of a cluster
+// first, longest first, then single blocks) ends earliest.  A problem's time
+// goes as cycles x (BATCH_SERIAL + cells / team): 3 stars took 319, 184, 121
+// and 86 ms on teams of 1, 2, 4 and 8, which leaves 14 % of a 32768-cell
+// problem to rank 0 and the barriers.  Larger clusters leave SMs idle (144 of
+// 152 in fours, 120 in eights), so many problems take smaller teams: 192
+// uneven problems 734, 420, 362 and 480 ms, 45 of them 730, 402, 238 and 185.
+constexpr double BATCH_SERIAL = 4000.0;
+
+void batch_shape(mg_hierarchy* const* hs, int count, size_t smem, int* team, long* team_cells) {
+  std::vector<std::pair<long, double>> work(count);  // cells, cycles
+  for (int i = 0; i < count; ++i)
+    work[i] = {(long)hs[i]->L[0].cells(), hs[i]->batch_cycles > 0 ? hs[i]->batch_cycles : 100.0};
+  std::sort(work.begin(), work.end(), [](const auto& a, const auto& b) {
+    return a.first * a.second > b.first * b.second;
+  });
+  double best = -1.0;
+  for (int t = 1; t <= BATCH_TEAM; t *= 2) {
+    const int clusters = batch_clusters(smem, t);
+    if (clusters < 1) continue;
+    for (long c = 4096; c <= (t == 1 ? 4096 : 65536); c *= 2) {
+      using Heap = std::priority_queue<double, std::vector<double>, std::greater<double>>;
+      Heap free;  // when each cluster, then each block, is free
+      for (int q = 0; q < std::min(clusters, count); ++q) free.push(0.0);
+      double end = 0.0;
+      auto take = [&](const std::pair<long, double>& w, int on) {
+        const double f = free.top() + w.second * (BATCH_SERIAL + (double)w.first / on);
+        free.pop();
+        free.push(f);
+        end = std::max(end, f);
+      };
+      if (t > 1) {
+        for (const auto& w : work)
+          if (w.first >= c) take(w, t);
+        Heap blocks;
+        for (; !free.empty(); free.pop())
+          for (int q = 0; q < t; ++q) blocks.push(free.top());
+        free.swap(blocks);
+      }
+      for (const auto& w : work)
+        if (t == 1 || w.first < c) take(w, 1);
+      if (best < 0.0 || end < 0.98 * best) {
+        best = end;
+        *team = t;
+        *team_cells = c;
+      }
+    }
+  }
+}
+
+}  // namespace
+
+extern "C" {
+
 int mg_solve_cfc_batch(mg_hierarchy* const* hs, int count, const mg_cfc_sources* src, mg_cfc_fields* io, int flags,
                        const mg_batch_opts* opts, mg_cfc_report* rep, mg_batch_report* brep) {
   if (!hs || !src || !io || count <= 0) return fail(MG_ERR_INVALID, "null argument or empty batch");
+  const bool choose = !(opts && (opts->team || opts->team_cells > 0));
   int team_opt = opts && opts->team ? opts->team : BATCH_TEAM_DEFAULT;
-  const long team_cells = opts && opts->team_cells > 0 ? (long)opts->team_cells : BATCH_TEAM_CELLS;
+  long team_cells = opts && opts->team_cells > 0 ? (long)opts->team_cells : BATCH_TEAM_CELLS;
   if (team_opt != 1 && team_opt != 2 && team_opt != 4 && team_opt != 8)
     return fail(MG_ERR_INVALID, "team must be 1, 2, 4 or 8");
   if (flags & MG_HOST_POINTERS) return fail(MG_ERR_INVALID, "batched solves take device pointers");
@@ -2795,6 +2856,7 @@ int mg_solve_cfc_batch(mg_hierarchy* const* hs, int count, const mg_cfc_sources*
   // shortest: the estimated cost is cells x cycles, the cycles those of the
   // problem's previous batched solve (100 before one); the problems a whole
   // cluster runs come before the others
+  if (choose) batch_shape(hs, count, smem, &team_opt, &team_cells);
   std::vector<int> order(count);
   for (int i = 0; i < count; ++i) order[i] = i;
   auto team_of = [&](int a) { return team_opt > 1 && hs[a]->L[0].cells() >= team_cells; };
