@@ -18,7 +18,7 @@ namespace gmg {
 // cell); here a cell costs it three (conversion of the sum, one FMA, the
 // rounding to FP32) and the integer units ~110 instructions.
 template <int KZ>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
     k_resid_cart(LevelView<double> L, const double* __restrict__ u, const double* __restrict__ f,
                  double* __restrict__ r, float* __restrict__ r32, unsigned long long* red, int weighted) {
   pdl_entry();
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(256)
   long p = L.idx(i, j, k0);
   double uc = u[p];
   Fixed c = fix_decode(uc), dn = k0 > 0 ? fix_decode(u[p - sy]) : c;
-#pragma unroll
+#pragma unroll 1
   for (int t = 0; t < KZ; ++t, p += sy) {
     const int k = k0 + t;
     const double un = k < L.n2 - 1 ? u[p + sy] : uc;

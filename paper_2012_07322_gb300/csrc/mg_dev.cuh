@@ -159,7 +159,7 @@ __device__ __forceinline__ T ghost_rule(const LevelView<T>& L, int comp, int d, 
         i = 0;
         return f;
       }
-      int ks = L.three ? (k + n2 / 2) % n2 : k;
+      const int ks = L.three ? (k + (n2 >> 1)) & (n2 - 1) : k;  // sizes are powers of two
       if (L.geom == CYL) {
         i = 0;
         k = ks;
@@ -176,7 +176,7 @@ __device__ __forceinline__ T ghost_rule(const LevelView<T>& L, int comp, int d, 
   }
   if (d == 1) {
     if (L.geom == SPH) {
-      int ks = L.three ? (k + n2 / 2) % n2 : k;
+      const int ks = L.three ? (k + (n2 >> 1)) & (n2 - 1) : k;  // sizes are powers of two
       j = (j < 0) ? 0 : n1 - 1;
       k = ks;
       return T(parity_axis(comp));

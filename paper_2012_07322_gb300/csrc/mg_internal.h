@@ -112,14 +112,17 @@ inline long ncells(const LevelView<T>& L) {
   return (long)L.n0 * L.n1 * L.n2;  // of one problem
 }
 // Blocks of a pass over all cells, and of one over the cells of one colour.
-// FP32 passes are not bound by their pipe: larger blocks.
+// FP32 passes are not bound by their pipe: a 3D block of 256 (two planes
+// deep) takes 5.8 us for the 128x64x64 colour pass, one of 32 x 8 x 1 7.0.
 template <typename T>
 inline dim3 cells_block(const LevelView<T>& L) {
-  return fit_block(L.n0, L.n1, L.n2, spread_threads(L.nb * ncells(L), sizeof(T) == 8 ? 32 : 128));
+  if (sizeof(T) == 4) return L.three ? dim3(32, 4, 2) : dim3(32, 8, 1);
+  return fit_block(L.n0, L.n1, L.n2, spread_threads(L.nb * ncells(L), 32));
 }
 template <typename T>
 inline dim3 colour_block(const LevelView<T>& L) {
-  return fit_block(L.n0 / 2, L.n1, L.n2, spread_threads(L.nb * ncells(L) / 2, sizeof(T) == 8 ? 32 : 128));
+  if (sizeof(T) == 4) return L.three ? dim3(32, 4, 2) : dim3(32, 8, 1);
+  return fit_block(L.n0 / 2, L.n1, L.n2, spread_threads(L.nb * ncells(L) / 2, 32));
 }
 // Passes that end in block maxima and atomics: at most 512 blocks until
 // they have 256 threads.
@@ -462,7 +465,10 @@ void launch_loop_decide(LoopState* S, const unsigned long long* red, const LoopP
 // the levels l0 .. l0 + nl - 1 of a hierarchy, the last the coarsest, all
 // held in the block's shared memory (same ghosted layout as in HBM).
 constexpr int BC_MAX = 8;                     // levels one block cycle may span
-constexpr long BLOCK_CYCLE_CELLS = 4096;       // levels this small run in the block cycle
+// Levels this small run in the block cycle: scalar equations from 8192 cells
+// on (a pass over 8192 cells takes one SM ~0.9 us, a launch 2.5), vector ones
+// and the batch's from 4096.
+constexpr long BLOCK_CYCLE_CELLS = 4096, BLOCK_CYCLE_CELLS_SCALAR = 8192;
 constexpr size_t BC_SMEM_MAX = 200 * 1024;     // dynamic shared memory of the block cycle
 struct BlockLevel32 {
   LevelView<float> v;        // boundary rule applied
