@@ -1,5 +1,5 @@
-// The FP64 coarsest-grid solves of mg_coarse.cuh as kernels, and the dense
-// rows of the vector solve.
+// The FP64 coarsest-grid solves of mg_coarse.cuh as kernels, and the matrix
+// the rows of the vector solve come from.
 #include "mg_coarse.cuh"
 
 namespace gmg {
@@ -35,7 +35,8 @@ bool launch_coarse_scalar_small(const LevelView<double>& L, int kind, double* u,
   return true;
 }
 
-// Rows of the coarsest vector operator for k_coarse_vec_dense: column col <
+// The coarsest vector operator as a matrix, from which the host takes the rows
+// of coarse_vec_rows: column col <
 // n of A (A[col * n + r]) is the operator (its ghost rules folded in) applied
 // to the unit field of unknown col = comp * cells + q; columns n .. n + 2
 // are the operator applied to the constant fields of each component; D[r]
@@ -71,11 +72,11 @@ __global__ void k_coarse_rows_vec(LevelView<double> L, double* __restrict__ scra
 
 template <int G>
 __global__ void __launch_bounds__(CV_THREADS)
-    k_coarse_vec_dense(LevelView<double> L, double* U, double* V, double* W, const double* f0, const double* f1,
-                       const double* f2, const double* A, const double* invD, int n, int max_sweeps) {
+    k_coarse_vec_rows(LevelView<double> L, double* U, double* V, double* W, const double* f0, const double* f1,
+                      const double* f2, const __grid_constant__ CoarseRows R, int max_sweeps) {
   pdl_entry();
   __shared__ CoarseShared sh;
-  coarse_vec_dense<G>(sh, L, U, V, W, f0, f1, f2, A, invD, n, max_sweeps);
+  coarse_vec_rows<G>(sh, L, U, V, W, f0, f1, f2, R, max_sweeps);
 }
 
 void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double* A, double* invD, int n,
@@ -89,18 +90,15 @@ void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double*
     launch_k(k_coarse_rows_vec<SPH>, n + 3, 256, 0, st, L, scratch, A, invD, n);
 }
 
-void launch_coarse_vec_dense(const LevelView<double>& L, double* const V[3], const double* const f[3],
-                             const double* A, const double* invD, int n, int max_sweeps, cudaStream_t st) {
+void launch_coarse_vec_rows(const LevelView<double>& L, double* const V[3], const double* const f[3],
+                            const CoarseRows& R, int max_sweeps, cudaStream_t st) {
   count_launch();
   if (L.geom == CART)
-    launch_k(k_coarse_vec_dense<CART>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], A, invD, n,
-             max_sweeps);
+    launch_k(k_coarse_vec_rows<CART>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R, max_sweeps);
   else if (L.geom == CYL)
-    launch_k(k_coarse_vec_dense<CYL>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], A, invD, n,
-             max_sweeps);
+    launch_k(k_coarse_vec_rows<CYL>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R, max_sweeps);
   else
-    launch_k(k_coarse_vec_dense<SPH>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], A, invD, n,
-             max_sweeps);
+    launch_k(k_coarse_vec_rows<SPH>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R, max_sweeps);
 }
 
 }  // namespace gmg

@@ -24,7 +24,8 @@ union CoarseShared {
     unsigned long long r[2];
   } scalar;
   struct {
-    double x[CV_N], f[CV_N], id[CV_N];
+    double x[CV_N + 1], old[CV_N + 1], f[CV_N], id[CV_N];
+    unsigned long long res[2];
     unsigned char colour_q[2][CV_N / 6];  // cells of each colour
   } vec;
 };
@@ -220,88 +221,125 @@ __device__ __forceinline__ void coarse_scalar_small(CoarseShared& sh, const Leve
 
 // ------------------------------------------------------ vector equations
 
-// Row r of the operator applied to x, by the g lanes of a group (g a power of
-// two up to 32): each component's entries multiply differences to that
-// component's value in the row's own cell, and the operator's action on
-// constants multiplies that value, so that, as in the flux form, smooth
-// fields are subtracted before they are multiplied.
-__device__ __forceinline__ double dense_row(const double* __restrict__ A, const double* x, int n, int cells, int r,
-                                            int q, int sub, int g, bool on) {
-  double acc = 0.0;
+// Row r of the operator applied to x, by the CV_LANES lanes of a group: entry
+// m adds cf (x[a] - x[b]), b the row's own cell in a's component (or the zero
+// behind x, for the operator's action on constants), so that, as in the flux
+// form, smooth fields are subtracted before they are multiplied.
+constexpr int CV_LANES = 4, CV_PER_LANE = 8;
+
+__device__ __forceinline__ double sparse_row(const CoarseRows& R, const double* x, int r, int sub, bool on) {
+  double s0 = 0.0, s1 = 0.0;
   if (on) {
-    for (int col = sub; col < n; col += g) {
-      const int c = (col >= cells) + (col >= 2 * cells);
-      acc += A[(long)col * n + r] * (x[col] - x[c * cells + q]);
+#pragma unroll
+    for (int m = 0; m < CV_PER_LANE; ++m) {
+      const int e = sub + CV_LANES * m;
+      if (e < R.width) {
+        const unsigned ab = R.ab[e * R.n + r];
+        const double t = x[ab & 0xffffu] - x[ab >> 16], cf = R.cf[e * R.n + r];
+        if (m & 1)
+          s1 += cf * t;
+        else
+          s0 += cf * t;
+      }
     }
-    for (int c = sub; c < 3; c += g) acc += A[(long)(n + c) * n + r] * x[c * cells + q];
   }
-  for (int o = g >> 1; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, 32);
-  return acc;
+  double s = s0 + s1;
+#pragma unroll
+  for (int o = CV_LANES >> 1; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, 32);
+  return s;
 }
 
-// The coarsest vector solve from its dense rows: a pass (colour, component)
-// computes its cells' values from the state before the pass, rows split over
-// the lanes of a group, then stores them: no ghost fills (the rules are in
-// the rows), no metric factors, chains of a few FMAs.  Sweeps and stopping
-// rule as coarse_vec_body.  4 x 2 x 2 cells: 455 -> 70 us.
-// Called by a block of CV_THREADS threads.
+// The coarsest vector solve from its rows.  A pass (colour, component)
+// computes its cells' values from the state before the pass, then stores
+// them: no ghost fills (the rules are in the rows) and no metric factors.  As
+// few warps sweep as hold the rows of a pass (one for 16 cells, no block
+// barriers then): every warp instruction costs the FP64 pipe 16 cycles, which
+// a pass spread over eight warps waits for (158 us per solve of 4 x 2 x 2
+// cells from dense rows in eight warps).  The other warps evaluate the
+// residual maximum of the state before the sweep meanwhile, as in
+// coarse_scalar_small.  Sweeps and stopping rule as coarse_vec_body; called
+// by a block of CV_THREADS threads.
 template <int G>
-__device__ __forceinline__ void coarse_vec_dense(CoarseShared& sh, const LevelView<double>& L, double* U, double* V,
-                                                 double* W, const double* f0, const double* f1, const double* f2,
-                                                 const double* __restrict__ A, const double* __restrict__ invD, int n,
-                                                 int max_sweeps) {
+__device__ __forceinline__ void coarse_vec_rows(CoarseShared& sh, const LevelView<double>& L, double* U, double* V,
+                                                double* W, const double* f0, const double* f1, const double* f2,
+                                                const CoarseRows& R, int max_sweeps) {
   auto& x = sh.vec.x;
+  auto& old = sh.vec.old;
   auto& fs = sh.vec.f;
   auto& id = sh.vec.id;
   auto& colour_q = sh.vec.colour_q;
-  const int cells = n / 3, half = cells / 2, tid = threadIdx.x;
+  const int n = R.n, cells = n / 3, half = cells / 2, tid = threadIdx.x, warp = tid >> 5;
+  const int sweepers = (half * CV_LANES + 31) / 32;  // warps; at most 4 of the 8
   for (int r = tid; r < n; r += CV_THREADS) {
-    const int c = r / cells;
+    const int c = (r >= cells) + (r >= 2 * cells);
     const long p = interior_p(L, r - c * cells);
     const double* f = c == 0 ? f0 : (c == 1 ? f1 : f2);
     x[r] = (c == 0 ? U : (c == 1 ? V : W))[p];
     fs[r] = f ? f[p] : 0.0;
-    id[r] = invD[r];
+    id[r] = R.invD[r];
   }
+  if (tid == 0) x[n] = old[n] = 0.0;
+  if (tid < 2) sh.vec.res[tid] = 0ULL;
   for (int r = tid; r < cells; r += CV_THREADS) {
     int i, j, k;
     L.colour_cell(r < half ? r : r - half, r >= half, i, j, k);
     colour_q[r >= half][r < half ? r : r - half] = (unsigned char)(i + L.n0 * (j + L.n1 * k));
   }
   __syncthreads();
-  auto resmax = [&]() -> double {
-    unsigned long long m = 0ULL;
-    constexpr int g = 8;
-    for (int base = 0; base < n; base += CV_THREADS / g) {
-      const int r = base + tid / g;
-      const int c = (r >= cells) + (r >= 2 * cells);
-      const double Lu = dense_row(A, x, n, cells, r, r - c * cells, tid % g, g, r < n);
-      if (r < n) m = umax64(m, abs_bits(fs[r] - Lu));
-    }
-    return block_max_abs(m);
+  auto pass_sync = [&] {
+    if (sweepers == 1)
+      __syncwarp();
+    else
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * sweepers) : "memory");
   };
-  const double r0 = resmax();
-  if (!(r0 > 0.0)) return;
-  int g = 32;
-  while (g > 1 && half * g > CV_THREADS) g >>= 1;
-  const int t = tid / g, sub = tid % g;
+  double r0 = 0.0;
+  bool back = false;  // the state before the last sweep is the result
   for (int it = 0; it < max_sweeps; ++it) {
-    for (int colour = 0; colour < 2; ++colour)
-      for (int c = 0; c < 3; ++c) {
-        const bool on = t < half;
-        const int q = on ? colour_q[colour][t] : 0, r = c * cells + q;
-        const double Lu = dense_row(A, x, n, cells, r, q, sub, g, on);
-        const double v = x[r] - (Lu - fs[r]) * id[r];
-        __syncthreads();
-        if (on && sub == 0) x[r] = v;
-        __syncthreads();
+    for (int r = tid; r < n; r += CV_THREADS) old[r] = x[r];
+    __syncthreads();
+    if (warp < sweepers) {
+      const int t = tid / CV_LANES, sub = tid % CV_LANES;
+      const bool on = t < half;
+      for (int colour = 0; colour < 2; ++colour) {
+        const int q = on ? colour_q[colour][t] : 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int r = c * cells + q;
+          const double Lu = sparse_row(R, x, r, sub, on);
+          const double v = x[r] - (Lu - fs[r]) * id[r];
+          pass_sync();
+          if (on && sub == 0) x[r] = v;
+          pass_sync();
+        }
       }
-    const double r = resmax();
-    if (!(r > 1e-12 * r0)) break;
+    } else {
+      const int w = tid - 32 * sweepers, rows = (CV_THREADS - 32 * sweepers) / CV_LANES, sub = w % CV_LANES;
+      unsigned long long m = 0ULL;
+      for (int base = 0; base < n; base += rows) {
+        const int r = base + w / CV_LANES;
+        const double Lu = sparse_row(R, old, r, sub, r < n);
+        if (r < n) m = umax64(m, abs_bits(fs[r] - Lu));
+      }
+      m = warp_max_bits(m);
+      if ((tid & 31) == 0) atomicMax(&sh.vec.res[it & 1], m);
+    }
+    __syncthreads();
+    // the residual before sweep it (after it sweeps)
+    const double r = __longlong_as_double((long long)sh.vec.res[it & 1]);
+    __syncthreads();
+    if (tid == 0) sh.vec.res[it & 1] = 0ULL;
+    if (it == 0) {
+      r0 = r;
+      back = !(r0 > 0.0);  // the solution already
+    } else {
+      back = !(r > 1e-12 * r0);
+    }
+    if (back) break;
   }
+  __syncthreads();
   for (int r = tid; r < n; r += CV_THREADS) {
-    const int c = r / cells;
-    (c == 0 ? U : (c == 1 ? V : W))[interior_p(L, r - c * cells)] = x[r];
+    const int c = (r >= cells) + (r >= 2 * cells);
+    (c == 0 ? U : (c == 1 ? V : W))[interior_p(L, r - c * cells)] = back ? old[r] : x[r];
   }
   __syncthreads();
   const long ngh = ghost_count(L);

@@ -100,9 +100,10 @@ struct mg_hierarchy {
   int cinv_state[3] = {0, 0, 0};
   double* cmat[3] = {};  // scalar equations: the coarsest operator per boundary rule (same states)
   int cmat_state[3] = {0, 0, 0};
-  // FP64 vector equations: dense rows of the coarsest operator and its
-  // inverted Newton diagonal per boundary rule (same states)
+  // FP64 vector equations: rows of the coarsest operator and its inverted
+  // Newton diagonal per boundary rule (same states)
   double* crow[3] = {};
+  CoarseRows crows[3] = {};
   int crow_state[3] = {0, 0, 0};
   double* d_aa_part = nullptr;  // AA_SCRATCH_DOUBLES of device scratch
   // ghost-push tables of the vector colour passes: state 0 not built, 1
@@ -695,10 +696,8 @@ void coarse64(mg_hierarchy* H, const Eq& e, int l) {
                            H->st);
   } else {
     const double* f[3] = {fptr(H, e, l, 0), fptr(H, e, l, 1), fptr(H, e, l, 2)};
-    const int n = (int)(3 * L.cells());
     if (H->crow_state[e.bc] == 1)
-      launch_coarse_vec_dense(v, L.u, f, H->crow[e.bc], H->crow[e.bc] + (size_t)(n + 3) * n, n, COARSE_SWEEPS,
-                              H->st);
+      launch_coarse_vec_rows(v, L.u, f, H->crows[e.bc], COARSE_SWEEPS, H->st);
     else
       launch_coarse_vec(v, L.u, f, COARSE_SWEEPS, H->st);
   }
@@ -1302,14 +1301,14 @@ int ensure_coarse_inverse(mg_hierarchy* H, int bc) {
   return MG_OK;
 }
 
-// FP64 vector equations: dense rows of the coarsest operator, built once per
+// FP64 vector equations: the rows of the coarsest operator, taken once per
 // boundary rule before the first cycle (outside graph capture).  Coarsest
 // levels of more than CV_N unknowns keep the stencil sweeps.
 int ensure_coarse_rows(mg_hierarchy* H, int bc) {
   if (H->crow_state[bc] != 0) return MG_OK;
   H->crow_state[bc] = -1;
   Level& Lc = H->L[H->nlev - 1];
-  const int n = (int)(3 * Lc.cells());
+  const int n = (int)(3 * Lc.cells()), cells = n / 3;
   if (n > CV_N) return MG_OK;
   double *scratch = nullptr, *d = nullptr;
   if (cudaMalloc(&scratch, sizeof(double) * 3 * (size_t)(n + 3) * Lc.ng) != cudaSuccess ||
@@ -1320,13 +1319,51 @@ int ensure_coarse_rows(mg_hierarchy* H, int bc) {
     return MG_OK;
   }
   launch_coarse_rows_vec(with_bc(Lc.v64, bc), scratch, d, d + (size_t)(n + 3) * n, n, H->st);
-  const cudaError_t ce = cudaStreamSynchronize(H->st);
+  std::vector<double> A((size_t)(n + 4) * n);
+  cudaError_t ce = cudaMemcpyAsync(A.data(), d, sizeof(double) * A.size(), cudaMemcpyDeviceToHost, H->st);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(H->st);
   cudaFree(scratch);
+  cudaFree(d);
+  if (ce != cudaSuccess) return fail(MG_ERR_CUDA, cudaGetErrorString(ce));
+  // row r: its nonzeros as differences to the row's own cell in the entry's
+  // component, then the operator's action on each component's constants
+  std::vector<std::vector<std::pair<unsigned, double>>> rows(n);
+  size_t width = 1;
+  for (int r = 0; r < n; ++r) {
+    const int q = r % cells;
+    for (int col = 0; col < n + 3; ++col) {
+      const double a = A[(size_t)col * n + r];
+      if (a == 0.0 || col == r) continue;
+      const int own = (col < n ? col / cells : col - n) * cells + q;
+      if (col < n && col == own) continue;
+      rows[r].push_back({col < n ? (unsigned)col | (unsigned)own << 16 : (unsigned)own | (unsigned)n << 16, a});
+    }
+    width = std::max(width, rows[r].size());
+  }
+  if (width > CV_WIDTH_MAX) return MG_OK;
+  // coefficients, inverted diagonal, then the index pairs
+  std::vector<double> buf(width * n + n + (width * n + 1) / 2, 0.0);
+  unsigned* ab = reinterpret_cast<unsigned*>(buf.data() + width * n + n);
+  for (size_t m = 0; m < width; ++m)
+    for (int r = 0; r < n; ++r) {
+      const bool in = m < rows[r].size();
+      buf[m * n + r] = in ? rows[r][m].second : 0.0;
+      ab[m * n + r] = in ? rows[r][m].first : (unsigned)n | (unsigned)n << 16;
+    }
+  for (int r = 0; r < n; ++r) buf[width * n + r] = A[(size_t)(n + 3) * n + r];
+  double* o = nullptr;
+  if (cudaMalloc(&o, sizeof(double) * buf.size()) != cudaSuccess) {
+    cudaGetLastError();
+    return MG_OK;
+  }
+  ce = cudaMemcpyAsync(o, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice, H->st);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(H->st);
   if (ce != cudaSuccess) {
-    cudaFree(d);
+    cudaFree(o);
     return fail(MG_ERR_CUDA, cudaGetErrorString(ce));
   }
-  H->crow[bc] = d;
+  H->crow[bc] = o;
+  H->crows[bc] = CoarseRows{n, (int)width, reinterpret_cast<const unsigned*>(o + width * n + n), o, o + width * n};
   H->crow_state[bc] = 1;
   return MG_OK;
 }

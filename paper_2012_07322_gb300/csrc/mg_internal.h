@@ -279,16 +279,23 @@ void launch_coarse_scalar(const LevelView<T>& L, int kind, T* u, const T* f, con
                           int max_sweeps, cudaStream_t st);
 // The same FP64 solves on coarsest levels of a few dozen cells (mg_coarse.cu):
 // scalar equations in two warps (false when the level is larger); vector
-// equations from dense rows of the operator (A: n + 3 columns of n, n = 3 x
-// cells at most CV_N, and the inverted Newton diagonal), built once per
-// hierarchy and boundary rule; scratch holds 3 (n + 3) ghosted fields.
+// equations from the nonzeros of the operator's rows, taken once per hierarchy
+// and boundary rule from its matrix (A: n + 3 columns of n, n = 3 x cells at
+// most CV_N; scratch holds 3 (n + 3) ghosted fields).
 constexpr int CV_N = 192;
+constexpr int CV_WIDTH_MAX = 32;  // entries per row
+struct CoarseRows {
+  int n, width;
+  const unsigned* ab;  // [width][n]: a | b << 16 of cf (x[a] - x[b]); index n is a zero
+  const double* cf;    // [width][n]
+  const double* invD;  // [n]: the inverted Newton diagonal (ghosts held fixed)
+};
 bool launch_coarse_scalar_small(const LevelView<double>& L, int kind, double* u, const double* f, const double* s0,
                                 const double* s1, int max_sweeps, cudaStream_t st);
 void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double* A, double* invD, int n,
                             cudaStream_t st);
-void launch_coarse_vec_dense(const LevelView<double>& L, double* const V[3], const double* const f[3],
-                             const double* A, const double* invD, int n, int max_sweeps, cudaStream_t st);
+void launch_coarse_vec_rows(const LevelView<double>& L, double* const V[3], const double* const f[3],
+                            const CoarseRows& R, int max_sweeps, cudaStream_t st);
 
 // The FP64 FAS V-cycle of a scalar equation on small levels in one cluster launch (mg_fas.cu):
 // levels lv[0 .. nl - 1], the last the coarsest; from solo_from on (at most
