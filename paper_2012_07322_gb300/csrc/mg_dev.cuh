@@ -296,7 +296,7 @@ __device__ __forceinline__ T lap_scalar(const LevelView<T>& L, const T* __restri
     nb.up = L.three ? u[p + L.sy] : uc;
     nb.dn = L.three ? u[p - L.sy] : uc;
   } else if constexpr (INNER) {
-  } else if constexpr (sizeof(T) == 4) {
+  } else if constexpr (sizeof(T) == 4 || G == SPH) {
     // FP32: the edge rules inline (speculating them costs the FP32 units
     // little; a call passes the neighbours through local memory)
     nb = lap_edge_neighbours_body<T, G>(L, u, i, j, k, p);

@@ -107,17 +107,25 @@ template <int G, int KIND>
 __global__ void __launch_bounds__(FAS_THREADS) k_fas_cycle(const __grid_constant__ FasCycle P) {
   pdl_entry();
   __shared__ CoarseShared cs;
+  // the levels in shared memory: handed by reference to the out-of-line edge
+  // rules, a kernel parameter would be read through the generic address of
+  // the constant bank, a dependent load per field
+  __shared__ __align__(16) unsigned char lv_raw[sizeof(FasLevel) * FAS_MAX];
+  FasLevel* const lv = reinterpret_cast<FasLevel*>(lv_raw);
+  for (int q = threadIdx.x; q < (int)(sizeof(FasLevel) / 4) * P.nl; q += FAS_THREADS)
+    reinterpret_cast<unsigned*>(lv_raw)[q] = reinterpret_cast<const unsigned*>(P.lv)[q];
+  __syncthreads();
   const int rank = (int)cg::this_cluster().block_rank(), size = (int)cg::this_cluster().num_blocks();
   const FasTeam all{rank, size}, solo{rank, 1};
   // levels solo_from .. nl - 1 run on block 0
   for (int l = 0; l + 1 < P.nl; ++l) {
     const FasTeam T = l < P.solo_from ? all : solo, TC = l + 1 < P.solo_from ? all : solo;
     if (rank >= T.size) break;
-    fas_smooth<G, KIND>(T, P.lv[l], P.nu1);
-    fas_down<G, KIND>(T, TC, P.lv[l], P.lv[l + 1]);
+    fas_smooth<G, KIND>(T, lv[l], P.nu1);
+    fas_down<G, KIND>(T, TC, lv[l], lv[l + 1]);
   }
   if (rank == 0) {
-    const FasLevel& C = P.lv[P.nl - 1];
+    const FasLevel& C = lv[P.nl - 1];
     coarse_scalar_small<G, KIND>(cs, C.v, C.u, C.f, C.s0, C.s1, P.coarse_sweeps);
     __syncthreads();
   }
@@ -126,8 +134,8 @@ __global__ void __launch_bounds__(FAS_THREADS) k_fas_cycle(const __grid_constant
     if (rank >= T.size) continue;
     // block 0 hands the coarse level over to the cluster
     if (T.size > 1 && l + 1 >= P.solo_from) T.sync();
-    fas_up(T, P.lv[l], P.lv[l + 1]);
-    fas_smooth<G, KIND>(T, P.lv[l], P.nu2);
+    fas_up(T, lv[l], lv[l + 1]);
+    fas_smooth<G, KIND>(T, lv[l], P.nu2);
   }
 }
 
