@@ -73,10 +73,10 @@ __global__ void k_coarse_rows_vec(LevelView<double> L, double* __restrict__ scra
 template <int G>
 __global__ void __launch_bounds__(CV_THREADS)
     k_coarse_vec_rows(LevelView<double> L, double* U, double* V, double* W, const double* f0, const double* f1,
-                      const double* f2, const __grid_constant__ CoarseRows R, int max_sweeps) {
+                      const double* f2, const __grid_constant__ CoarseRows R) {
   pdl_entry();
   __shared__ CoarseShared sh;
-  coarse_vec_rows<G>(sh, L, U, V, W, f0, f1, f2, R, max_sweeps);
+  coarse_vec_rows<G>(sh, L, U, V, W, f0, f1, f2, R);
 }
 
 void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double* A, double* invD, int n,
@@ -91,14 +91,14 @@ void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double*
 }
 
 void launch_coarse_vec_rows(const LevelView<double>& L, double* const V[3], const double* const f[3],
-                            const CoarseRows& R, int max_sweeps, cudaStream_t st) {
+                            const CoarseRows& R, cudaStream_t st) {
   count_launch();
   if (L.geom == CART)
-    launch_k(k_coarse_vec_rows<CART>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R, max_sweeps);
+    launch_k(k_coarse_vec_rows<CART>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R);
   else if (L.geom == CYL)
-    launch_k(k_coarse_vec_rows<CYL>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R, max_sweeps);
+    launch_k(k_coarse_vec_rows<CYL>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R);
   else
-    launch_k(k_coarse_vec_rows<SPH>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R, max_sweeps);
+    launch_k(k_coarse_vec_rows<SPH>, 1, CV_THREADS, 0, st, L, V[0], V[1], V[2], f[0], f[1], f[2], R);
 }
 
 }  // namespace gmg

@@ -24,9 +24,7 @@ union CoarseShared {
     unsigned long long r[2];
   } scalar;
   struct {
-    double x[CV_N + 1], old[CV_N + 1], f[CV_N], id[CV_N];
-    unsigned long long res[2];
-    unsigned char colour_q[2][CV_N / 6];  // cells of each colour
+    double x[CV_N + 1], r[CV_N];
   } vec;
 };
 
@@ -249,97 +247,54 @@ __device__ __forceinline__ double sparse_row(const CoarseRows& R, const double* 
   return s;
 }
 
-// The coarsest vector solve from its rows.  A pass (colour, component)
-// computes its cells' values from the state before the pass, then stores
-// them: no ghost fills (the rules are in the rows) and no metric factors.  As
-// few warps sweep as hold the rows of a pass (one for 16 cells, no block
-// barriers then): every warp instruction costs the FP64 pipe 16 cycles, which
-// a pass spread over eight warps waits for (158 us per solve of 4 x 2 x 2
-// cells from dense rows in eight warps).  The other warps evaluate the
-// residual maximum of the state before the sweep meanwhile, as in
-// coarse_scalar_small.  Sweeps and stopping rule as coarse_vec_body; called
-// by a block of CV_THREADS threads.
+// The coarsest vector solve.  The sweeps of a linear equation are one affine
+// map of the state: u + S (f - A u), S the sum of the sweeps' response to a
+// residual, which the host tabulates by sweeping the rows on unit residuals
+// (CoarseRows).  What is left is one residual and one product with S, two
+// short FP64 chains in place of max_sweeps x 6 dependent passes: 158 us per
+// solve of 4 x 2 x 2 cells from dense rows, 106 us swept from the nonzeros.
+// The sweeps' early stop (residual down 1e-12 x) has no counterpart: past it
+// a sweep moves u by less than that.  Called by a block of CV_THREADS threads.
 template <int G>
 __device__ __forceinline__ void coarse_vec_rows(CoarseShared& sh, const LevelView<double>& L, double* U, double* V,
                                                 double* W, const double* f0, const double* f1, const double* f2,
-                                                const CoarseRows& R, int max_sweeps) {
+                                                const CoarseRows& R) {
   auto& x = sh.vec.x;
-  auto& old = sh.vec.old;
-  auto& fs = sh.vec.f;
-  auto& id = sh.vec.id;
-  auto& colour_q = sh.vec.colour_q;
-  const int n = R.n, cells = n / 3, half = cells / 2, tid = threadIdx.x, warp = tid >> 5;
-  const int sweepers = (half * CV_LANES + 31) / 32;  // warps; at most 4 of the 8
+  auto& res = sh.vec.r;
+  const int n = R.n, cells = n / 3, tid = threadIdx.x, t = tid / CV_LANES, sub = tid % CV_LANES;
+  constexpr int rows = CV_THREADS / CV_LANES;
   for (int r = tid; r < n; r += CV_THREADS) {
     const int c = (r >= cells) + (r >= 2 * cells);
     const long p = interior_p(L, r - c * cells);
     const double* f = c == 0 ? f0 : (c == 1 ? f1 : f2);
     x[r] = (c == 0 ? U : (c == 1 ? V : W))[p];
-    fs[r] = f ? f[p] : 0.0;
-    id[r] = R.invD[r];
+    res[r] = f ? f[p] : 0.0;
   }
-  if (tid == 0) x[n] = old[n] = 0.0;
-  if (tid < 2) sh.vec.res[tid] = 0ULL;
-  for (int r = tid; r < cells; r += CV_THREADS) {
-    int i, j, k;
-    L.colour_cell(r < half ? r : r - half, r >= half, i, j, k);
-    colour_q[r >= half][r < half ? r : r - half] = (unsigned char)(i + L.n0 * (j + L.n1 * k));
+  if (tid == 0) x[n] = 0.0;
+  __syncthreads();
+  for (int base = 0; base < n; base += rows) {
+    const int r = base + t;
+    const double Lu = sparse_row(R, x, r, sub, r < n);
+    if (r < n && sub == 0) res[r] -= Lu;
   }
   __syncthreads();
-  auto pass_sync = [&] {
-    if (sweepers == 1)
-      __syncwarp();
-    else
-      asm volatile("bar.sync 1, %0;" ::"r"(32 * sweepers) : "memory");
-  };
-  double r0 = 0.0;
-  bool back = false;  // the state before the last sweep is the result
-  for (int it = 0; it < max_sweeps; ++it) {
-    for (int r = tid; r < n; r += CV_THREADS) old[r] = x[r];
-    __syncthreads();
-    if (warp < sweepers) {
-      const int t = tid / CV_LANES, sub = tid % CV_LANES;
-      const bool on = t < half;
-      for (int colour = 0; colour < 2; ++colour) {
-        const int q = on ? colour_q[colour][t] : 0;
+  for (int base = 0; base < n; base += rows) {
+    const int r = base + t;
+    double s0 = 0.0, s1 = 0.0;
+    if (r < n) {
+      const double* __restrict__ S = R.S + r;
+      for (int q = sub; q < n; q += 2 * CV_LANES) {
+        s0 += S[(long)q * n] * res[q];
+        if (q + CV_LANES < n) s1 += S[(long)(q + CV_LANES) * n] * res[q + CV_LANES];
+      }
+    }
+    double s = s0 + s1;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const int r = c * cells + q;
-          const double Lu = sparse_row(R, x, r, sub, on);
-          const double v = x[r] - (Lu - fs[r]) * id[r];
-          pass_sync();
-          if (on && sub == 0) x[r] = v;
-          pass_sync();
-        }
-      }
-    } else {
-      const int w = tid - 32 * sweepers, rows = (CV_THREADS - 32 * sweepers) / CV_LANES, sub = w % CV_LANES;
-      unsigned long long m = 0ULL;
-      for (int base = 0; base < n; base += rows) {
-        const int r = base + w / CV_LANES;
-        const double Lu = sparse_row(R, old, r, sub, r < n);
-        if (r < n) m = umax64(m, abs_bits(fs[r] - Lu));
-      }
-      m = warp_max_bits(m);
-      if ((tid & 31) == 0) atomicMax(&sh.vec.res[it & 1], m);
+    for (int o = CV_LANES >> 1; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, 32);
+    if (r < n && sub == 0) {
+      const int c = (r >= cells) + (r >= 2 * cells);
+      (c == 0 ? U : (c == 1 ? V : W))[interior_p(L, r - c * cells)] = x[r] + s;
     }
-    __syncthreads();
-    // the residual before sweep it (after it sweeps)
-    const double r = __longlong_as_double((long long)sh.vec.res[it & 1]);
-    __syncthreads();
-    if (tid == 0) sh.vec.res[it & 1] = 0ULL;
-    if (it == 0) {
-      r0 = r;
-      back = !(r0 > 0.0);  // the solution already
-    } else {
-      back = !(r > 1e-12 * r0);
-    }
-    if (back) break;
-  }
-  __syncthreads();
-  for (int r = tid; r < n; r += CV_THREADS) {
-    const int c = (r >= cells) + (r >= 2 * cells);
-    (c == 0 ? U : (c == 1 ? V : W))[interior_p(L, r - c * cells)] = back ? old[r] : x[r];
   }
   __syncthreads();
   const long ngh = ghost_count(L);

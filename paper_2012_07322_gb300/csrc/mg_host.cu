@@ -697,7 +697,7 @@ void coarse64(mg_hierarchy* H, const Eq& e, int l) {
   } else {
     const double* f[3] = {fptr(H, e, l, 0), fptr(H, e, l, 1), fptr(H, e, l, 2)};
     if (H->crow_state[e.bc] == 1)
-      launch_coarse_vec_rows(v, L.u, f, H->crows[e.bc], COARSE_SWEEPS, H->st);
+      launch_coarse_vec_rows(v, L.u, f, H->crows[e.bc], H->st);
     else
       launch_coarse_vec(v, L.u, f, COARSE_SWEEPS, H->st);
   }
@@ -1341,16 +1341,41 @@ int ensure_coarse_rows(mg_hierarchy* H, int bc) {
     width = std::max(width, rows[r].size());
   }
   if (width > CV_WIDTH_MAX) return MG_OK;
-  // coefficients, inverted diagonal, then the index pairs
-  std::vector<double> buf(width * n + n + (width * n + 1) / 2, 0.0);
-  unsigned* ab = reinterpret_cast<unsigned*>(buf.data() + width * n + n);
+  // coefficients, the sweeps' response, then the index pairs
+  const size_t nn = (size_t)n * n;
+  std::vector<double> buf(width * n + nn + (width * n + 1) / 2, 0.0);
+  unsigned* ab = reinterpret_cast<unsigned*>(buf.data() + width * n + nn);
   for (size_t m = 0; m < width; ++m)
     for (int r = 0; r < n; ++r) {
       const bool in = m < rows[r].size();
       buf[m * n + r] = in ? rows[r][m].second : 0.0;
       ab[m * n + r] = in ? rows[r][m].first : (unsigned)n | (unsigned)n << 16;
     }
-  for (int r = 0; r < n; ++r) buf[width * n + r] = A[(size_t)(n + 3) * n + r];
+  // column col: COARSE_SWEEPS sweeps of A x = unit residual col from x = 0, by
+  // the passes (colour, component) of the stencil sweeps, each from the state
+  // before it
+  const double* invD = A.data() + (size_t)(n + 3) * n;
+  std::vector<int> pass[2];
+  for (int q = 0; q < cells; ++q) {
+    const int i = q & (Lc.v64.n0 - 1), j = (q >> Lc.v64.ln0) & (Lc.v64.n1 - 1), k = q >> (Lc.v64.ln0 + Lc.v64.ln1);
+    pass[(i + j + k) & 1].push_back(q);
+  }
+  std::vector<double> x(n + 1), y(cells);
+  for (int col = 0; col < n; ++col) {
+    std::fill(x.begin(), x.end(), 0.0);
+    for (int p = 0; p < 6 * COARSE_SWEEPS; ++p) {
+      const int at = p % 3 * cells;
+      const std::vector<int>& cellsp = pass[p / 3 % 2];
+      for (int q : cellsp) {
+        const int r = at + q;
+        double Lu = r == col ? -1.0 : 0.0;
+        for (const auto& e : rows[r]) Lu += e.second * (x[e.first & 0xffffu] - x[e.first >> 16]);
+        y[q] = x[r] - Lu * invD[r];
+      }
+      for (int q : cellsp) x[at + q] = y[q];
+    }
+    std::copy(x.begin(), x.begin() + n, buf.begin() + width * n + (size_t)col * n);
+  }
   double* o = nullptr;
   if (cudaMalloc(&o, sizeof(double) * buf.size()) != cudaSuccess) {
     cudaGetLastError();
@@ -1363,7 +1388,7 @@ int ensure_coarse_rows(mg_hierarchy* H, int bc) {
     return fail(MG_ERR_CUDA, cudaGetErrorString(ce));
   }
   H->crow[bc] = o;
-  H->crows[bc] = CoarseRows{n, (int)width, reinterpret_cast<const unsigned*>(o + width * n + n), o, o + width * n};
+  H->crows[bc] = CoarseRows{n, (int)width, reinterpret_cast<const unsigned*>(o + width * n + nn), o, o + width * n};
   H->crow_state[bc] = 1;
   return MG_OK;
 }

@@ -288,14 +288,14 @@ struct CoarseRows {
   int n, width;
   const unsigned* ab;  // [width][n]: a | b << 16 of cf (x[a] - x[b]); index n is a zero
   const double* cf;    // [width][n]
-  const double* invD;  // [n]: the inverted Newton diagonal (ghosts held fixed)
+  const double* S;     // [col][row]: response of the sweeps (from zero) to a unit residual
 };
 bool launch_coarse_scalar_small(const LevelView<double>& L, int kind, double* u, const double* f, const double* s0,
                                 const double* s1, int max_sweeps, cudaStream_t st);
 void launch_coarse_rows_vec(const LevelView<double>& L, double* scratch, double* A, double* invD, int n,
                             cudaStream_t st);
 void launch_coarse_vec_rows(const LevelView<double>& L, double* const V[3], const double* const f[3],
-                            const CoarseRows& R, int max_sweeps, cudaStream_t st);
+                            const CoarseRows& R, cudaStream_t st);
 
 // The FP64 FAS V-cycle of a scalar equation on small levels in one cluster launch (mg_fas.cu):
 // levels lv[0 .. nl - 1], the last the coarsest; from solo_from on (at most
