@@ -752,9 +752,9 @@ void fas_up64(mg_hierarchy* H, const Eq& e, int l) {
 // most FAS_CLUSTER_CELLS cells, at least two levels, a coarsest level its
 // solves take; nlev when there is none.
 int fas_cluster_level(const mg_hierarchy* H, const Eq& e) {
-  if (e.kind == EQ_VEC || !fas_cycle_available() || H->L[H->nlev - 1].cells() > CS_CELLS) return H->nlev;
+  if (e.kind == EQ_VEC || H->L[H->nlev - 1].cells() > CS_CELLS) return H->nlev;
   for (int l = std::max(0, H->nlev - FAS_MAX); l + 1 < H->nlev; ++l)
-    if (H->L[l].cells() <= FAS_CLUSTER_CELLS) return l;
+    if (H->L[l].cells() <= fas_cycle_cells()) return l;
   return H->nlev;
 }
 

@@ -313,7 +313,7 @@ struct FasCycle {
   FasLevel lv[FAS_MAX];
 };
 void init_fas_attributes();   // once a device is current, before any capture
-bool fas_cycle_available();
+long fas_cycle_cells();       // cells of the largest level the cycle takes, 0: not available
 void launch_fas_cycle(const FasCycle& P, int geom, int kind, cudaStream_t st);
 constexpr int CS_CELLS = 64;  // scalar coarsest levels the cycle solves
 template <typename T>
