@@ -82,9 +82,11 @@ struct LevelView {
   // The z block index of a launch over all problems (grid.z = problems x
   // blocks of one), split into the block within a problem (returned) and the
   // problem's offset in this level's arrays.
+  // NB false: there is one problem.
+  template <bool NB = true>
   __device__ __forceinline__ int z_block(int& b) const {
     b = 0;
-    if (nb == 1) return blockIdx.z;
+    if (!NB || nb == 1) return blockIdx.z;
     const int gz = gridDim.z / nb;
     b = blockIdx.z / gz;
     return blockIdx.z - b * gz;

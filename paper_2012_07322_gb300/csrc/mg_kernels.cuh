@@ -299,6 +299,54 @@ __device__ __forceinline__ void prolong_cell(const LevelView<T>& F, const LevelV
   u[F.idx(i, j, k)] += add;
 }
 
+// prolong_cell for several components: the parent's neighbours and their rules
+// resolved once.  A rule's index is the same for every component; its sign
+// differs across the origin and the axis only.  (The rules inlined per
+// component and neighbour made the 64x32x32 FP64 vector pass 19 us, most of
+// it instruction fetch; @@ us so.)
+template <typename T>
+struct ProlongNb {
+  long q[4];  // parent, its neighbour in each dimension
+  T f[3];     // outer factor
+  int par[3]; // 1: across the origin, 2: the axis
+  __device__ __forceinline__ ProlongNb(const LevelView<T>& F, const LevelView<T>& C, int i, int j, int k) {
+    const int I = i >> 1, J = j >> 1, K = F.three ? (k >> 1) : 0;
+    q[0] = C.idx(I, J, K);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      int a = I, b = J, c = K;
+      if (d == 0)
+        a += (i & 1) ? 1 : -1;
+      else if (d == 1)
+        b += (j & 1) ? 1 : -1;
+      else if (F.three)
+        c += (k & 1) ? 1 : -1;
+      f[d] = T(1);
+      par[d] = 0;
+      if (d == 0 ? (a < 0 || a >= C.n0) : (d == 1 ? (b < 0 || b >= C.n1) : (F.three && (c < 0 || c >= C.n2)))) {
+        if (d == 0 && a < 0 && C.geom != CART) par[d] = 1;
+        if (d == 1 && C.geom == SPH) par[d] = 2;
+        f[d] = ghost_rule(C, -1, d, a, b, c);
+      }
+      q[d + 1] = C.idx(a, b, c);
+    }
+  }
+};
+template <typename T>
+__device__ __forceinline__ void prolong_nb(const LevelView<T>& F, const ProlongNb<T>& N, T* __restrict__ u,
+                                           const T* __restrict__ uH, const T* __restrict__ uhH, int comp, long p) {
+  auto e = [&](long q) { return uhH ? uH[q] - uhH[q] : uH[q]; };
+  auto nb = [&](int d) {
+    const T s = N.par[d] == 1 ? T(parity_origin(comp)) : (N.par[d] == 2 ? T(parity_axis(comp)) : N.f[d]);
+    return s * e(N.q[d + 1]);
+  };
+  const T ec = e(N.q[0]), ex = nb(0), ey = nb(1);
+  if (F.three)
+    u[p] += T(0.25) * (ec + ex + ey + nb(2));
+  else
+    u[p] += T(0.25) * (T(2) * ec + ex + ey);
+}
+
 // ----------------------------------------------------------- coarsest grid
 
 constexpr int COARSE_INV_MAX = 1024;      // scalar cells with a cached inverse diagonal
