@@ -111,9 +111,9 @@ __device__ __forceinline__ void bc_cp16(float* dst, const float* src) {
 
 // Copies of every level's coefficient tables into shared memory
 // (asynchronous: bc_run waits); they do not change during a solve.
-__device__ __forceinline__ void bc_stage_tables(const BlockCycle32& P) {
+__device__ __forceinline__ void bc_stage_tables(const BlockCycle32& P, int from = 0) {
   float* sm = bc_smem();
-  for (int l = 0; l < P.nl; ++l) {
+  for (int l = from; l < P.nl; ++l) {
     const BlockLevel32& B = P.lv[l];
     const int nti = NTI * (B.v.n0 + 2), ntj = NTJ * (B.v.n1 + 2);
     for (int q = threadIdx.x; q < nti; q += BC_THREADS) bc_cp4(sm + B.ti_at + q, B.v.ti + q);
@@ -121,14 +121,24 @@ __device__ __forceinline__ void bc_stage_tables(const BlockCycle32& P) {
   }
 }
 
+// c of levels from .. to - 1 from HBM (asynchronous).
+__device__ __forceinline__ void bc_stage_k(const BlockCycle32& P, int from, int to = BC_MAX) {
+  for (int l = from; l < P.nl && l < to; ++l)
+    if (P.lv[l].k32) {
+      const int ng = (int)(P.lv[l].v.sy * (P.lv[l].v.n2 + 2 * P.lv[l].v.three));
+      float* k = bc_smem() + P.lv[l].k_at;
+      for (int q = threadIdx.x; q < ng / 4; q += BC_THREADS) bc_cp16(k + 4 * q, P.lv[l].k32 + 4 * q);
+    }
+}
+
 // Ghost rules of every level, evaluated once per cycle: scalar levels with a
 // position-dependent outer factor (Cartesian and cylindrical Robin), the
 // factors per face; vector levels, the source and the signs of every ghost
 // (+-1 times an interior cell; with the Robin rule a factor as well).
 template <int G, bool VEC>
-__device__ __forceinline__ void bc_rules(const BlockCycle32& P) {
+__device__ __forceinline__ void bc_rules(const BlockCycle32& P, int from = 0) {
   float* sm = bc_smem();
-  for (int l = 0; l < P.nl; ++l) {
+  for (int l = from; l < P.nl; ++l) {
     const BlockLevel32& B = P.lv[l];
     const LevelView<float>& L = B.v;
     if (VEC) {
@@ -555,6 +565,26 @@ __device__ void bc_coarse(const BlockCycle32& P, const BcLevel& B) {
   }
 }
 
+// The cycle from level from of P down and back, its right-hand side and zero
+// correction in shared memory.
+template <int G, bool VEC, bool DENSE_ONLY = false>
+__device__ __forceinline__ void bc_levels(const BlockCycle32& P, int from) {
+  // down: pre-smooth, residual restricted into the next level's right-hand
+  // side, zero correction there
+  for (int l = from; l + 1 < P.nl; ++l) {
+    const BcLevel F = bc_level<VEC>(P, l);
+    bc_smooth<G, VEC>(F, P.nu1);
+    bc_down<G, VEC>(F, bc_level<VEC>(P, l + 1), P.fold_k);
+  }
+  bc_coarse<G, VEC, DENSE_ONLY>(P, bc_level<VEC>(P, P.nl - 1));
+  // up: Kwak prolongation of the correction, post-smooth
+  for (int l = P.nl - 2; l >= from; --l) {
+    const BcLevel F = bc_level<VEC>(P, l);
+    bc_up<G, VEC>(F, bc_level<VEC>(P, l + 1));
+    bc_smooth<G, VEC>(F, P.nu2);
+  }
+}
+
 // The whole cycle from level l0 of P: its right-hand side in from P.f_in,
 // the correction out to P.e_out (ghosts included).  No barrier after the
 // final stores.  DENSE_ONLY: P carries the dense coarsest operator (cA) or
@@ -574,31 +604,12 @@ __device__ void bc_run(const BlockCycle32& P, long problem_at = 0) {
       for (int q = threadIdx.x; q < (int)P.ng0 / 4; q += BC_THREADS) bc_cp16(B.f[c] + 4 * q, P.f_in[c] + problem_at + 4 * q);
       for (int q = threadIdx.x; q < (int)P.ng0; q += BC_THREADS) B.e[c][q] = 0.0f;
     }
-    if (!VEC)
-      for (int l = 0; l < (P.fold_k ? 1 : P.nl); ++l)
-        if (P.lv[l].k32) {
-          const int ng = (int)(P.lv[l].v.sy * (P.lv[l].v.n2 + 2 * P.lv[l].v.three));
-          float* k = bc_smem() + P.lv[l].k_at;
-          for (int q = threadIdx.x; q < ng / 4; q += BC_THREADS) bc_cp16(k + 4 * q, P.lv[l].k32 + 4 * q);
-        }
+    if (!VEC) bc_stage_k(P, 0, P.fold_k ? 1 : BC_MAX);
     bc_rules<G, VEC>(P);
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
   }
-  // down: pre-smooth, residual restricted into the next level's right-hand
-  // side, zero correction there
-  for (int l = 0; l + 1 < P.nl; ++l) {
-    const BcLevel F = bc_level<VEC>(P, l);
-    bc_smooth<G, VEC>(F, P.nu1);
-    bc_down<G, VEC>(F, bc_level<VEC>(P, l + 1), P.fold_k);
-  }
-  bc_coarse<G, VEC, DENSE_ONLY>(P, bc_level<VEC>(P, P.nl - 1));
-  // up: Kwak prolongation of the correction, post-smooth
-  for (int l = P.nl - 2; l >= 0; --l) {
-    const BcLevel F = bc_level<VEC>(P, l);
-    bc_up<G, VEC>(F, bc_level<VEC>(P, l + 1));
-    bc_smooth<G, VEC>(F, P.nu2);
-  }
+  bc_levels<G, VEC, DENSE_ONLY>(P, 0);
   // level l0 correction out (ghosts included)
   const BcLevel B = bc_level<VEC>(P, 0);
 #pragma unroll

@@ -48,6 +48,7 @@ struct Level {
   float* tj32 = nullptr;
   double *u[3] = {}, *uh[3] = {}, *f[3] = {}, *r[3] = {}, *s0 = nullptr, *s1 = nullptr;
   float *e[3] = {}, *f32[3] = {}, *k32 = nullptr;
+  ClusterLevel32 cluster{};  // readers' tables of a vector level on a cluster (mask, list, start), or empty
   GhostPush push[3][2];  // per component and colour (Dirichlet-0 ghosts), or empty
   // tensor maps of the FP32 one-launch sweep (inputs e[leg], f32[0], k32)
   // per sweep leg, when the level stages its planes with them
@@ -110,6 +111,9 @@ struct mg_hierarchy {
   // built, -1 unavailable; one device buffer holds every level's tables
   int push_state = 0;
   int* push_buf = nullptr;
+  // readers' tables of the vector levels that run on a cluster
+  int cluster_state = 0;
+  unsigned char* cluster_buf = nullptr;
   // MG_DIVB_EXACT: the hierarchy of the parity-class problems (n / 2 cells
   // per dimension), on this hierarchy's stream
   mg_hierarchy* sub = nullptr;
@@ -348,8 +352,10 @@ size_t layout(mg_hierarchy* H, const mg_grid_desc* d, char* base, int nb = 1) {
     t64(L ? &L->ti64 : &dummy64, sizeof(double) * NTI * (n[l][0] + 2));
     t64(L ? &L->tj64 : &dummy64, sizeof(double) * NTJ * (n[l][1] + 2));
     t32(L ? &L->ti32 : &dummy32, sizeof(float) * NTI * (n[l][0] + 2));
-    if (d->geom != MG_SPH && d->mixed_deriv == MG_MIXED_4PT)
+    if (d->geom != MG_SPH && d->mixed_deriv == MG_MIXED_4PT) {
       t64(L ? &L->vc64 : &dummy64, sizeof(double) * (d->geom == MG_CYL ? VY_N * n[l][0] : VX_N));
+      if (mixed) t32(L ? &L->vc32 : &dummy32, sizeof(float) * (d->geom == MG_CYL ? VY_N * n[l][0] : VX_N));
+    }
     if (d->geom == MG_SPH && d->mixed_deriv == MG_MIXED_4PT) {
       t64(L ? &L->vc64 : &dummy64, sizeof(double) * VC_N * n[l][0] * n[l][1]);
       if (mixed) t32(L ? &L->vc32 : &dummy32, sizeof(float) * VC_N * n[l][0] * n[l][1]);
@@ -940,10 +946,20 @@ void coarse32(mg_hierarchy* H, const Eq& e, int l) {
   if (e.kind == EQ_VEC) launch_fill_ghosts3<float>(with_bc(L.v32, e.bc), L.e, 3, 1, H->st);
 }
 
+template <typename T>
+void unpad(LevelView<T>& v) {
+  v.sx = v.n0 + 2;
+  v.sy = v.sx * (v.n1 + 2);
+  v.off = 1 + v.sx + (v.three ? v.sy : 0);
+}
+
 // Parameters of the one-block coarse cycle from level l0 (mg_block.cu):
 // shared-memory offsets of every level's arrays; P.smem = 0 when they do
 // not fit.
-BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0) {
+// top: level l0 runs on a cluster, and only its correction is held here (with
+// what the cluster needs besides at w_at); vector levels without the padding
+// of their rows.
+BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0, bool top = false, int* w_at = nullptr) {
   BlockCycle32 P{};
   const bool hasK = e.kind == EQ_PSI || e.has_c;
   const int nc = e.kind == EQ_VEC ? 3 : 1;
@@ -963,10 +979,15 @@ BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0) {
     Level& L = H->L[l0 + q];
     BlockLevel32& B = P.lv[q];
     B.v = with_bc(L.v32, e.bc);
+    if (top && P.vec) unpad(B.v);
+    const long ng = top && P.vec ? B.v.sy * (B.v.n2 + 2 * B.v.three) : L.ng;
+    if (q == 0) P.ng0 = (ng + 3) & ~3L;
     for (int c = 0; c < 3; ++c) {
-      B.e[c] = c < nc ? take(L.ng) : B.e[0];
-      B.f32[c] = c < nc ? take(L.ng) : B.f32[0];
+      B.e[c] = c < nc ? take(ng) : B.e[0];
+      if (top && q == 0) continue;
+      B.f32[c] = c < nc ? take(ng) : B.f32[0];
     }
+    if (top && q == 0) continue;
     B.k32 = hasK ? L.k32 : nullptr;
     B.ti_at = take((long)NTI * (L.n[0] + 2));
     B.tj_at = take((long)NTJ * (L.n[1] + 2));
@@ -989,8 +1010,10 @@ BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0) {
       B.gf_at = take(at);
     }
   }
+  if (w_at) *w_at = take(3 * 512);
   Level& Lc = H->L[H->nlev - 1];
   P.c64 = with_bc(Lc.v64, e.bc);
+  if (top && P.vec) unpad(P.c64);
   P.fp64_at = (long)sizeof(float) * fl;
   long dl = 0;  // doubles
   auto taked = [&](long n) {
@@ -1012,13 +1035,12 @@ BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0) {
     P.cn = (int)Lc.cells();
   }
   Level& L0 = H->L[l0];
-  P.ng0 = L0.ng;
   for (int c = 0; c < 3; ++c) {
     P.f_in[c] = L0.f32[c];
     P.e_out[c] = L0.e[c];
   }
   const size_t bytes = (size_t)P.fp64_at + sizeof(double) * (size_t)dl;
-  P.smem = bytes <= BC_SMEM_MAX ? bytes : 0;
+  P.smem = bytes <= (top ? CL_SMEM_MAX : BC_SMEM_MAX) ? bytes : 0;
   return P;
 }
 
@@ -1046,8 +1068,53 @@ void block_vcycle32(mg_hierarchy* H, const Eq& e, int l0) {
   prof_end(H, tok);
 }
 
+// The level of the cycle that a cluster takes (mg_clus.cu), -1 for none: the
+// first of CL_CELLS_MIN .. CL_CELLS_MAX cells (a cell per thread).  A smaller
+// level is as fast in the one block: a pass of 1024 cells takes it ~0.45 us,
+// as the cluster's barrier and refill do.
+int cluster_size_level(const mg_hierarchy* H) {
+  const long most = std::min<long>(CL_CELLS_MAX, 512L * cluster_cycle_blocks());
+  for (int l = 0; l + 1 < H->nlev; ++l)
+    if (H->L[l].cells() <= most) return H->L[l].cells() >= CL_CELLS_MIN ? l : -1;
+  return -1;
+}
+int cluster_cycle_level(mg_hierarchy* H, const Eq& e) {
+  const int l = H->nb == 1 ? cluster_size_level(H) : -1;
+  if (l < 0 || (e.kind == EQ_VEC && (e.bc != MG_BC_DIRICHLET || !H->L[l].cluster.mask))) return -1;
+  int w_at;
+  return block_cycle_params(H, e, l, true, &w_at).smem > 0 ? l : -1;
+}
+
+// vcycle32 from level l0 down, on a cluster.
+void cluster_vcycle32(mg_hierarchy* H, const Eq& e, int l0) {
+  Level& L = H->L[l0];
+  ClusterCycle32 Q;
+  Q.P = block_cycle_params(H, e, l0, true, &Q.w_at);
+  Q.P.fold_k = H->fold_k32;
+  Q.P.nb = 1;
+  Q.off = L.off;
+  Q.sx = L.sx;
+  Q.sy = L.sy;
+  Q.solo_from = Q.P.nl - 1;
+  for (int q = Q.P.nl - 1; q >= 0; --q) {
+    Level& M = H->L[l0 + q];
+    Q.lv[q] = M.cluster;
+    Q.lv[q].k = e.kind == EQ_PSI || e.has_c ? M.k32 : nullptr;
+    Q.lv[q].vc = M.vc32;
+    if (M.cells() <= CL_SOLO_CELLS) Q.solo_from = q;
+  }
+  for (int l = l0; l + 1 < H->nlev; ++l) H->updates += (int64_t)(H->d.nu1 + H->d.nu2) * H->L[l].cells() * e.ncomp;
+  long tok = prof_begin(H, l0, MG_PROF_BLOCK_CYCLE32, L.cells());
+  launch_cluster_vcycle32(Q, H->d.geom, H->st);
+  prof_end(H, tok);
+}
+
 // Linear correction-scheme V-cycle on (L - K) e = f32, e = 0 initially.
 void vcycle32(mg_hierarchy* H, const Eq& e, int l) {
+  if (l == cluster_cycle_level(H, e)) {
+    cluster_vcycle32(H, e, l);
+    return;
+  }
   if (l >= block_cycle_level(H, e)) {
     block_vcycle32(H, e, l);
     return;
@@ -1424,6 +1491,134 @@ int ensure_coarse_matrix(mg_hierarchy* H, int bc) {
   return MG_OK;
 }
 
+// Readers' tables (ClusterLevel32) of the vector levels a cluster takes, with
+// Dirichlet-0 ghosts, built once per hierarchy before its first vector solve
+// (outside graph capture).  The sources come from the device's own ghost
+// rules; a hierarchy with a ghost that is not plus or minus one interior
+// cell, the same for every component, keeps the other cycles.
+int ensure_cluster_tables(mg_hierarchy* H) {
+  if (H->cluster_state != 0) return MG_OK;
+  H->cluster_state = -1;
+  const int l0 = H->nb == 1 ? cluster_size_level(H) : -1;
+  if (l0 < 0 || H->d.mixed_deriv != MG_MIXED_4PT) return MG_OK;
+  const long gmax = ghost_count_host(H->L[l0].v64);
+  int* dgc = nullptr;
+  double* dfac = nullptr;
+  if (cudaMalloc(&dgc, sizeof(int) * 8 * 3 * (size_t)gmax) != cudaSuccess ||
+      cudaMalloc(&dfac, sizeof(double) * 3 * (size_t)gmax) != cudaSuccess) {
+    cudaFree(dgc);
+    cudaFree(dfac);
+    cudaGetLastError();
+    return MG_OK;
+  }
+  std::vector<int> gc(8 * 3 * (size_t)gmax);
+  std::vector<double> fac(3 * (size_t)gmax);
+  std::vector<unsigned char> buf;
+  struct Where {
+    size_t list, start, mask;
+  };
+  std::vector<Where> where(H->nlev);
+  cudaError_t ce = cudaSuccess;
+  bool ok = true;
+  for (int l = l0; l + 1 < H->nlev && ok && ce == cudaSuccess; ++l) {
+    Level& L = H->L[l];
+    const LevelView<double> v = with_bc(L.v64, MG_BC_DIRICHLET);
+    const long ng = ghost_count_host(v);
+    for (int c = 0; c < 3; ++c) launch_ghost_sources(v, c, dgc + 8 * c * ng, dfac + c * ng, H->st);
+    ce = cudaGetLastError();
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(gc.data(), dgc, sizeof(int) * 8 * 3 * ng, cudaMemcpyDeviceToHost, H->st);
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(fac.data(), dfac, sizeof(double) * 3 * ng, cudaMemcpyDeviceToHost, H->st);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(H->st);
+    if (ce != cudaSuccess) break;
+    const int n0 = v.n0, n1 = v.n1, n2 = v.n2, three = v.three;
+    auto team = [&](const Level& M) { return M.cells() > CL_SOLO_CELLS ? cluster_cycle_blocks() : 1; };
+    const int blocks = team(L), groups = (int)(L.cells() >> (three ? 3 : 2)) / blocks;
+    auto owner = [&](int i, int j, int k) {
+      return ((i >> 1) + (n0 >> 1) * ((j >> 1) + (n1 >> 1) * (k >> 1))) / groups;
+    };
+    LevelView<double> c = v;
+    unpad(c);
+    auto at = [&](int i, int j, int k) { return (size_t)(c.off + i + j * c.sx + (long)k * c.sy); };
+    // the blocks that read a place of the array: as a cell's neighbour, in
+    // the prolongation to the finer level, or as the source of a ghost
+    std::vector<unsigned> readers(c.sy * (n2 + 2 * three), 0u);
+    const int fine_groups = l > l0 && blocks > 1 ? (int)(L.cells() / team(H->L[l - 1])) : 0;
+    for (int k = 0; k < n2; ++k)
+      for (int j = 0; j < n1; ++j)
+        for (int i = 0; i < n0; ++i)
+          for (int d = three ? -1 : 0; d <= (three ? 1 : 0); ++d)
+            for (int b = -1; b <= 1; ++b)
+              for (int a = -1; a <= 1; ++a) {
+                const int far = std::abs(a) + std::abs(b) + std::abs(d);
+                if (far <= 2) readers[at(i + a, j + b, k + d)] |= 1u << owner(i, j, k);
+                if (far <= 1 && fine_groups) readers[at(i + a, j + b, k + d)] |= 1u << (i + n0 * (j + n1 * k)) / fine_groups;
+              }
+    std::vector<std::vector<uint2>> list(blocks);
+    ok = readers.size() <= 0xffff;
+    for (long g = 0; g < ng && ok; ++g) {
+      const int* o = &gc[8 * g];
+      unsigned sign = 0;
+      for (int m = 0; m < 3; ++m) {
+        const double f = fac[m * ng + g];
+        ok = ok && (f == 1.0 || f == -1.0) && gc[8 * (m * ng + g) + 7] == o[7];
+        sign |= (f < 0.0 ? 1u : 0u) << m;
+      }
+      ok = ok && o[3] >= 0 && o[3] < n0 && o[4] >= 0 && o[4] < n1 && o[5] >= 0 && o[5] < n2 && o[6] >= 0 && o[6] < L.ng &&
+           o[0] >= -1 && o[0] <= n0 && o[1] >= -1 && o[1] <= n1 && o[2] >= -three && o[2] < n2 + three;
+      if (!ok) break;
+      const size_t dst = at(o[0], o[1], o[2]), src = at(o[3], o[4], o[5]);
+      const unsigned r = readers[dst] ? readers[dst] : 1u << owner(o[3], o[4], o[5]);
+      for (int b = 0; b < blocks; ++b)
+        if (r >> b & 1u) list[b].push_back(make_uint2((unsigned)(dst | src << 16), sign | (unsigned)o[6] << 3));
+      readers[src] |= r;
+    }
+    if (!ok) break;
+    auto room = [&](size_t n) {
+      const size_t p = buf.size();
+      buf.resize((p + n + 7) & ~(size_t)7);
+      return p;
+    };
+    std::vector<int> start(blocks + 1, 0);
+    for (int b = 0; b < blocks; ++b) start[b + 1] = start[b] + (int)list[b].size();
+    Where& w = where[l];
+    w.list = room(sizeof(uint2) * start[blocks]);
+    w.start = room(sizeof(int) * (blocks + 1));
+    w.mask = room(sizeof(unsigned short) * L.cells());
+    for (int b = 0; b < blocks; ++b)
+      std::memcpy(buf.data() + w.list + sizeof(uint2) * start[b], list[b].data(), sizeof(uint2) * list[b].size());
+    std::memcpy(buf.data() + w.start, start.data(), sizeof(int) * (blocks + 1));
+    unsigned short* mask = reinterpret_cast<unsigned short*>(buf.data() + w.mask);
+    for (int k = 0; k < n2; ++k)
+      for (int j = 0; j < n1; ++j)
+        for (int i = 0; i < n0; ++i)
+          mask[i + n0 * (j + n1 * k)] = (unsigned short)(readers[at(i, j, k)] & ~(1u << owner(i, j, k)));
+  }
+  cudaFree(dgc);
+  cudaFree(dfac);
+  if (ce != cudaSuccess) return fail(MG_ERR_CUDA, cudaGetErrorString(ce));
+  if (!ok) return MG_OK;
+  unsigned char* d = nullptr;
+  if (cudaMalloc(&d, buf.size()) != cudaSuccess) {
+    cudaGetLastError();
+    return MG_OK;
+  }
+  ce = cudaMemcpyAsync(d, buf.data(), buf.size(), cudaMemcpyHostToDevice, H->st);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(H->st);
+  if (ce != cudaSuccess) {
+    cudaFree(d);
+    return fail(MG_ERR_CUDA, cudaGetErrorString(ce));
+  }
+  H->cluster_buf = d;
+  for (int l = l0; l + 1 < H->nlev; ++l) {
+    ClusterLevel32& C = H->L[l].cluster;
+    C.list = reinterpret_cast<const uint2*>(d + where[l].list);
+    C.start = reinterpret_cast<const int*>(d + where[l].start);
+    C.mask = reinterpret_cast<const unsigned short*>(d + where[l].mask);
+  }
+  H->cluster_state = 1;
+  return MG_OK;
+}
+
 // Ghost-push tables (GhostPush) of the vector colour passes with Dirichlet-0
 // ghosts, for every level below the coarsest, built once per hierarchy
 // before its first vector solve (outside graph capture).  The sources come
@@ -1748,6 +1943,8 @@ int run_solve_body(mg_hierarchy* H, const Eq& e, mg_solve_report* rep) {
     if (int est = ensure_coarse_rows(H, e.bc)) return est;
   if (e.kind == EQ_VEC && e.bc == MG_BC_DIRICHLET)
     if (int est = ensure_ghost_push(H)) return est;
+  if (mixed && e.kind == EQ_VEC && e.bc == MG_BC_DIRICHLET)
+    if (int est = ensure_cluster_tables(H)) return est;
   if (e.kind == EQ_VEC) fill_all64(H, e, 0);
   restrict_sources(H, e);
   if (mixed && e.kind == EQ_LIN && e.has_c) {
@@ -2382,6 +2579,8 @@ int create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, int nb, mg_hie
   init_fused_sweep_attributes<float>();
   init_block_cycle_attributes();
   init_fas_attributes();
+  init_cluster_cycle_attributes();
+  init_cluster_cycle_attributes();
   const int three = H->d.ndim == 3;
   for (int l = 0; l < H->nlev; ++l) {
     Level& L = H->L[l];
@@ -2513,6 +2712,7 @@ int mg_destroy_hierarchy(mg_hierarchy* H) {
   for (cudaEvent_t e : H->b_ev)
     if (e) cudaEventDestroy(e);
   if (H->push_buf) cudaFree(H->push_buf);
+  if (H->cluster_buf) cudaFree(H->cluster_buf);
   for (GraphEntry& g : H->graphs) cudaGraphExecDestroy(g.exec);
   for (auto& g : H->loops) cudaGraphExecDestroy(g.exec);
   if (H->d_loop) cudaFree(H->d_loop);

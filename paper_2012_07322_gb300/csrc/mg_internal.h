@@ -505,6 +505,32 @@ struct BlockCycle32 {
   size_t smem;            // dynamic shared memory bytes
 };
 void launch_block_vcycle32(const BlockCycle32& P, int geom, cudaStream_t st);
+
+// The same cycle on a thread-block cluster (mg_clus.cu).  Shared memory holds
+// of level P.lv[0] the correction alone; vector levels are not padded there.
+constexpr long CL_CELLS_MIN = 2048, CL_CELLS_MAX = 8192;  // of the first level
+constexpr long CL_SOLO_CELLS = 512;  // levels this small run on the first block
+constexpr size_t CL_SMEM_MAX = 212 * 1024;  // dynamic; the coarsest solves take 14 KB besides
+struct ClusterLevel32 {
+  const float* k;              // c of (L - c) e = f in HBM, or null
+  // vector equations:
+  const float* vc;             // the level's coefficient table
+  const unsigned short* mask;  // per cell, the other blocks that read it
+  // per block, start[b] .. start[b + 1] - 1: the ghosts it reads, (ghost |
+  // source << 16 in shared memory, sign per component | ghost in HBM << 3)
+  const uint2* list;
+  const int* start;
+};
+struct ClusterCycle32 {
+  BlockCycle32 P;
+  ClusterLevel32 lv[BC_MAX];
+  long off, sx, sy;  // layout of level P.lv[0] in HBM
+  int solo_from;     // the levels the first block runs alone
+  int w_at;          // offset (floats) of 3 x BC_THREADS values
+};
+void init_cluster_cycle_attributes();  // once a device is current, before any capture
+int cluster_cycle_blocks();            // blocks of its cluster, 0: not available
+void launch_cluster_vcycle32(const ClusterCycle32& Q, int geom, cudaStream_t st);
 void init_block_cycle_attributes();
 // The largest coarsest vector system solved exactly (3 x cells).
 constexpr int BC_CINV_MAX = 768;
