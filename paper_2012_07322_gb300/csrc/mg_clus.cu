@@ -40,7 +40,7 @@ __device__ __forceinline__ void cl_sync() {
 // black ones to the others; thread g of a colour takes pair g % pairs (same
 // (j, k)) of group g / pairs.
 struct ClCell {
-  int tid, rank, size, half, groups, lp, colour;
+  int tid, rank, size, half, groups, lgroups, lp, colour;
   bool on;
   int i, j, k, p;  // p: offset in the ghosted level (P.lv[l].v)
   __device__ __forceinline__ ClCell(const LevelView<float>& L, int r, int s) : tid(threadIdx.x), rank(r), size(s) {
@@ -48,8 +48,9 @@ struct ClCell {
     half = max(mine, 32);  // a colour's threads, in whole warps
     lp = L.three ? 2 : 1;
     groups = (n >> (lp + 1)) / size;
+    lgroups = 31 - __clz(groups);
     colour = tid >= half;
-    const int g = tid - colour * half, pc = g & ((1 << lp) - 1), G0 = rank * groups + (g >> lp), dj = pc & 1, dk = pc >> 1;
+    const int g = tid - colour * half, pc = g & ((1 << lp) - 1), G0 = (rank << lgroups) + (g >> lp), dj = pc & 1, dk = pc >> 1;
     on = g < mine;
     i = 2 * (G0 & ((L.n0 >> 1) - 1)) + (colour ^ dj ^ dk);
     j = 2 * ((G0 >> (L.ln0 - 1)) & ((L.n1 >> 1) - 1)) + dj;
@@ -64,7 +65,7 @@ struct ClCell {
       __syncthreads();
   }
   __device__ __forceinline__ int owner(const LevelView<float>& L, int a, int b, int c) const {
-    return ((a >> 1) + ((b >> 1) << (L.ln0 - 1)) + ((c >> 1) << (L.ln0 + L.ln1 - 2))) / groups;
+    return ((a >> 1) + ((b >> 1) << (L.ln0 - 1)) + ((c >> 1) << (L.ln0 + L.ln1 - 2))) >> lgroups;
   }
   // Restriction weight, normalised over the cell's group.
   __device__ __forceinline__ float weight(const LevelView<float>& L) const {
@@ -90,11 +91,32 @@ struct ClScalar {
   float* e;          // the level's cells, without ghosts
   unsigned mask;     // blocks that own a neighbour
   int q, nb[6];
-  float c[5], cC, iD, f, K, u;
-  __device__ __forceinline__ ClScalar(const ClCell& t_, const ClusterCycle32& Q, int l, float* sm)
+  float c[5], cC, iD, f, K, wt, u;
+  // down: resolve the stencil and keep it in shared memory for the visit up
+  __device__ __forceinline__ ClScalar(const ClCell& t_, const ClusterCycle32& Q, int l, float* sm, bool down)
       : t(t_), L(Q.P.lv[l].v), e(sm + Q.P.lv[l].e[0]), mask(0) {
     if (!t.on) return;
     const BlockLevel32& B = Q.P.lv[l];
+    float* const slot = sm + Q.slot_at[l] + t.tid;
+    const int stride = 2 * t.half;
+    if (!down) {
+      q = t.i + L.n0 * (t.j + L.n1 * t.k);
+#pragma unroll
+      for (int m = 0; m < 5; ++m) c[m] = slot[m * stride];
+      cC = slot[5 * stride];
+      iD = slot[6 * stride];
+      f = slot[7 * stride];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        const unsigned x = __float_as_uint(slot[(8 + m) * stride]);
+        nb[2 * m] = (int)(x & 0xffffu);
+        nb[2 * m + 1] = (int)(x >> 16);
+      }
+      mask = __float_as_uint(slot[11 * stride]);
+      u = e[q];
+      return;
+    }
+    wt = t.weight(L);
     const int n0 = L.n0, n1 = L.n1, n2 = L.n2, i = t.i, j = t.j, k = t.k;
     q = i + n0 * (j + n1 * k);
     c[0] = L.TI(TI_CE, i);
@@ -138,6 +160,14 @@ struct ClScalar {
     side(4, 2, 1);
     side(5, 2, -1);
     mask &= ~(1u << t.rank);
+#pragma unroll
+    for (int m = 0; m < 5; ++m) slot[m * stride] = c[m];
+    slot[5 * stride] = cC;
+    slot[6 * stride] = iD;
+    slot[7 * stride] = f;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) slot[(8 + m) * stride] = __uint_as_float((unsigned)nb[2 * m] | (unsigned)nb[2 * m + 1] << 16);
+    slot[11 * stride] = __uint_as_float(mask);
   }
   // L e - K e - f
   __device__ __forceinline__ float defect() const {
@@ -164,7 +194,6 @@ struct ClScalar {
   }
   __device__ __forceinline__ void restrict_to(const BlockCycle32& P, int l, const ClCell& tc, float* sm, float* w) {
     if (t.on) {
-      const float wt = t.weight(L);
       w[t.tid] = -wt * defect();
       if (P.fold_k) w[BC_THREADS + t.tid] = wt * K;
     }
@@ -233,10 +262,11 @@ struct ClVector {
   unsigned mask;       // blocks that read the cell
   const uint2* list;   // ghosts this block reads: ghost | source << 16, sign per component
   int nlist;
-  uint2 g0;
+  uint2 g[2];
   long hp;             // the cell in HBM
+  float wt;
   float a[12], b[10], c[10], iD[3], f[3];
-  __device__ __forceinline__ ClVector(const ClCell& t_, const ClusterCycle32& Q, int l, float* sm)
+  __device__ __forceinline__ ClVector(const ClCell& t_, const ClusterCycle32& Q, int l, float* sm, bool down)
       : t(t_), L(Q.P.lv[l].v), mask(0) {
     const BlockLevel32& W = Q.P.lv[l];
     const ClusterLevel32& T = Q.lv[l];
@@ -244,8 +274,11 @@ struct ClVector {
     for (int m = 0; m < 3; ++m) e[m] = sm + W.e[m];
     list = T.list + T.start[t.rank];
     nlist = T.start[t.rank + 1] - T.start[t.rank];
-    g0 = t.tid < nlist ? list[t.tid] : make_uint2(0, 0);
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      g[r] = t.tid + r * BC_THREADS < nlist ? list[t.tid + r * BC_THREADS] : make_uint2(0, 0);
     if (!t.on) return;
+    if (down) wt = t.weight(L);
     hp = Q.off + t.i + t.j * Q.sx + t.k * Q.sy;
     mask = T.mask[t.i + L.n0 * (t.j + L.n1 * t.k)];
 #pragma unroll
@@ -324,11 +357,14 @@ struct ClVector {
     for (unsigned k = mask; k; k &= k - 1u) cl_store(cl_addr(p), __ffs(k) - 1, v);
   }
   __device__ __forceinline__ void fill(int m) {
-    for (int q = t.tid; q < nlist; q += BC_THREADS) {
-      const uint2 g = q == t.tid ? g0 : list[q];
-      const float x = e[m][g.x >> 16];
-      e[m][g.x & 0xffffu] = (g.y >> m) & 1u ? -x : x;
-    }
+    auto one = [&](uint2 a) {
+      const float x = e[m][a.x >> 16];
+      e[m][a.x & 0xffffu] = (a.y >> m) & 1u ? -x : x;
+    };
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (t.tid + r * BC_THREADS < nlist) one(g[r]);
+    for (int q = t.tid + 2 * BC_THREADS; q < nlist; q += BC_THREADS) one(list[q]);
   }
   __device__ __forceinline__ void fill() {
 #pragma unroll
@@ -352,7 +388,6 @@ struct ClVector {
   }
   __device__ __forceinline__ void restrict_to(const BlockCycle32& P, int l, const ClCell& tc, float* sm, float* w) {
     if (t.on) {
-      const float wt = t.weight(L);
       w[t.tid] = -wt * defect<0>();
       w[BC_THREADS + t.tid] = -wt * defect<1>();
       w[2 * BC_THREADS + t.tid] = -wt * defect<2>();
@@ -417,7 +452,7 @@ __global__ void __launch_bounds__(BC_THREADS, 1) k_cluster_vcycle32(const __grid
   cl_sync();  // every block has started, with a zero correction
   for (int l = 0; l + 1 < nl && rank < team(l); ++l) {
     const ClCell t(P.lv[l].v, rank, team(l)), tc(P.lv[l + 1].v, rank, team(l + 1));
-    Top T(t, Q, l, sm);
+    Top T(t, Q, l, sm, true);
     T.sweeps(P.nu1, false);
     T.restrict_to(P, l, tc, sm, w);
     t.sync();
@@ -426,7 +461,7 @@ __global__ void __launch_bounds__(BC_THREADS, 1) k_cluster_vcycle32(const __grid
   for (int l = nl - 2; l >= 0; --l) {
     if (rank >= team(l)) continue;
     const ClCell t(P.lv[l].v, rank, team(l));
-    Top T(t, Q, l, sm);
+    Top T(t, Q, l, sm, false);
     t.sync();  // the coarse level's values
     T.prolong(P, l, team(l) > team(l + 1), sm);
     t.sync();

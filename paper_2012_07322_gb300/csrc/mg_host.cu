@@ -956,10 +956,11 @@ void unpad(LevelView<T>& v) {
 // Parameters of the one-block coarse cycle from level l0 (mg_block.cu):
 // shared-memory offsets of every level's arrays; P.smem = 0 when they do
 // not fit.
-// top: level l0 runs on a cluster, and only its correction is held here (with
-// what the cluster needs besides at w_at); vector levels without the padding
-// of their rows.
-BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0, bool top = false, int* w_at = nullptr) {
+// Q: the cycle runs on a cluster; of level l0 only the correction is held here
+// (with what the cluster needs besides), vector levels without the padding of
+// their rows.
+BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0, ClusterCycle32* Q = nullptr) {
+  const bool top = Q != nullptr;
   BlockCycle32 P{};
   const bool hasK = e.kind == EQ_PSI || e.has_c;
   const int nc = e.kind == EQ_VEC ? 3 : 1;
@@ -1010,7 +1011,14 @@ BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0, bool top =
       B.gf_at = take(at);
     }
   }
-  if (w_at) *w_at = take(3 * 512);
+  if (Q) {
+    Q->w_at = take(3 * 512);
+    for (int q = 0; q + 1 < P.nl && !P.vec; ++q) {
+      const long n = H->L[l0 + q].cells();
+      const long mine = n > CL_SOLO_CELLS ? n / cluster_cycle_blocks() : n;
+      Q->slot_at[q] = take(CL_WORDS * std::max(mine, 64L));
+    }
+  }
   Level& Lc = H->L[H->nlev - 1];
   P.c64 = with_bc(Lc.v64, e.bc);
   if (top && P.vec) unpad(P.c64);
@@ -1081,15 +1089,15 @@ int cluster_size_level(const mg_hierarchy* H) {
 int cluster_cycle_level(mg_hierarchy* H, const Eq& e) {
   const int l = H->nb == 1 ? cluster_size_level(H) : -1;
   if (l < 0 || (e.kind == EQ_VEC && (e.bc != MG_BC_DIRICHLET || !H->L[l].cluster.mask))) return -1;
-  int w_at;
-  return block_cycle_params(H, e, l, true, &w_at).smem > 0 ? l : -1;
+  ClusterCycle32 Q;
+  return block_cycle_params(H, e, l, &Q).smem > 0 ? l : -1;
 }
 
 // vcycle32 from level l0 down, on a cluster.
 void cluster_vcycle32(mg_hierarchy* H, const Eq& e, int l0) {
   Level& L = H->L[l0];
   ClusterCycle32 Q;
-  Q.P = block_cycle_params(H, e, l0, true, &Q.w_at);
+  Q.P = block_cycle_params(H, e, l0, &Q);
   Q.P.fold_k = H->fold_k32;
   Q.P.nb = 1;
   Q.off = L.off;

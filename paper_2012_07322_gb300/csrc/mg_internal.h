@@ -527,7 +527,9 @@ struct ClusterCycle32 {
   long off, sx, sy;  // layout of level P.lv[0] in HBM
   int solo_from;     // the levels the first block runs alone
   int w_at;          // offset (floats) of 3 x BC_THREADS values
+  int slot_at[BC_MAX];  // scalar levels: offsets of CL_WORDS values per thread
 };
+constexpr int CL_WORDS = 12;
 void init_cluster_cycle_attributes();  // once a device is current, before any capture
 int cluster_cycle_blocks();            // blocks of its cluster, 0: not available
 void launch_cluster_vcycle32(const ClusterCycle32& Q, int geom, cudaStream_t st);
