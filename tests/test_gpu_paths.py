@@ -1,0 +1,177 @@
+"""The launch paths of small levels against the FP64 oracle, at the sizes where
+each path begins, ends or degenerates: the FP64 cluster cycle of scalar
+equations (mg_fas.cu), the tabulated FP64 coarsest vector solve
+(mg_coarse.cuh), the FP32 correction cycle on a cluster (mg_clus.cu), the
+integer stencils of Cartesian levels (mg_cart.cu), the batch's launch shapes
+and the one-launch divergence norms.
+
+FP64 solves follow the oracle's cycles: the count within one, every field
+within 1e-9 at a converged relative residual of 1e-10, as in the solver-level
+parity tests.  Mixed solves reach the same discrete solution by other
+iterates: both sides converge to 1e-11, which leaves a factor 50 for the
+response of the smoothest modes (2 x 50 x 1e-11 = 1e-9)."""
+import numpy as np
+import pytest
+
+import oracle.oracle as o
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+PI = np.pi
+BOX = {"sph": ([0.0, 0.0, 0.0], [30.0, PI, 2 * PI]), "cyl": ([0.0, -30.0, 0.0], [30.0, 34.0, 2 * PI]),
+       "cart": ([-30.0, -25.0, -20.0], [34.0, 27.0, 31.0]),
+       "cube": ([-1.0] * 3, [1.0] * 3)}  # equal spacings on equal sizes
+
+
+@pytest.fixture(scope="module")
+def mg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2012_07322_gb300 import mg as m
+    m.lib()
+    return m
+
+
+def dev(a):
+    return torch.from_numpy(np.array(a, dtype=np.float64, copy=True)).cuda()
+
+
+def host(t):
+    return t.detach().cpu().numpy()
+
+
+def solve_pair(mg, geom, n, kind, bc, precision, nu, tol, accel=0, scale=1.0):
+    """The same random problem through the oracle and through the GPU."""
+    lo, hi = BOX[geom][0][:len(n)], BOX[geom][1][:len(n)]
+    geom = "cart" if geom == "cube" else geom
+    kw = dict(tol=tol, max_cycles=1000, nu1=nu[0], nu2=nu[1], stall_window=0)
+    d = o.desc(geom, n, lo, hi, accel_depth=8 if accel else 0, **kw)
+    gd = mg.grid_desc(geom, n, lo, hi, precision=precision, accel_depth=accel, **kw)
+    rng = np.random.default_rng(sum(n) + len(kind))
+    h = mg.Hierarchy(gd)
+    zero = lambda: torch.zeros(o.shape(d), dtype=torch.float64, device="cuda")
+    try:
+        if kind == "vec":
+            f = [scale * rng.standard_normal(o.shape(d)) for _ in range(3)]
+            V = [np.zeros(o.shape(d)) for _ in range(3)]
+            ro = o.solve_vector(d, bc, f, V)
+            Vt = [zero() for _ in range(3)]
+            rg = mg.mg_solve_vector(h, bc, [dev(x) for x in f], Vt)
+            return ro, rg, np.stack(V), np.stack([host(x) for x in Vt])
+        if kind == "psi":
+            args = dict(U=rng.uniform(0, 1e-3, o.shape(d)), A2=rng.uniform(0, 1e-4, o.shape(d)))
+        else:
+            args = dict(f=scale * rng.standard_normal(o.shape(d)))
+            if kind == "lin_c":
+                args["c"] = rng.uniform(0, 0.01, o.shape(d))
+            if bc == "neumann":
+                args["f"] -= args["f"].mean()
+        k = "psi" if kind == "psi" else "lin"
+        u = np.zeros(o.shape(d))
+        ro = o.solve_scalar(d, k, bc, u, zero_mean=bc == "neumann", **args)
+        ut = zero()
+        rg = mg.mg_solve_scalar(h, k, bc, ut, zero_mean=bc == "neumann", **{q: dev(v) for q, v in args.items()})
+        return ro, rg, u, host(ut)
+    finally:
+        h.close()
+
+
+def check(ro, rg, want, got, cycles):
+    assert ro["status"] == "ok" and rg["status"] == "ok"
+    if cycles:
+        assert abs(rg["cycles"] - ro["cycles"]) <= 1, (rg["cycles"], ro["cycles"])
+    assert np.abs(got - want).max() <= 1e-9 * np.abs(want).max()
+
+
+# 4096 and 2048 cells (the cluster's largest level and one below), 256 cells
+# (its smallest), 128 and fewer (one block), wide and flat coarsest levels
+@pytest.mark.parametrize("geom,n,kind,bc,nu", [
+    ("sph", [64, 32], "psi", "robin", (2, 2)),
+    ("sph", [32, 16, 8], "psi", "robin", (1, 2)),
+    ("sph", [16, 8], "lin_c", "dirichlet", (2, 1)),
+    ("sph", [16, 16], "psi", "robin", (3, 1)),
+    ("cyl", [32, 64], "lin_c", "robin", (2, 2)),
+    ("cyl", [16, 16, 16], "lin", "dirichlet", (1, 1)),
+    ("cyl", [8, 16], "psi", "robin", (2, 0)),
+    ("cart", [16, 16, 16], "lin", "robin", (2, 2)),
+    ("cart", [32, 8], "lin", "neumann", (2, 2)),
+    ("cart", [64, 64], "psi", "dirichlet", (0, 2)),
+])
+def test_fp64_scalar_small_levels(mg, geom, n, kind, bc, nu):
+    check(*solve_pair(mg, geom, n, kind, bc, "fp64", nu, 1e-10), cycles=True)
+
+
+# coarsest systems of 24 to 192 unknowns, two and three dimensions, and a
+# level below the warp size
+@pytest.mark.parametrize("geom,n,bc", [
+    ("sph", [8, 4], "dirichlet"), ("sph", [32, 16, 8], "dirichlet"), ("cyl", [16, 64], "dirichlet"),
+    ("cyl", [8, 8, 8], "dirichlet"), ("cart", [16, 8], "dirichlet"), ("cart", [16, 16, 8], "robin"),
+])
+def test_fp64_vector_small_levels(mg, geom, n, bc):
+    check(*solve_pair(mg, geom, n, "vec", bc, "fp64", (2, 2), 1e-10), cycles=True)
+
+
+# first levels of 2048 and 8192 cells, levels either side of the one-block
+# ones (512 cells), a coarser level of the cluster below a launched one
+@pytest.mark.parametrize("geom,n,kind,bc,nu", [
+    ("sph", [64, 32], "psi", "robin", (2, 2)),
+    ("sph", [64, 32], "vec", "dirichlet", (1, 2)),
+    ("sph", [32, 16, 16], "psi", "robin", (2, 1)),
+    ("sph", [32, 16, 16], "vec", "dirichlet", (2, 2)),
+    ("sph", [32, 32, 16], "lin_c", "robin", (2, 2)),
+    ("cyl", [64, 128], "lin_c", "robin", (2, 2)),
+    ("cyl", [64, 128], "vec", "dirichlet", (2, 2)),
+    ("cyl", [16, 16, 16], "vec", "dirichlet", (2, 2)),
+    ("cart", [16, 16, 16], "lin", "robin", (2, 2)),
+    ("cart", [128, 32], "lin", "dirichlet", (2, 2)),
+    ("cart", [16, 16, 16], "vec", "dirichlet", (2, 2)),
+    ("cart", [64, 64], "vec", "dirichlet", (2, 2)),
+    ("cart", [32, 64], "lin", "neumann", (2, 2)),
+])
+def test_fp32_cycle_on_a_cluster(mg, geom, n, kind, bc, nu):
+    check(*solve_pair(mg, geom, n, kind, bc, "mixed", nu, 1e-11, accel=8), cycles=False)
+
+
+# fields near the ends of the exponent range go the stencils' other way; a
+# linear equation scales exactly with its right-hand side
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("geom,exponent", [("cube", -80), ("cube", 60), ("cart", 60)])
+def test_cartesian_stencils_scale_with_the_field(mg, precision, geom, exponent):
+    n = [32, 32, 32]
+    one = solve_pair(mg, geom, n, "lin", "robin", precision, (2, 2), 1e-10)
+    far = solve_pair(mg, geom, n, "lin", "robin", precision, (2, 2), 1e-10, scale=2.0 ** exponent)
+    check(*one, cycles=precision == "fp64")
+    assert far[1]["status"] == "ok"
+    assert np.abs(far[3] * 2.0 ** -exponent - one[3]).max() <= 1e-9 * np.abs(one[3]).max()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_cartesian_stencils_carry_bad_values(mg, bad):
+    gd = mg.grid_desc("cart", [32, 32, 32], [-1.0] * 3, [1.0] * 3, max_cycles=5)
+    h = mg.Hierarchy(gd)
+    f = np.zeros((32, 32, 32))
+    f[3, 4, 5] = bad
+    u = torch.zeros((32, 32, 32), dtype=torch.float64, device="cuda")
+    rg = mg.mg_solve_scalar(h, "lin", "dirichlet", u, f=dev(f), allow=tuple(range(8)))
+    h.close()
+    assert rg["status"] != "ok"
+
+
+# one cell, one row, sizes around a block and no powers of two
+@pytest.mark.parametrize("n", [[1, 1], [3, 5, 7], [257, 3], [31, 33, 2], [1, 64, 5]])
+def test_divergence_norms_of_odd_grids(mg, n):
+    rng = np.random.default_rng(sum(n))
+    B = [rng.standard_normal(tuple(reversed(n))) for _ in n]
+    lo, hi = [0.0] * len(n), [0.5 + 0.25 * k for k in range(len(n))]
+    div = 0.0
+    for d, b in enumerate(B):
+        ax = len(n) - 1 - d
+        p = np.pad(b, [(1, 1) if a == ax else (0, 0) for a in range(len(n))], mode="edge")
+        up, dn = np.take(p, range(2, n[d] + 2), ax), np.take(p, range(n[d]), ax)
+        div = div + (up - dn) / (2 * (hi[d] - lo[d]) / n[d])
+    st, mx, l2 = mg.mg_divb_norms_noalloc([dev(b) for b in B], lo, hi)
+    # a sum of three differences of O(1) values over the spacing, ~10 roundings of its largest term
+    tiny = 1e-14 * max(n[d] / (hi[d] - lo[d]) for d in range(len(n)))
+    assert st == mg.MG_OK
+    assert abs(mx - np.abs(div).max()) <= tiny and abs(l2 - np.sqrt(np.mean(div ** 2))) <= tiny
