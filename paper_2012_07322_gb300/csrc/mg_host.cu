@@ -1053,15 +1053,12 @@ BlockCycle32 block_cycle_params(mg_hierarchy* H, const Eq& e, int l0, ClusterCyc
 }
 
 // First level of the one-block coarse cycle: the first level of at most
-// max_cells cells whose levels down to the coarsest fit the block's
+// BLOCK_CYCLE_CELLS cells whose levels down to the coarsest fit the block's
 // shared memory.
-int block_cycle_level(mg_hierarchy* H, const Eq& e, long max_cells) {
-  for (int l = 0; l < H->nlev; ++l)
-    if (H->L[l].cells() <= max_cells && block_cycle_params(H, e, l).smem > 0) return l;
-  return H->nlev;
-}
 int block_cycle_level(mg_hierarchy* H, const Eq& e) {
-  return block_cycle_level(H, e, e.kind == EQ_VEC ? BLOCK_CYCLE_CELLS : BLOCK_CYCLE_CELLS_SCALAR);
+  for (int l = 0; l < H->nlev; ++l)
+    if (H->L[l].cells() <= BLOCK_CYCLE_CELLS && block_cycle_params(H, e, l).smem > 0) return l;
+  return H->nlev;
 }
 
 // vcycle32 from level l0 down, in one block.
@@ -2940,7 +2937,7 @@ int batch_item(mg_hierarchy* h, const mg_cfc_sources& src, const mg_cfc_fields& 
   // cycle fits the batch kernel's shared memory beside its static arrays
   const size_t limit = batch_smem_limit();
   auto first_fit = [&](const Eq& e, BlockCycle32* out) {
-    for (int l = block_cycle_level(h, e, BLOCK_CYCLE_CELLS); l < h->nlev && l <= BATCH_MAX_LEVELS; ++l) {
+    for (int l = block_cycle_level(h, e); l < h->nlev && l <= BATCH_MAX_LEVELS; ++l) {
       const BlockCycle32 Q = block_cycle_params(h, e, l);
       if (Q.smem && Q.smem <= limit) {
         *out = Q;

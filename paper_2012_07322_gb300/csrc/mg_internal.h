@@ -471,10 +471,7 @@ void launch_loop_decide(LoopState* S, const unsigned long long* red, const LoopP
 // the levels l0 .. l0 + nl - 1 of a hierarchy, the last the coarsest, all
 // held in the block's shared memory (same ghosted layout as in HBM).
 constexpr int BC_MAX = 8;                     // levels one block cycle may span
-// Levels this small run in the block cycle: scalar equations from 8192 cells
-// on (a pass over 8192 cells takes one SM ~0.9 us, a launch 2.5), vector ones
-// and the batch's from 4096.
-constexpr long BLOCK_CYCLE_CELLS = 4096, BLOCK_CYCLE_CELLS_SCALAR = 8192;
+constexpr long BLOCK_CYCLE_CELLS = 4096;      // levels this small run in the block cycle
 constexpr size_t BC_SMEM_MAX = 200 * 1024;     // dynamic shared memory of the block cycle
 struct BlockLevel32 {
   LevelView<float> v;        // boundary rule applied
