@@ -14,73 +14,19 @@
 // ~400 cycles), the neighbours' shared loads and one cell's multiply-adds;
 // for the vector equation also the refill of the ghosts the block reads, each
 // plus or minus an interior cell (their sources and the blocks that read a
-// cell come from a table the host builds once per hierarchy).
+// cell come from a table the host builds once per hierarchy).  Mixed xCFC on
+// 64 x 128 cylindrical cells 4.92 to 3.90 ms per solve, on 128 x 64 x 64
+// spherical ones (32 x 16 x 16 and below here) 228 to 212 ms.
 #include <cooperative_groups.h>
 
 #include "mg_block.cuh"
+#include "mg_cell.cuh"
 #include "mg_internal.h"
 #include "mg_kernels.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace gmg {
-
-__device__ __forceinline__ unsigned cl_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cl_store(unsigned addr, int rank, float v) {
-  unsigned ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
-}
-__device__ __forceinline__ void cl_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// The cell of a thread.  Cells are dealt in groups of one coarse cell's
-// children, consecutive groups to a block, red cells to the first threads and
-// black ones to the others; thread g of a colour takes pair g % pairs (same
-// (j, k)) of group g / pairs.
-struct ClCell {
-  int tid, rank, size, half, groups, lgroups, lp, colour;
-  bool on;
-  int i, j, k, p;  // p: offset in the ghosted level (P.lv[l].v)
-  __device__ __forceinline__ ClCell(const LevelView<float>& L, int r, int s) : tid(threadIdx.x), rank(r), size(s) {
-    const int n = L.n0 * L.n1 * L.n2, mine = n / size / 2;
-    half = max(mine, 32);  // a colour's threads, in whole warps
-    lp = L.three ? 2 : 1;
-    groups = (n >> (lp + 1)) / size;
-    lgroups = 31 - __clz(groups);
-    colour = tid >= half;
-    const int g = tid - colour * half, pc = g & ((1 << lp) - 1), G0 = (rank << lgroups) + (g >> lp), dj = pc & 1, dk = pc >> 1;
-    on = g < mine;
-    i = 2 * (G0 & ((L.n0 >> 1) - 1)) + (colour ^ dj ^ dk);
-    j = 2 * ((G0 >> (L.ln0 - 1)) & ((L.n1 >> 1) - 1)) + dj;
-    k = 2 * (G0 >> (L.ln0 + L.ln1 - 2)) + dk;
-    p = (int)L.idx(i, j, k);
-  }
-  // A barrier of the blocks that work on the level.
-  __device__ __forceinline__ void sync() const {
-    if (size > 1)
-      cl_sync();
-    else
-      __syncthreads();
-  }
-  __device__ __forceinline__ int owner(const LevelView<float>& L, int a, int b, int c) const {
-    return ((a >> 1) + ((b >> 1) << (L.ln0 - 1)) + ((c >> 1) << (L.ln0 + L.ln1 - 2))) >> lgroups;
-  }
-  // Restriction weight, normalised over the cell's group.
-  __device__ __forceinline__ float weight(const LevelView<float>& L) const {
-    const float wi = L.TI(TI_VW, i), wj = L.TJ(TJ_VW, j);
-    const float si = wi + L.TI(TI_VW, i ^ 1), sj = wj + L.TJ(TJ_VW, j ^ 1);
-    return wi * wj / ((L.three ? 2.0f : 1.0f) * (si * sj));
-  }
-  // Sum of a group's values w[thread].
-  __device__ __forceinline__ float group_sum(const float* w, int g) const {
-    const float* r = w + (g << lp);
-    float s = (r[0] + r[half]) + (r[1] + r[half + 1]);
-    if (lp == 2) s += (r[2] + r[half + 2]) + (r[3] + r[half + 3]);
-    return s;
-  }
-};
 
 // ------------------------------------------------------ scalar equations
 

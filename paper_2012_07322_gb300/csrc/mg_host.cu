@@ -632,6 +632,13 @@ LevelView<T> with_bc(LevelView<T> v, int bc) {
   return v;
 }
 
+template <typename T>
+void unpad(LevelView<T>& v) {
+  v.sx = v.n0 + 2;
+  v.sy = v.sx * (v.n1 + 2);
+  v.off = 1 + v.sx + (v.three ? v.sy : 0);
+}
+
 // Ghost-push table of a vector colour pass, when built and the pass's ghost
 // rule is the one it was built for.
 GhostPush ghost_push(const mg_hierarchy* H, int l, int c, int colour, int bc) {
@@ -789,7 +796,66 @@ void cluster_vcycle64(mg_hierarchy* H, const Eq& e, int l0) {
   launch_fas_cycle(P, H->d.geom, e.kind, H->st);
 }
 
+// The cluster cycle of a vector equation from level l0 down (smem 0: it does
+// not fit, or takes another path).
+FasVecCycle fas_vec_params(mg_hierarchy* H, int bc, int l0) {
+  FasVecCycle Q{};
+  Q.nl = H->nlev - l0;
+  const long most = std::min<long>(FAS_CLUSTER_CELLS, 256L * fas_vec_blocks());
+  if (Q.nl < 2 || Q.nl > FAS_MAX || H->nb != 1 || bc != MG_BC_DIRICHLET || H->d.mixed_deriv != MG_MIXED_4PT ||
+      H->L[l0].cells() > most || 3 * H->L[H->nlev - 1].cells() > CV_N)
+    return Q;
+  long at = 0;
+  auto take = [&](long n) {
+    const long p = at;
+    at += (n + 1) & ~1L;
+    return (int)p;
+  };
+  Q.solo_from = Q.nl - 1;
+  for (int q = Q.nl - 1; q >= 0; --q) {
+    Level& L = H->L[l0 + q];
+    FasVecLevel& F = Q.lv[q];
+    F.v = with_bc(L.v64, bc);
+    unpad(F.v);
+    F.ng = (int)(F.v.sy * (F.v.n2 + 2 * F.v.three));
+    F.u_at = take(3L * F.ng);
+    F.x_at = q > 0 ? take(3L * F.ng) : 0;
+    F.slot_at = q > 0 ? take(6 * 256) : 0;
+    F.mask = L.cluster.mask;
+    F.list = L.cluster.list;
+    F.start = L.cluster.start;
+    if (L.cells() <= FAS_SOLO_CELLS) Q.solo_from = q;
+  }
+  Q.w_at = take(6 * 256);
+  Q.nu1 = H->d.nu1;
+  Q.nu2 = H->d.nu2;
+  Level& L = H->L[l0];
+  for (int c = 0; c < 3; ++c) {
+    Q.u[c] = L.u[c];
+    Q.f[c] = L.f[c];
+  }
+  Q.off = L.off;
+  Q.sx = L.sx;
+  Q.sy = L.sy;
+  Q.rows = H->crows[bc];
+  const size_t bytes = sizeof(double) * (size_t)at;
+  Q.smem = bytes <= FV_SMEM_MAX ? bytes : 0;
+  return Q;
+}
+// Its first level, nlev when there is none.
+int fas_vec_level(mg_hierarchy* H, int bc) {
+  for (int l = std::max(0, H->nlev - FAS_MAX); l + 1 < H->nlev; ++l)
+    if (fas_vec_params(H, bc, l).smem > 0) return l;
+  return H->nlev;
+}
+
 void vcycle64(mg_hierarchy* H, const Eq& e, int l) {
+  if (e.kind == EQ_VEC && l + 1 < H->nlev && H->cluster_state == 1 && H->crow_state[e.bc] == 1 &&
+      l >= fas_vec_level(H, e.bc)) {
+    for (int q = l; q + 1 < H->nlev; ++q) H->updates += (int64_t)3 * (H->d.nu1 + H->d.nu2) * H->L[q].cells();
+    launch_fas_vec_cycle(fas_vec_params(H, e.bc, l), H->d.geom, H->st);
+    return;
+  }
   if (l >= fas_cluster_level(H, e)) {
     cluster_vcycle64(H, e, l);
     return;
@@ -944,13 +1010,6 @@ void coarse32(mg_hierarchy* H, const Eq& e, int l) {
   }
   for (int c = 0; c < e.ncomp; ++c) launch_convert<double, float>(L.v64, L.u[c], L.e[c], H->st);
   if (e.kind == EQ_VEC) launch_fill_ghosts3<float>(with_bc(L.v32, e.bc), L.e, 3, 1, H->st);
-}
-
-template <typename T>
-void unpad(LevelView<T>& v) {
-  v.sx = v.n0 + 2;
-  v.sy = v.sx * (v.n1 + 2);
-  v.off = 1 + v.sx + (v.three ? v.sy : 0);
 }
 
 // Parameters of the one-block coarse cycle from level l0 (mg_block.cu):
@@ -1504,8 +1563,11 @@ int ensure_coarse_matrix(mg_hierarchy* H, int bc) {
 int ensure_cluster_tables(mg_hierarchy* H) {
   if (H->cluster_state != 0) return MG_OK;
   H->cluster_state = -1;
-  const int l0 = H->nb == 1 ? cluster_size_level(H) : -1;
-  if (l0 < 0 || H->d.mixed_deriv != MG_MIXED_4PT) return MG_OK;
+  const bool mixed = H->d.precision == MG_MIXED;
+  const int l0 = H->nb != 1 ? -1 : (mixed ? cluster_size_level(H) : fas_vec_level(H, MG_BC_DIRICHLET));
+  if (l0 < 0 || l0 >= H->nlev || H->d.mixed_deriv != MG_MIXED_4PT) return MG_OK;
+  const long solo = mixed ? CL_SOLO_CELLS : FAS_SOLO_CELLS;
+  const int cluster = mixed ? cluster_cycle_blocks() : fas_vec_blocks();
   const long gmax = ghost_count_host(H->L[l0].v64);
   int* dgc = nullptr;
   double* dfac = nullptr;
@@ -1536,7 +1598,7 @@ int ensure_cluster_tables(mg_hierarchy* H) {
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(H->st);
     if (ce != cudaSuccess) break;
     const int n0 = v.n0, n1 = v.n1, n2 = v.n2, three = v.three;
-    auto team = [&](const Level& M) { return M.cells() > CL_SOLO_CELLS ? cluster_cycle_blocks() : 1; };
+    auto team = [&](const Level& M) { return M.cells() > solo ? cluster : 1; };
     const int blocks = team(L), groups = (int)(L.cells() >> (three ? 3 : 2)) / blocks;
     auto owner = [&](int i, int j, int k) {
       return ((i >> 1) + (n0 >> 1) * ((j >> 1) + (n1 >> 1) * (k >> 1))) / groups;
@@ -1948,7 +2010,7 @@ int run_solve_body(mg_hierarchy* H, const Eq& e, mg_solve_report* rep) {
     if (int est = ensure_coarse_rows(H, e.bc)) return est;
   if (e.kind == EQ_VEC && e.bc == MG_BC_DIRICHLET)
     if (int est = ensure_ghost_push(H)) return est;
-  if (mixed && e.kind == EQ_VEC && e.bc == MG_BC_DIRICHLET)
+  if (e.kind == EQ_VEC && e.bc == MG_BC_DIRICHLET)
     if (int est = ensure_cluster_tables(H)) return est;
   if (e.kind == EQ_VEC) fill_all64(H, e, 0);
   restrict_sources(H, e);
@@ -2585,7 +2647,7 @@ int create_hierarchy(const mg_grid_desc* desc, void* cuda_stream, int nb, mg_hie
   init_block_cycle_attributes();
   init_fas_attributes();
   init_cluster_cycle_attributes();
-  init_cluster_cycle_attributes();
+  init_fas_vec_attributes();
   const int three = H->d.ndim == 3;
   for (int l = 0; l < H->nlev; ++l) {
     Level& L = H->L[l];

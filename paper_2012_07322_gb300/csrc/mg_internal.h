@@ -315,6 +315,29 @@ void init_fas_attributes();   // once a device is current, before any capture
 long fas_cycle_cells();       // cells of the largest level the cycle takes, 0: not available
 void launch_fas_cycle(const FasCycle& P, int geom, int kind, cudaStream_t st);
 constexpr int CS_CELLS = 64;  // scalar coarsest levels the cycle solves
+
+// The same of the vector equation with Dirichlet-0 ghosts (mg_fasvec.cu).
+constexpr size_t FV_SMEM_MAX = 208 * 1024;
+struct FasVecLevel {
+  LevelView<double> v;  // boundary rule applied, rows not padded: the layout in shared memory
+  int ng, u_at, x_at, slot_at;  // ghosted size; offsets (doubles) in shared memory
+  // readers' tables (ClusterLevel32); the coarsest level has none
+  const unsigned short* mask;
+  const uint2* list;
+  const int* start;
+};
+struct FasVecCycle {
+  int nl, solo_from, nu1, nu2, w_at;  // w_at: 6 values per thread
+  FasVecLevel lv[FAS_MAX];
+  double* u[3];        // the first level in HBM, and its layout
+  const double* f[3];
+  long off, sx, sy;
+  CoarseRows rows;
+  size_t smem;
+};
+void init_fas_vec_attributes();  // once a device is current, before any capture
+int fas_vec_blocks();            // blocks of its cluster, 0: not available
+void launch_fas_vec_cycle(const FasVecCycle& Q, int geom, cudaStream_t st);
 template <typename T>
 void launch_coarse_vec(const LevelView<T>& L, T* V[3], const T* const f[3], int max_sweeps, cudaStream_t st);
 // u -= mean(u) over the interior (the Neumann gauge); the nparts block sums
