@@ -514,8 +514,8 @@ int mg_profile_read(mg_hierarchy* h, int klass, int64_t* launches, double* ms, i
  * combined result) is a file-scope __device__ array.  The first call on a
  * device looks up that array's device address with the device current
  * (cudaGetSymbolAddress); make that first call before any stream capture.
- * Every call shares the array and it keeps the last call's contents (the
- * max word is cleared by each call): calls whose work overlaps on the GPU
+ * Every call shares the array (the counter is back at zero behind each
+ * call, the other words are written before they are read): calls whose work overlaps on the GPU
  * (different streams or threads at once) race, so serialise them.
  */
 int mg_divb_norms_noalloc(int ndim, const int n[3], const double lo[3], const double hi[3],

