@@ -443,46 +443,64 @@ __device__ void bc_coarse(const BlockCycle32& P, const BcLevel& B) {
   const BcView& Lv = B.v;
   constexpr int nc = VEC ? 3 : 1;
   if (!VEC && P.cA) {
-    // red-black NGS sweeps with dense rows of the coarsest operator (its
-    // boundary rules folded in), K subtracted on the diagonal: row r of a
-    // colour is summed by the BC_SPLIT lanes of one group, their entries in
-    // registers, and folded by shuffles; the cells of one colour couple only
-    // to the other colour
-    constexpr int BC_SPLIT = 8;
-    static_assert(BC_THREADS / BC_SPLIT >= BC_CMAT_MAX, "a group of lanes per row");
+    // red-black NGS sweeps with rows of the coarsest operator (its boundary
+    // rules folded in): a thread per cell, the red ones in the first warp, the
+    // black ones in the second, the row's face neighbours in registers.  A
+    // pass is six shared loads and ~5 dependent FP64 operations (~64 cycles
+    // each); summed densely by eight lanes a row it took ~1000 cycles, and the
+    // solve 11.6 k.
     double* const uq = bc_coarse_sh.uq;
-    const int n = P.cn, sub = threadIdx.x % BC_SPLIT, r = threadIdx.x / BC_SPLIT;
-    double a[BC_CMAT_MAX / BC_SPLIT];
-    double fq = 0.0, kq = 0.0, dq = 0.0;
-    int p = 0, i = 0, j = 0, k = 0, col = -1;
-    if (r < n) {
-#pragma unroll
-      for (int m = 0; m < BC_CMAT_MAX / BC_SPLIT; ++m)
-        a[m] = sub + BC_SPLIT * m < n ? P.cA[(long)(sub + BC_SPLIT * m) * n + r] : 0.0;
-      Lv.cell(r, i, j, k);
-      p = Lv.idx(i, j, k);
-      col = (i + j + k) & 1;
-      fq = (double)B.f[0][p];
-      kq = B.k ? (double)B.k[p] : 0.0;
-      dq = 1.0 / (P.cA[(long)r * n + r] - kq);
-      if (sub == 0) uq[r] = 0.0;
-    }
-    __syncthreads();
-    for (int h = 0; h < 2 * P.coarse_sweeps; ++h) {
-      // whole warps skip the sums when none of their rows has the colour
-      if (__any_sync(0xffffffffu, col == (h & 1))) {
-        double x = 0.0;
-        if (col == (h & 1))
-#pragma unroll
-          for (int m = 0; m < BC_CMAT_MAX / BC_SPLIT; ++m)
-            if (sub + BC_SPLIT * m < n) x += a[m] * uq[sub + BC_SPLIT * m];
-#pragma unroll
-        for (int o = BC_SPLIT / 2; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o, BC_SPLIT);
-        if (col == (h & 1) && sub == 0) uq[r] -= (x - kq * uq[r] - fq) * dq;
+    const int n = P.cn, tid = threadIdx.x, g = tid & 31;
+    if (tid < 64) {
+      const bool on = g < n / 2;
+      double a[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, d = 0.0, iD = 0.0, f = 0.0, u = 0.0;
+      int nb[6] = {0, 0, 0, 0, 0, 0}, p = 0, r = 0, i = 0, j = 0, k = 0;
+      if (on) {
+        Lv.colour_cell(g, tid >> 5, i, j, k);
+        r = i + Lv.n0 * (j + Lv.n1 * k);
+        p = Lv.idx(i, j, k);
+        const int sj = Lv.n0, sk = Lv.n0 * Lv.n1;
+        auto side = [&](int m, int q) {
+          nb[m] = q;
+          a[m] = P.cA[(long)q * n + r];
+        };
+        if (i < Lv.n0 - 1) side(0, r + 1);
+        if (i > 0) side(1, r - 1);
+        if (j < Lv.n1 - 1) side(2, r + sj);
+        if (j > 0) side(3, r - sj);
+        // phi wraps; two planes are each other's neighbour once
+        const bool wrap = G != CART && Lv.three && Lv.n2 > 2;
+        if (k < Lv.n2 - 1)
+          side(4, r + sk);
+        else if (wrap)
+          side(4, r - (Lv.n2 - 1) * sk);
+        if (k > 0)
+          side(5, r - sk);
+        else if (wrap)
+          side(5, r + (Lv.n2 - 1) * sk);
+        f = (double)B.f[0][p];
+        d = P.cA[(long)r * n + r] - (B.k ? (double)B.k[p] : 0.0);
+        iD = 1.0 / d;
+        uq[r] = 0.0;
       }
-      __syncthreads();
+      auto warps = [] { asm volatile("bar.sync 1, 64;" ::: "memory"); };
+      warps();
+      for (int h = 0; h < 2 * P.coarse_sweeps; ++h) {
+        if (on && (tid >> 5) == (h & 1)) {
+          double x = fma(a[0], uq[nb[0]], fma(d, u, -f)), y = a[2] * uq[nb[2]];
+          x = fma(a[1], uq[nb[1]], x);
+          y = fma(a[3], uq[nb[3]], y);
+          if (Lv.three) {
+            x = fma(a[4], uq[nb[4]], x);
+            y = fma(a[5], uq[nb[5]], y);
+          }
+          u = fma(-(x + y), iD, u);
+          uq[r] = u;
+        }
+        warps();
+      }
+      if (on) bc_put<G>(B, p, i, j, k, (float)u);
     }
-    if (r < n && sub == 0) bc_put<G>(B, p, i, j, k, (float)uq[r]);
     __syncthreads();
     return;
   }
