@@ -447,7 +447,6 @@ static cudaLaunchConfig_t cluster_config(int cluster, size_t smem, cudaStream_t 
 static int g_cluster32 = -1;
 
 void init_cluster_cycle_attributes() {
-  if (g_cluster32 >= 0) return;
   int best = 16;
   for (int g = 0; g < 3; ++g)
     for (int vec = 0; vec < 2; ++vec) {
@@ -457,7 +456,7 @@ void init_cluster_cycle_attributes() {
         cudaGetLastError();
         best = 0;
       }
-      for (; best >= 8; best /= 2) {
+      for (; g_cluster32 < 0 && best >= 8; best /= 2) {
         cudaLaunchAttribute at[2];
         cudaLaunchConfig_t cfg = cluster_config(best, CL_SMEM_MAX, nullptr, at);
         cfg.numAttrs = 1;
@@ -466,7 +465,7 @@ void init_cluster_cycle_attributes() {
         cudaGetLastError();
       }
     }
-  g_cluster32 = best >= 8 ? best : 0;
+  if (g_cluster32 < 0) g_cluster32 = best >= 8 ? best : 0;
 }
 
 int cluster_cycle_blocks() { return g_cluster32 > 0 ? g_cluster32 : 0; }

@@ -540,14 +540,16 @@ static cudaLaunchConfig_t fas_config(int cluster, size_t smem, cudaStream_t st, 
 }
 
 void init_fas_attributes() {
-  if (g_fas_cluster >= 0) return;
   int best = 16;
   for (int g = 0; g < 3; ++g)
     for (int kind = EQ_PSI; kind <= EQ_LIN; ++kind) {
       FasKernel k = fas_kernel(g, kind);
       cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fas_smem_max(8));
-      for (; best >= 8; best /= 2) {
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fas_smem_max(8)) != cudaSuccess) {
+        cudaGetLastError();
+        best = 0;
+      }
+      for (; g_fas_cluster < 0 && best >= 8; best /= 2) {
         cudaLaunchAttribute at[2];
         cudaLaunchConfig_t cfg = fas_config(best, fas_smem_max(best), nullptr, at);
         cfg.numAttrs = 1;
@@ -556,7 +558,7 @@ void init_fas_attributes() {
         cudaGetLastError();
       }
     }
-  g_fas_cluster = best >= 8 ? best : 0;
+  if (g_fas_cluster < 0) g_fas_cluster = best >= 8 ? best : 0;
 }
 
 long fas_cycle_cells() { return std::min<long>(FAS_CLUSTER_CELLS, (long)g_fas_cluster * FAS_THREADS); }

@@ -343,7 +343,6 @@ static cudaLaunchConfig_t fas_vec_config(int cluster, size_t smem, cudaStream_t 
 static int g_fas_vec_cluster = -1;
 
 void init_fas_vec_attributes() {
-  if (g_fas_vec_cluster >= 0) return;
   int best = 16;
   for (int g = 0; g < 3; ++g) {
     FasVecKernel k = fas_vec_kernel(g);
@@ -352,7 +351,7 @@ void init_fas_vec_attributes() {
       cudaGetLastError();
       best = 0;
     }
-    for (; best >= 8; best /= 2) {
+    for (; g_fas_vec_cluster < 0 && best >= 8; best /= 2) {
       cudaLaunchAttribute at[2];
       cudaLaunchConfig_t cfg = fas_vec_config(best, FV_SMEM_MAX, nullptr, at);
       cfg.numAttrs = 1;
@@ -361,7 +360,7 @@ void init_fas_vec_attributes() {
       cudaGetLastError();
     }
   }
-  g_fas_vec_cluster = best >= 8 ? best : 0;
+  if (g_fas_vec_cluster < 0) g_fas_vec_cluster = best >= 8 ? best : 0;
 }
 
 int fas_vec_blocks() { return g_fas_vec_cluster > 0 ? g_fas_vec_cluster : 0; }

@@ -311,7 +311,7 @@ struct FasCycle {
   int nl, solo_from, nu1, nu2, coarse_sweeps;
   FasLevel lv[FAS_MAX];
 };
-void init_fas_attributes();   // once a device is current, before any capture
+void init_fas_attributes();   // for the current device, before any capture
 long fas_cycle_cells();       // cells of the largest level the cycle takes, 0: not available
 void launch_fas_cycle(const FasCycle& P, int geom, int kind, cudaStream_t st);
 constexpr int CS_CELLS = 64;  // scalar coarsest levels the cycle solves
@@ -335,7 +335,7 @@ struct FasVecCycle {
   CoarseRows rows;
   size_t smem;
 };
-void init_fas_vec_attributes();  // once a device is current, before any capture
+void init_fas_vec_attributes();  // for the current device, before any capture
 int fas_vec_blocks();            // blocks of its cluster, 0: not available
 void launch_fas_vec_cycle(const FasVecCycle& Q, int geom, cudaStream_t st);
 template <typename T>
@@ -550,7 +550,7 @@ struct ClusterCycle32 {
   int slot_at[BC_MAX];  // scalar levels: offsets of CL_WORDS values per thread
 };
 constexpr int CL_WORDS = 12;
-void init_cluster_cycle_attributes();  // once a device is current, before any capture
+void init_cluster_cycle_attributes();  // for the current device, before any capture
 int cluster_cycle_blocks();            // blocks of its cluster, 0: not available
 void launch_cluster_vcycle32(const ClusterCycle32& Q, int geom, cudaStream_t st);
 void init_block_cycle_attributes();
