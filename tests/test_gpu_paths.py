@@ -175,3 +175,40 @@ def test_divergence_norms_of_odd_grids(mg, n):
     tiny = 1e-14 * max(n[d] / (hi[d] - lo[d]) for d in range(len(n)))
     assert st == mg.MG_OK
     assert abs(mx - np.abs(div).max()) <= tiny and abs(l2 - np.sqrt(np.mean(div ** 2))) <= tiny
+
+
+# the mixing sums are taken in the same parts whatever the team, so a problem's
+# fields and cycles do not depend on the launch shape (chosen or given): bit for bit
+@pytest.mark.parametrize("team,team_cells", [(1, 0), (2, 2048), (8, 8192)])
+def test_batch_does_not_depend_on_the_team(mg, team, team_cells):
+    from paper_2012_07322_gb300 import inputs
+    ps = []
+    for geom, n in (("sph", [64, 32]), ("cyl", [64, 128])):
+        if geom == "sph":
+            S = inputs.rotating_polytrope_sph2d(n[0], n[1], 100.0, 1e-3, 10.0, axis_ratio=0.8, omega=0.02)
+            lo, hi = [0.0, 0.0], [100.0, PI]
+        else:
+            S = inputs.rotating_polytrope_cyl(n, 100.0, 1e-3, 10.0, axis_ratio=0.8, omega=0.02)
+            lo, hi = [0.0, -100.0], [100.0, 100.0]
+        h = mg.Hierarchy(mg.grid_desc(geom, n, lo, hi, precision="mixed", tol=1e-10, accel_depth=16, stall_window=0))
+        one = lambda: torch.ones(S[0].shape, dtype=torch.float64, device="cuda")
+        ps.append((h, dev(S[0]), dev(S[1]), [dev(x) for x in S[2]], one(), one(), [one() for _ in range(3)],
+                   [one() for _ in range(3)]))
+
+    def solve(**shape):
+        for p in ps:
+            for t in (p[4], p[5]):
+                t.fill_(1.0)
+            for t in p[6] + p[7]:
+                t.zero_()
+        reps, b = mg.mg_solve_cfc_batch(ps, **shape)
+        assert b["status"] == "ok"
+        return ([t.clone() for p in ps for t in [p[4], p[5]] + p[6] + p[7]],
+                [r[k]["cycles"] for r in reps for k in ("X", "psi", "alphapsi", "beta")])
+
+    want, cycles = solve()
+    got, again = solve(team=team, team_cells=team_cells)
+    for p in ps:
+        p[0].close()
+    assert again == cycles
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
