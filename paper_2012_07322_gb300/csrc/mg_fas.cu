@@ -310,7 +310,9 @@ struct Fas {
     }
   }
 
-  // Right-hand side L_H(u_H) + R r of a level below the first.
+  // Right-hand side L_H(u_H) + R r of a level below the first.  It reads the
+  // neighbours' restricted u, which the first sweep replaces: a barrier of the
+  // level's team stands between the two.
   __device__ __forceinline__ void rhs(const FasIndex& ix) {
     if (!on) return;
     f = 0.0;
@@ -324,8 +326,15 @@ struct Fas {
     go(m);
     FasIndex ix;
     load(ix);
-    if (m > 0) rhs(ix);
-    if (on && nu1 > 0) own_part();
+    auto own = [&] {
+      if (on && nu1 > 0) own_part();
+    };
+    if (m > 0) {
+      rhs(ix);
+      sync(m, own);  // every right-hand side before the first new value
+    } else {
+      own();
+    }
     double nl_term = 0.0;
     auto before = [&] {
       if (on) {
@@ -413,7 +422,9 @@ struct Fas {
     FasIndex ix;
     load(ix);
     rhs(ix);
-    if (on) own_part();
+    sync(nl - 1, [&] {  // every right-hand side before the first new value
+      if (on) own_part();
+    });
     sweeps(ix, n, true, [] {});
     finish(ix);
   }

@@ -10,6 +10,8 @@ within 1e-9 at a converged relative residual of 1e-10, as in the solver-level
 parity tests.  Mixed solves reach the same discrete solution by other
 iterates: both sides converge to 1e-11, which leaves a factor 50 for the
 response of the smoothest modes (2 x 50 x 1e-11 = 1e-9)."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -212,3 +214,79 @@ def test_batch_does_not_depend_on_the_team(mg, team, team_cells):
         p[0].close()
     assert again == cycles
     assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+# ---- order of the cluster cycles: a value is replaced only behind every read of it
+
+
+class Busy:
+    """Another hierarchy solving on its own stream: blocks of the measured cycle are held back at places that change
+    from run to run."""
+
+    def __init__(self, mg):
+        self.mg, self.stop = mg, threading.Event()
+        self.thread = threading.Thread(target=self.loop)
+
+    def loop(self):
+        mg, n = self.mg, [64, 64, 32]
+        with torch.cuda.stream(torch.cuda.Stream()):
+            h = mg.Hierarchy(mg.grid_desc("cart", n, BOX["cart"][0], BOX["cart"][1], precision="mixed", tol=1e-10))
+            f = torch.ones(tuple(reversed(n)), dtype=torch.float64, device="cuda")
+            u = torch.zeros_like(f)
+            while not self.stop.is_set():
+                u.zero_()
+                mg.mg_solve_scalar(h, "lin", "dirichlet", u, f=f)
+            h.close()
+
+    def __enter__(self):
+        self.thread.start()
+
+    def __exit__(self, *exc):
+        self.stop.set()
+        self.thread.join()
+
+
+def first_cycles(mg, geom, n, kind, bc, precision, nu, cycles, repeats):
+    """The iterate behind some cycles from zero, by the oracle (once) and by the GPU (repeated beside other work)."""
+    lo, hi = BOX[geom][0][:len(n)], BOX[geom][1][:len(n)]
+    kw = dict(tol=1e-14, max_cycles=cycles, nu1=nu[0], nu2=nu[1], stall_window=0)
+    d = o.desc(geom, n, lo, hi, **kw)
+    shape = (3,) + o.shape(d) if kind == "vec" else o.shape(d)
+    rng = np.random.default_rng(sum(n))
+    want = np.zeros(shape)
+    if kind == "vec":
+        f = rng.standard_normal(shape)
+        o.solve_vector(d, bc, list(f), list(want))
+    else:
+        args = dict(f=rng.standard_normal(shape), c=rng.uniform(0, 0.01, shape))
+        if kind == "psi":
+            args = dict(U=rng.uniform(0, 1e-3, shape), A2=rng.uniform(0, 1e-4, shape))
+        o.solve_scalar(d, kind, bc, want, **args)
+        args = {k: dev(v) for k, v in args.items()}
+    h = mg.Hierarchy(mg.grid_desc(geom, n, lo, hi, precision=precision, **kw))
+    got = []
+    with Busy(mg):
+        for _ in range(repeats):
+            u = torch.zeros(shape, dtype=torch.float64, device="cuda")
+            if kind == "vec":
+                mg.mg_solve_vector(h, bc, list(dev(f)), list(u), allow=tuple(range(8)))
+            else:
+                mg.mg_solve_scalar(h, kind, bc, u, allow=tuple(range(8)), **args)
+            got.append(u)
+    h.close()
+    return want, got
+
+
+# A right-hand side formed from half-swept values is off by the size of the
+# correction (1e-3 and more); a few hundred passes of a contraction carry
+# rounding errors of a few 1e-16 each, and the oracle's coarsest solve may stop
+# at a residual of 1e-12: 1e-10 in all.
+@pytest.mark.parametrize("geom,n,kind,bc,nu", [
+    ("sph", [64, 32], "psi", "robin", (2, 2)), ("sph", [32, 16, 8], "psi", "robin", (1, 2)),
+    ("cyl", [32, 64], "lin", "robin", (2, 1)), ("cart", [16, 16, 16], "lin", "robin", (2, 2)),
+    ("cart", [16, 8], "lin", "dirichlet", (2, 2)),
+])
+def test_fp64_scalar_cycles_in_order(mg, geom, n, kind, bc, nu):
+    want, got = first_cycles(mg, geom, n, kind, bc, "fp64", nu, 3, 50)
+    assert np.abs(host(got[0]) - want).max() <= 1e-10 * np.abs(want).max()
+    assert all(torch.equal(g, got[0]) for g in got)
