@@ -315,7 +315,7 @@ struct ClVector {
   __device__ __forceinline__ void fill() {
 #pragma unroll
     for (int m = 0; m < 3; ++m) fill(m);
-    __syncthreads();
+    t.sync();  // the first pass replaces sources of ghosts other blocks refill
   }
   template <int M>
   __device__ __forceinline__ void pass(int colour) {

@@ -155,7 +155,6 @@ struct FasVec {
   __device__ __forceinline__ void fill(double* const* F) {
 #pragma unroll
     for (int m = 0; m < 3; ++m) fill(F, m);
-    __syncthreads();
   }
   template <int M>
   __device__ __forceinline__ void pass(int colour) {
@@ -176,6 +175,7 @@ struct FasVec {
   // but for its ghosts).
   __device__ __forceinline__ void rhs() {
     fill(u);
+    __syncthreads();
     if (!t.on) return;
     f[0] = defect<0>() + x[0][t.p];
     f[1] = defect<1>() + x[1][t.p];
@@ -237,6 +237,7 @@ struct FasVec {
       for (int m = 0; m < 3; ++m) put(x, m, u[m][t.p] - slot[(3 + m) * FV_THREADS]);
     t.sync();
     fill(x);
+    __syncthreads();
   }
   __device__ __forceinline__ void out(const FasVecCycle& Q) const {
 #pragma unroll
@@ -309,6 +310,7 @@ __global__ void __launch_bounds__(FV_THREADS, 1) k_fas_vec_cycle(const __grid_co
     T.prolong(Q, l, team(l) > team(l + 1), sm);
     t.sync();
     T.fill(T.u);
+    t.sync();  // the first pass replaces sources of ghosts other blocks refill
     T.sweeps(Q.nu2);
     if (l > 0)
       T.correction();

@@ -290,3 +290,15 @@ def test_fp64_scalar_cycles_in_order(mg, geom, n, kind, bc, nu):
     want, got = first_cycles(mg, geom, n, kind, bc, "fp64", nu, 3, 50)
     assert np.abs(host(got[0]) - want).max() <= 1e-10 * np.abs(want).max()
     assert all(torch.equal(g, got[0]) for g in got)
+
+
+# levels on all blocks and on the first one; ghosts from across the origin, the
+# axis and the poles, which other blocks' cells are the sources of
+@pytest.mark.parametrize("geom,n,nu", [
+    ("sph", [64, 32], (2, 2)), ("sph", [32, 16, 16], (1, 1)), ("cyl", [64, 128], (2, 2)), ("cyl", [16, 16, 16], (0, 2)),
+    ("cart", [64, 64], (2, 0)),
+])
+def test_fp32_vector_cycles_in_order(mg, geom, n, nu):
+    _, got = first_cycles(mg, geom, n, "vec", "dirichlet", "mixed", nu, 8, 50)
+    assert bool(torch.isfinite(got[0]).all()) and float(got[0].abs().max()) > 0.0
+    assert all(torch.equal(g, got[0]) for g in got)
