@@ -172,7 +172,7 @@ struct FasVec {
     }
   }
   // Right-hand side L_H(u_H) + R r of a level below the first (u_H current
-  // but for its ghosts).
+  // but for its ghosts).  It reads what the first sweep replaces.
   __device__ __forceinline__ void rhs() {
     fill(u);
     __syncthreads();
@@ -273,7 +273,10 @@ __global__ void __launch_bounds__(FV_THREADS, 1) k_fas_vec_cycle(const __grid_co
   for (int l = 0; l + 1 < nl && rank < team(l); ++l) {
     const ClCell t(Q.lv[l].v, rank, team(l)), tc(Q.lv[l + 1].v, rank, team(l + 1));
     FasVec<G> T(t, Q, l, sm);
-    if (l > 0) T.rhs();
+    if (l > 0) {
+      T.rhs();
+      t.sync();  // every right-hand side before the first new value
+    }
     T.sweeps(Q.nu1);
     T.restrict_to(Q, l, tc, sm, w);
     t.sync();

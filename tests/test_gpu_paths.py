@@ -302,3 +302,15 @@ def test_fp32_vector_cycles_in_order(mg, geom, n, nu):
     _, got = first_cycles(mg, geom, n, "vec", "dirichlet", "mixed", nu, 8, 50)
     assert bool(torch.isfinite(got[0]).all()) and float(got[0].abs().max()) > 0.0
     assert all(torch.equal(g, got[0]) for g in got)
+
+
+# at least two levels on all blocks, one level above the first block's, none;
+# tolerance as for the scalar cycles
+@pytest.mark.parametrize("geom,n,nu", [
+    ("sph", [32, 16, 8], (2, 2)), ("sph", [16, 8, 8], (1, 2)), ("cyl", [32, 64], (2, 2)), ("cyl", [16, 16, 16], (2, 1)),
+    ("cart", [16, 16, 16], (2, 2)), ("cart", [16, 8], (2, 2)),
+])
+def test_fp64_vector_cycles_in_order(mg, geom, n, nu):
+    want, got = first_cycles(mg, geom, n, "vec", "dirichlet", "fp64", nu, 3, 50)
+    assert np.abs(host(got[0]) - want).max() <= 1e-10 * np.abs(want).max()
+    assert all(torch.equal(g, got[0]) for g in got)
