@@ -514,9 +514,11 @@ int mg_profile_read(mg_hierarchy* h, int klass, int64_t* launches, double* ms, i
  * combined result) is a file-scope __device__ array.  The first call on a
  * device looks up that array's device address with the device current
  * (cudaGetSymbolAddress); make that first call before any stream capture.
- * Every call shares the array (the counter is back at zero behind each
- * call, the other words are written before they are read): calls whose work overlaps on the GPU
- * (different streams or threads at once) race, so serialise them.
+ * Every call shares the array: calls whose work overlaps on the GPU
+ * (different streams or threads at once) race and may return each other's
+ * norms, so serialise them.  What such calls leave behind does not reach a
+ * later one (the counter is cleared behind them, the other words are written
+ * before they are read).
  */
 int mg_divb_norms_noalloc(int ndim, const int n[3], const double lo[3], const double hi[3],
                           const double* B[3], void* cuda_stream, double* max_div, double* l2_div);

@@ -314,3 +314,28 @@ def test_fp64_vector_cycles_in_order(mg, geom, n, nu):
     want, got = first_cycles(mg, geom, n, "vec", "dirichlet", "fp64", nu, 3, 50)
     assert np.abs(host(got[0]) - want).max() <= 1e-10 * np.abs(want).max()
     assert all(torch.equal(g, got[0]) for g in got)
+
+
+# two threads at once (which the call's description rules out) may get each
+# other's norms; the calls behind them get their own
+def test_divergence_norms_after_overlapping_calls(mg):
+    def field(n):
+        B = [dev(np.random.default_rng(n).standard_normal((n, n, n))) for _ in range(3)]
+        return B, [0.0] * 3, [1.0] * 3
+
+    fields = [field(16), field(48), field(96)]
+    want = [mg.mg_divb_norms_noalloc(*f) for f in fields]
+    torch.cuda.synchronize()
+
+    def loop(f):
+        s = torch.cuda.Stream()
+        for _ in range(400):
+            mg.mg_divb_norms_noalloc(*f, stream=s)
+
+    threads = [threading.Thread(target=loop, args=(f,)) for f in fields]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for _ in range(3):
+        assert [mg.mg_divb_norms_noalloc(*f) for f in fields] == want
