@@ -1173,9 +1173,11 @@ void cluster_vcycle32(mg_hierarchy* H, const Eq& e, int l0) {
   prof_end(H, tok);
 }
 
-// Linear correction-scheme V-cycle on (L - K) e = f32, e = 0 initially.
-void vcycle32(mg_hierarchy* H, const Eq& e, int l) {
-  if (l == cluster_cycle_level(H, e)) {
+// Linear correction-scheme V-cycle on (L - K) e = f32 from e = 0, or with guess
+// from the e that level l holds: launched then, since the cluster's cycle (like
+// the one block's, which FMG has at its coarsest level only) starts from zero.
+void vcycle32(mg_hierarchy* H, const Eq& e, int l, bool guess = false) {
+  if (!guess && l == cluster_cycle_level(H, e)) {
     cluster_vcycle32(H, e, l);
     return;
   }
@@ -1246,7 +1248,7 @@ void fmg32(mg_hierarchy* H, const Eq& e) {
     const float* eH[3] = {C.e[0], C.e[1], C.e[2]};
     launch_prolong3<float>(v, vc, L.e, eH, nullptr, e.ncomp, e.kind == EQ_VEC, H->st);
     if (e.kind == EQ_VEC) launch_fill_ghosts3<float>(v, L.e, 3, 1, H->st);
-    vcycle32(H, e, l);
+    vcycle32(H, e, l, true);
   }
 }
 

@@ -339,3 +339,28 @@ def test_divergence_norms_after_overlapping_calls(mg):
         t.join()
     for _ in range(3):
         assert [mg.mg_divb_norms_noalloc(*f) for f in fields] == want
+
+
+# FMG starts a level from the coarser level's correction, also the level whose
+# V-cycle runs on a cluster (8192 cells: the finest here).  Dropped, an FMG cycle
+# is a V-cycle.  Cycles: what passes launched one by one take.
+@pytest.mark.parametrize("geom,n,kind,bc,accel,cycles", [
+    ("cart", [128, 64], "lin", "dirichlet", 0, 9), ("cart", [32, 16, 16], "lin", "robin", 0, 12),
+    ("cart", [32, 16, 16], "vec", "dirichlet", 0, 12), ("cyl", [64, 128], "lin", "robin", 8, 6),
+    ("cyl", [64, 128], "vec", "dirichlet", 8, 6),
+])
+def test_mixed_fmg_keeps_its_starting_guess(mg, geom, n, kind, bc, accel, cycles):
+    lo, hi = BOX[geom][0][:len(n)], BOX[geom][1][:len(n)]
+    shape = (3,) * (kind == "vec") + tuple(reversed(n))
+    f = dev(np.random.default_rng(5).standard_normal(shape))
+    took = {}
+    for cycle in ("v", "fmg"):
+        h = mg.Hierarchy(mg.grid_desc(geom, n, lo, hi, precision="mixed", tol=1e-10, max_cycles=100, stall_window=0,
+                                      accel_depth=accel, cycle=cycle))
+        u = torch.zeros(shape, dtype=torch.float64, device="cuda")
+        if kind == "vec":
+            took[cycle] = mg.mg_solve_vector(h, bc, list(f), list(u))["cycles"]
+        else:
+            took[cycle] = mg.mg_solve_scalar(h, kind, bc, u, f=f)["cycles"]
+        h.close()
+    assert took["fmg"] < took["v"] and took["fmg"] <= cycles
