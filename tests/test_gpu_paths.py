@@ -364,3 +364,26 @@ def test_mixed_fmg_keeps_its_starting_guess(mg, geom, n, kind, bc, accel, cycles
             took[cycle] = mg.mg_solve_scalar(h, kind, bc, u, f=f)["cycles"]
         h.close()
     assert took["fmg"] < took["v"] and took["fmg"] <= cycles
+
+
+# The integer stencils hand over to the flux form where all seven values lie
+# below 2^-895 or the scaled coefficient is not normal: right-hand sides that
+# put the solution (2^-10 to 2^-5 of them on the unit cube) on both sides of
+# the first line and below it, close to overflow, and, with cells of 2^40, on
+# both sides of the second.  A linear equation scales exactly with powers of two.
+@pytest.mark.parametrize("side,exponent", [(0, -888), (0, -920), (0, 1008), (44, -963)])
+def test_cartesian_stencils_at_the_ends_of_the_range(mg, side, exponent):
+    f = np.random.default_rng(12).standard_normal((32, 32, 32))
+
+    def solve(side, exponent):
+        h = mg.Hierarchy(mg.grid_desc("cart", [32] * 3, [-2.0 ** side] * 3, [2.0 ** side] * 3, tol=1e-10,
+                                      max_cycles=100, stall_window=0))
+        u = torch.zeros((32, 32, 32), dtype=torch.float64, device="cuda")
+        rg = mg.mg_solve_scalar(h, "lin", "robin", u, f=dev(np.ldexp(f, exponent)))
+        h.close()
+        return rg, np.ldexp(host(u), -exponent - 2 * side)
+
+    one, want = solve(0, 0)
+    far, got = solve(side, exponent)
+    assert abs(far["cycles"] - one["cycles"]) <= 1
+    assert np.abs(got - want).max() <= 1e-9 * np.abs(want).max()
