@@ -69,7 +69,6 @@ struct FasAt {
   int mine;    // cells of a colour a block owns
   int groups;  // coarse cells a block owns the children of
   int lgroups; // log2
-  int cells;
 };
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -479,7 +478,6 @@ __global__ void __launch_bounds__(FAS_THREADS) k_fas_cycle(const __grid_constant
       o.mine = n / team / 2;
       o.groups = n / team / (T.three ? 8 : 4);
       o.lgroups = 31 - __clz(o.groups);
-      o.cells = n;
       at[l] = o;
       o.slot += 2 * o.half;
       o.u += n;

@@ -785,9 +785,7 @@ void cluster_vcycle64(mg_hierarchy* H, const Eq& e, int l0) {
     FasLevel& F = P.lv[q];
     F.v = with_bc(L.v64, e.bc);
     F.u = L.u[0];
-    F.uh = L.uh[0];
-    F.f = const_cast<double*>(fptr(H, e, l, 0));
-    F.r = L.r[0];
+    F.f = fptr(H, e, l, 0);
     F.s0 = s0ptr(H, e, l);
     F.s1 = s1ptr(H, e, l);
     if (L.cells() <= FAS_SOLO_CELLS) P.solo_from = q;

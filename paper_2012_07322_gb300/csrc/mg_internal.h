@@ -304,8 +304,8 @@ constexpr long FAS_CLUSTER_CELLS = 4096;  // the cycle runs from the first level
 constexpr long FAS_SOLO_CELLS = 128;
 struct FasLevel {
   LevelView<double> v;  // boundary rule applied
-  double *u, *uh, *f, *r;
-  const double *s0, *s1;
+  double* u;
+  const double *f, *s0, *s1;
 };
 struct FasCycle {
   int nl, solo_from, nu1, nu2, coarse_sweeps;
