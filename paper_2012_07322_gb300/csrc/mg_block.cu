@@ -4,9 +4,10 @@
 // level's kernels are too small to fill the GPU and each launch costs more
 // than its work; inside one block the same phases are separated by block
 // barriers instead of kernel boundaries, and every level lives in shared
-// memory (the same ghosted layout as in HBM).  Every phase applies the
-// per-cell functions the grid-wide kernels apply, in the same order, so the
-// result is identical to the launched cycle.
+// memory (the same ghosted layout as in HBM).  The phases are those of the
+// launched cycle in the same order; the arithmetic within a cell is mg_block.cuh's
+// own (ghosts kept in the arrays, residual and restriction in one), so the two
+// agree to FP32 rounding.
 #include "mg_internal.h"
 #include "mg_kernels.cuh"
 #include "mg_block.cuh"

@@ -3103,6 +3103,9 @@ namespace {
 // problem to rank 0 and the barriers.  Larger clusters leave SMs idle (144 of
 // 152 in fours, 120 in eights), so many problems take smaller teams: 192
 // uneven problems 734, 420, 362 and 480 ms, 45 of them 730, 402, 238 and 185.
+// The estimate is rough: it knows the cycles of psi and alpha psi only, so of
+// six draws of 192 rotating stars one gets teams of 2 after its first solve,
+// 417 ms in place of 318 (teams of 2 from 16384 cells: 411 to 432 on all six).
 constexpr double BATCH_SERIAL = 4000.0;
 
 void batch_shape(mg_hierarchy* const* hs, int count, size_t smem, int* team, long* team_cells) {

@@ -709,9 +709,6 @@ __global__ void k_fill_ghosts3(LevelView<T> L, T* __restrict__ u0, T* __restrict
 // of 9 for eq. psi in FP64).
 constexpr int RES_KZ = 4;
 constexpr long RES_KZ_CELLS = 1L << 21;
-// The vector residual carries three components' worth of FP64 work per
-// cell: one plane per thread and at most 128 registers (two blocks per SM)
-// spread it over more blocks.
 
 template <typename T, int G, int KIND, int KZ>
 __global__ void k_residual_scalar(LevelView<T> L, const T* __restrict__ u, const T* __restrict__ f,
