@@ -368,6 +368,13 @@ void init_fas_vec_attributes() {
   if (g_fas_vec_cluster < 0) g_fas_vec_cluster = best >= 8 ? best : 0;
 }
 
+bool fas_vec_attributes_set() {
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, fas_vec_kernel(SPH)) == cudaSuccess) return a.maxDynamicSharedSizeBytes >= (int)FV_SMEM_MAX;
+  cudaGetLastError();
+  return false;
+}
+
 int fas_vec_blocks() { return g_fas_vec_cluster > 0 ? g_fas_vec_cluster : 0; }
 
 void launch_fas_vec_cycle(const FasVecCycle& Q, int geom, cudaStream_t st) {

@@ -336,6 +336,7 @@ struct FasVecCycle {
   size_t smem;
 };
 void init_fas_vec_attributes();  // for the current device, before any capture
+bool fas_vec_attributes_set();   // whether its last attribute is set in the current context
 int fas_vec_blocks();            // blocks of its cluster, 0: not available
 void launch_fas_vec_cycle(const FasVecCycle& Q, int geom, cudaStream_t st);
 template <typename T>
