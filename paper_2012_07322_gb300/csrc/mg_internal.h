@@ -96,8 +96,11 @@ inline unsigned spread_threads(long n, unsigned lo) {
 }
 // Block of at most t threads (a power of two) that tiles nx x ny x nz items
 // (powers of two) without idle threads, z planes deep at least: the FP64
-// pipe spends a whole instruction slot on a warp with idle lanes too.
+// pipe spends a whole instruction slot on a warp with idle lanes too.  Deeper
+// where one plane per block would be more blocks than a launch has in z (65536
+// planes).
 inline dim3 fit_block(int nx, int ny, int nz, unsigned t, unsigned z = 1) {
+  while ((unsigned)nz > 65535u * z) z *= 2;
   dim3 b(1, 1, z);
   t = t > z ? t / z : 1;
   b.x = std::min<unsigned>({(unsigned)nx, 32u, t});

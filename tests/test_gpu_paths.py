@@ -387,3 +387,20 @@ def test_cartesian_stencils_at_the_ends_of_the_range(mg, side, exponent):
     far, got = solve(side, exponent)
     assert abs(far["cycles"] - one["cycles"]) <= 1
     assert np.abs(got - want).max() <= 1e-9 * np.abs(want).max()
+
+
+# as many planes as a launch of two-plane blocks takes, rows short enough for
+# blocks of one plane: the passes run and the first cycles converge
+@pytest.mark.parametrize("kind", ["lin", "vec"])
+def test_fp64_passes_of_65536_planes(mg, kind):
+    n = [16, 16, 65536]
+    h = mg.Hierarchy(mg.grid_desc("cart", n, [0.0] * 3, [1.0, 1.0, 4096.0], tol=1e-14, max_cycles=3, stall_window=0))
+    shape = (3,) * (kind == "vec") + tuple(reversed(n))
+    f = torch.randn(shape, generator=torch.Generator(device="cuda").manual_seed(1), dtype=torch.float64, device="cuda")
+    u = torch.zeros_like(f)
+    if kind == "vec":
+        rg = mg.mg_solve_vector(h, "dirichlet", list(f), list(u), allow=tuple(range(8)))
+    else:
+        rg = mg.mg_solve_scalar(h, "lin", "dirichlet", u, f=f, allow=tuple(range(8)))
+    h.close()
+    assert rg["cycles"] == 3 and rg["rel"] < 0.1
